@@ -31,6 +31,8 @@ struct mf_plan_s {
   mf_dtype bank_dtype = MF_F32;
   int64_t n_tmpl = 0, ld_bank = 0;
   float* scales_dev = nullptr;
+  unsigned* rmax = nullptr;       // per template, for quantising rows (16-bit banks)
+  double* norm_part = nullptr;    // partial sums of the templates' norms
   double* sigmasq_dev = nullptr;
   float* inv_sigma_dev = nullptr;
   int32_t* sel_all = nullptr;
@@ -209,14 +211,27 @@ void make_weights(const mf_plan_desc& d, const double* psd, std::vector<double>&
   }
 }
 
-mf_status recompute_sigmasq(mf_plan_t p, int64_t row0, int64_t n_rows) {
+// bank rows from row0 on, with the weights when the PSD is set
+mf::BankRows bank_rows(mf_plan_t p, int64_t row0) {
+  mf::BankRows b{};
+  b.rows = (char*)p->bank + (size_t)row0 * p->ld_bank * elem_bytes(p->bank_dtype);
+  b.type = bank_type(p->bank_dtype);
+  b.ld = p->ld_bank;
+  b.n1 = p->n1;
+  b.n2 = p->n2;
+  b.w = p->psd_set ? p->w_dev : nullptr;
+  b.part = p->norm_part + row0 * mf::norm_parts(p->n1, p->n2);
+  b.sigmasq = p->sigmasq_dev + row0;
+  b.inv_sigma = p->inv_sigma_dev + row0;
+  b.scales = p->scales_dev ? p->scales_dev + row0 : nullptr;
+  b.rmax = p->rmax ? p->rmax + row0 : nullptr;
+  return b;
+}
+
+// the bank or the PSD changes: what was derived from them is stale
+void bank_changed(mf_plan_t p) {
   p->scale_valid = false;
-  p->chisq_p = 0;  // band edges follow the bank and the PSD
-  if (!p->psd_set || !p->bank || n_rows <= 0) return MF_OK;
-  cudaError_t e = mf::launch_sigmasq(p->bank, bank_type(p->bank_dtype), p->ld_bank, p->scales_dev, row0, n_rows,
-                                     p->w_dev, p->nb, p->sigmasq_dev, p->inv_sigma_dev, p->st, p->n1, p->n2);
-  if (e != cudaSuccess) return cuda_fail(p, e, "sigma^2 kernel");
-  return MF_OK;
+  p->chisq_p = 0;  // band edges
 }
 
 // sigma_ref = max_t sigma_t (host copy of the FP64 norms), then ratio / thr_raw on the device
@@ -343,7 +358,7 @@ mf_status mf_plan(mf_plan_t* out, const mf_plan_desc* desc) {
 void mf_destroy(mf_plan_t p) {
   if (!p) return;
   if (p->st) cudaStreamSynchronize(p->st); else cudaDeviceSynchronize();
-  dfree(p->w_dev); dfree(p->bank); dfree(p->scales_dev); dfree(p->sigmasq_dev); dfree(p->inv_sigma_dev); dfree(p->ratio_dev); dfree(p->thr_raw_dev);
+  dfree(p->w_dev); dfree(p->bank); dfree(p->scales_dev); dfree(p->rmax); dfree(p->norm_part); dfree(p->sigmasq_dev); dfree(p->inv_sigma_dev); dfree(p->ratio_dev); dfree(p->thr_raw_dev);
   dfree(p->sel_all); dfree(p->q); dfree(p->scratch); dfree(p->slots); dfree(p->sel_copy); dfree(p->trig);
   dfree(p->count); dfree(p->bc); dfree(p->coincs); dfree(p->n_coinc); dfree(p->maxrho); dfree(p->nb_ptr);
   dfree(p->q_lp); dfree(p->dmax); dfree(p->dscale); dfree(p->row_valid); dfree(p->bpow); dfree(p->edges);
@@ -361,7 +376,12 @@ mf_status mf_set_psd(mf_plan_t p, const double* psd, int64_t nbins) {
   e = cudaStreamSynchronize(p->st);
   if (e != cudaSuccess) return cuda_fail(p, e, "mf_set_psd sync");
   p->psd_set = true;
-  return recompute_sigmasq(p, 0, p->n_tmpl);
+  bank_changed(p);
+  if (!p->bank || p->n_tmpl <= 0) return MF_OK;
+  e = mf::launch_norm_parts(bank_rows(p, 0), p->n_tmpl, p->st);
+  if (e == cudaSuccess) e = mf::launch_norms(bank_rows(p, 0), p->n_tmpl, p->st);
+  if (e != cudaSuccess) return cuda_fail(p, e, "sigma^2 kernel");
+  return MF_OK;
 }
 
 mf_status mf_bank_reserve(mf_plan_t p, mf_dtype dtype, int64_t n_tmpl) {
@@ -370,23 +390,26 @@ mf_status mf_bank_reserve(mf_plan_t p, mf_dtype dtype, int64_t n_tmpl) {
   if (n_tmpl < 1 || n_tmpl > 0x7fffffff) return fail(p, MF_EINVAL, "mf_bank_reserve: n_tmpl must be in [1, 2^31)");
   cudaStreamSynchronize(p->st);
   p->n_tmpl = 0;
-  p->scale_valid = false;
-  p->chisq_p = 0;
+  bank_changed(p);
   p->bank_dtype = dtype;
-  p->ld_bank = p->d.n / 2;  // column layout of the N/2 bins below Nyquist (launch_to_cols)
+  p->ld_bank = p->d.n / 2;  // column layout of the N/2 bins below Nyquist (mf::BankRows)
   const size_t bytes = (size_t)n_tmpl * p->ld_bank * elem_bytes(dtype);
   mf_status s;
   if ((s = dalloc(p, &p->bank, bytes, "bank")) != MF_OK ||
       (s = dalloc(p, &p->sigmasq_dev, n_tmpl * sizeof(double), "sigma^2")) != MF_OK ||
+      (s = dalloc(p, &p->norm_part, n_tmpl * mf::norm_parts(p->n1, p->n2) * sizeof(double), "sigma^2 sums")) != MF_OK ||
       (s = dalloc(p, &p->inv_sigma_dev, n_tmpl * sizeof(float), "1/sigma")) != MF_OK ||
       (s = dalloc(p, &p->ratio_dev, n_tmpl * sizeof(float), "sigma ratio")) != MF_OK ||
       (s = dalloc(p, &p->thr_raw_dev, n_tmpl * sizeof(float), "raw thresholds")) != MF_OK ||
       (s = dalloc(p, &p->sel_all, n_tmpl * sizeof(int32_t), "all-template selection")) != MF_OK)
     return s;
   if (dtype != MF_F32) {
-    if ((s = dalloc(p, &p->scales_dev, n_tmpl * sizeof(float), "scales")) != MF_OK) return s;
+    if ((s = dalloc(p, &p->scales_dev, n_tmpl * sizeof(float), "scales")) != MF_OK ||
+        (s = dalloc(p, &p->rmax, n_tmpl * sizeof(unsigned), "row maxima")) != MF_OK)
+      return s;
   } else {
     dfree(p->scales_dev);
+    dfree(p->rmax);
   }
   cudaError_t e = cudaMemsetAsync(p->bank, 0, bytes, p->st);
   if (e == cudaSuccess) e = cudaMemsetAsync(p->sigmasq_dev, 0, n_tmpl * sizeof(double), p->st);
@@ -412,7 +435,6 @@ mf_status mf_bank_set_rows(mf_plan_t p, int64_t row0, int64_t n_rows, const void
     return fail(p, MF_EINVAL, "mf_bank_set_rows: scales required for 16-bit banks and forbidden for MF_F32");
   if (n_rows == 0) return MF_OK;
   const size_t eb = elem_bytes(p->bank_dtype);
-  char* dst = (char*)p->bank + (size_t)row0 * p->ld_bank * eb;
   const void* src = htilde;
   void* tmp = nullptr;
   cudaError_t e = on_device ? after_default_stream(p) : cudaSuccess;
@@ -422,16 +444,14 @@ mf_status mf_bank_set_rows(mf_plan_t p, int64_t row0, int64_t n_rows, const void
     e = cudaMemcpyAsync(tmp, htilde, (size_t)n_rows * ld * eb, cudaMemcpyHostToDevice, p->st);
     src = tmp;
   }
-  if (e == cudaSuccess) e = mf::launch_to_cols(src, ld, dst, p->ld_bank, n_rows, p->n1, p->n2, (int)eb, p->st);
   if (e == cudaSuccess && scales)
     e = cudaMemcpyAsync(p->scales_dev + row0, scales, n_rows * sizeof(float), cudaMemcpyHostToDevice, p->st);
+  bank_changed(p);
+  if (e == cudaSuccess) e = mf::launch_put_rows(bank_rows(p, row0), src, ld, n_rows, false, p->nb, p->st);
+  if (e == cudaSuccess && p->psd_set) e = mf::launch_norms(bank_rows(p, row0), n_rows, p->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(p->st);
   if (tmp) cudaFree(tmp);
-  if (e != cudaSuccess) return cuda_fail(p, e, "mf_bank_set_rows copy");
-  mf_status s = recompute_sigmasq(p, row0, n_rows);
-  if (s != MF_OK) return s;
-  e = cudaStreamSynchronize(p->st);
-  if (e != cudaSuccess) return cuda_fail(p, e, "mf_bank_set_rows sigma^2");
+  if (e != cudaSuccess) return cuda_fail(p, e, "mf_bank_set_rows");
   return MF_OK;
 }
 
@@ -453,27 +473,12 @@ mf_status mf_bank_quantize_rows(mf_plan_t p, int64_t row0, int64_t n_rows, const
     e = cudaMemcpyAsync(tmp, htilde, (size_t)n_rows * ld * sizeof(float2), cudaMemcpyHostToDevice, p->st);
     src = tmp;
   }
-  const size_t eb = elem_bytes(p->bank_dtype);
-  void* q16 = nullptr;  // quantised rows in natural layout, then into the bank's column layout
-  if (e == cudaSuccess) {
-    mf_status s = dalloc(p, &q16, (size_t)n_rows * p->nb * eb, "quantised rows");
-    if (s != MF_OK) {
-      dfree(tmp);
-      return s;
-    }
-    e = mf::launch_quant_bank(src, ld, n_rows, p->nb, bank_type(p->bank_dtype), q16, p->nb, p->scales_dev + row0, p->st);
-  }
-  if (e == cudaSuccess)
-    e = mf::launch_to_cols(q16, p->nb, (char*)p->bank + (size_t)row0 * p->ld_bank * eb, p->ld_bank, n_rows, p->n1, p->n2,
-                           (int)eb, p->st);
+  bank_changed(p);
+  if (e == cudaSuccess) e = mf::launch_put_rows(bank_rows(p, row0), src, ld, n_rows, true, p->nb, p->st);
+  if (e == cudaSuccess && p->psd_set) e = mf::launch_norms(bank_rows(p, row0), n_rows, p->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(p->st);
   dfree(tmp);
-  if (q16) cudaFree(q16);
   if (e != cudaSuccess) return cuda_fail(p, e, "mf_bank_quantize_rows");
-  mf_status s = recompute_sigmasq(p, row0, n_rows);
-  if (s != MF_OK) return s;
-  e = cudaStreamSynchronize(p->st);
-  if (e != cudaSuccess) return cuda_fail(p, e, "mf_bank_quantize_rows sigma^2");
   return MF_OK;
 }
 
@@ -502,26 +507,43 @@ mf_status mf_bank_generate_taylorf2(mf_plan_t p, int64_t row0, int64_t n_rows, c
     return fail(p, MF_EINVAL, "mf_bank_generate_taylorf2: rows out of range");
   if (!(f_low > 0)) return fail(p, MF_EINVAL, "mf_bank_generate_taylorf2: f_low must be > 0");
   if (n_rows == 0) return MF_OK;
+  if (!mf::taylorf2_valid(m1, m2, n_rows, p->d.fs, p->d.n, f_low))
+    return fail(p, MF_EINVAL, "mf_bank_generate_taylorf2: bad masses or band");
+  // Rows are generated in the filter's scratch (nothing on this stream uses it now) in blocks of 128 MB, which are
+  // still in L2 when they are stored; a temporary buffer takes its place where the scratch holds no row.  One
+  // 256 MB block at a time in a buffer of its own cost an allocation, a free and 3 waits per 63 templates.
   const int64_t ld = (p->nb + 63) / 64 * 64;
-  const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(n_rows, (int64_t(256) << 20) / (ld * 8)));
-  float2* tmp = nullptr;
-  mf_status s = dalloc(p, &tmp, (size_t)chunk * ld * sizeof(float2), "generated rows");
-  if (s != MF_OK) return s;
-  for (int64_t r = 0; r < n_rows && s == MF_OK; r += chunk) {
-    const int64_t cnt = std::min<int64_t>(chunk, n_rows - r);
-    cudaError_t e = mf::launch_taylorf2(m1 + r, m2 + r, cnt, p->d.fs, p->d.n, f_low, tmp, ld, p->st);
-    if (e == cudaErrorInvalidValue) {
-      s = fail(p, MF_EINVAL, "mf_bank_generate_taylorf2: bad masses or band");
-    } else if (e != cudaSuccess) {
-      s = cuda_fail(p, e, "mf_bank_generate_taylorf2");
-    } else {
-      s = p->bank_dtype == MF_F32 ? mf_bank_set_rows(p, row0 + r, cnt, tmp, ld, nullptr, 1)
-                                  : mf_bank_quantize_rows(p, row0 + r, cnt, tmp, ld, 1);
-    }
+  const size_t table = mf::taylorf2_table_bytes(n_rows), row = (size_t)ld * sizeof(float2);
+  auto bytes = [&](int64_t c) {
+    return table + mf::taylorf2_work_bytes(c, p->d.fs, p->d.n, f_low) + (size_t)c * row;
+  };
+  int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(n_rows, (int64_t(128) << 20) / (int64_t)row));
+  const size_t have = p->scratch ? (size_t)p->batch * p->d.n_det * p->d.n * sizeof(float2) : 0;
+  char* work = reinterpret_cast<char*>(p->scratch);
+  char* tmp = nullptr;
+  if (have < bytes(1)) {
+    mf_status s = dalloc(p, &tmp, bytes(chunk), "generated rows");
+    if (s != MF_OK) return s;
+    work = tmp;
+  } else {
+    while (bytes(chunk) > have) chunk = (chunk + 1) / 2;
   }
-  cudaStreamSynchronize(p->st);
-  cudaFree(tmp);
-  return s;
+  char* anchors = work + table;
+  float2* rows = reinterpret_cast<float2*>(anchors + mf::taylorf2_work_bytes(chunk, p->d.fs, p->d.n, f_low));
+  cudaError_t e = mf::taylorf2_tables(m1, m2, n_rows, p->d.fs, p->d.n, f_low, work, p->st);
+  bank_changed(p);
+  for (int64_t r = 0; r < n_rows && e == cudaSuccess; r += chunk) {
+    const int64_t cnt = std::min<int64_t>(chunk, n_rows - r);
+    e = mf::launch_taylorf2(work, r, cnt, p->d.fs, p->d.n, f_low, anchors, rows, ld, p->st);
+    if (e == cudaSuccess)
+      e = mf::launch_put_rows(bank_rows(p, row0 + r), rows, ld, cnt, p->bank_dtype != MF_F32, p->nb, p->st);
+  }
+  if (e == cudaSuccess && p->psd_set) e = mf::launch_norms(bank_rows(p, row0), n_rows, p->st);
+  const cudaError_t e2 = cudaStreamSynchronize(p->st);
+  if (tmp) cudaFree(tmp);
+  if (e == cudaSuccess) e = e2;
+  if (e != cudaSuccess) return cuda_fail(p, e, "mf_bank_generate_taylorf2");
+  return MF_OK;
 }
 
 mf_status mf_set_intermediate(mf_plan_t p, mf_dtype dtype) {

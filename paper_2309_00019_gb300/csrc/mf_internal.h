@@ -111,11 +111,6 @@ __host__ __device__ inline int part_of(const FilterParts& ps, int64_t u, int per
 // scratch.
 cudaError_t launch_quant_q(const float2* q, int64_t ld_q, int64_t nb, int n_det, int q_type, void* q_lp,
                            unsigned* dmax, float* dscale, cudaStream_t st);
-// Quantise n_rows FP32 templates (src [n_rows][ld_src], nb bins) to the 16-bit
-// bank rows dst [n_rows][ld_dst] with a per-template power-of-two scale:
-// stored = h / scale, max |stored| in [2^14, 2^15); scales[i] = scale.
-cudaError_t launch_quant_bank(const float2* src, int64_t ld_src, int64_t n_rows, int64_t nb, int bank_type, void* dst,
-                              int64_t ld_dst, float* scales, cudaStream_t st);
 // Plan introspection for the length-class runner (mf_batch.cu): templates in
 // the bank; a fingerprint of everything a captured graph of mf_filter bakes in
 // (buffers, batch, storage types); and whether mf_filter on the whole bank would
@@ -137,7 +132,7 @@ int filter_fused(::mf_plan_s* const* plans, const void* const* dtilde, const int
                  int64_t scratch_series, const CUtensorMap& scratch_map, cudaStream_t st, std::string* err);
 // The TMA-staged filter passes (mf_filter.cu).  The bank rows and the
 // weighted data are in column layout: element k = k1 N2 + k2 of the non-zero
-// half (k1 < N1/2) at k2 N1/2 + k1 (see launch_to_cols).
+// half (k1 < N1/2) at k2 N1/2 + k1 (BankRows).
 cudaError_t launch_filter2_pass1(const FilterArgs& a, cudaStream_t st);
 cudaError_t launch_filter2_pass2(const FilterArgs& a, const CUtensorMap& scratch_map, cudaStream_t st);
 // the tensor-core row pass over the FP16 intermediate (mf_filter_tc.cu), N = 2^20
@@ -157,11 +152,31 @@ cudaError_t launch_fill_twiddles(int64_t n, float2* tw1, float2* tw2, cudaStream
 cudaError_t launch_fill_tw4(int64_t n, float2* tw4, cudaStream_t st);
 int64_t tw4_count(int64_t n);
 
-// Column layout of spectra rows: dst[r][k2 N1/2 + k1] = src[r][k1 N2 + k2] for
-// k1 < N1/2, k2 < N2 (the bins k < N/2), elem_bytes 8 (complex64) or 4 (16-bit
-// pairs); src rows ld_src elements apart, dst rows ld_dst.
-cudaError_t launch_to_cols(const void* src, int64_t ld_src, void* dst, int64_t ld_dst, int64_t n_rows, int n1, int n2,
-                           int elem_bytes, cudaStream_t st);
+// Rows of a bank in column layout: element k = k1 n2 + k2 of the non-zero half (k1 < n1/2, k2 < n2) at k2 n1/2 + k1,
+// and what a row's norm needs.  All pointers are those of the first row.
+struct BankRows {
+  void* rows;
+  int type;              // BankType of the stored elements
+  int64_t ld;
+  int n1, n2;
+  const double* w;       // PSD weights in natural order, or null: no norms
+  double* part;          // norm_parts(n1, n2) partial sums per row
+  double* sigmasq;
+  float* inv_sigma;
+  float* scales;         // per row (16-bit types)
+  unsigned* rmax;        // per row (quantising)
+};
+int64_t norm_parts(int n1, int n2);
+// Store n_rows natural-order rows src (ld_src elements apart) and, when b.w is set, the partial sums of their norms
+// (launch_norms finishes them).
+// quantise: src is complex64 (nb bins per row) and goes to the 16-bit type with a power-of-two scale per row:
+// stored = h / scale, max |stored| in [2^14, 2^15), scales[row] = scale; otherwise src has the stored type.
+cudaError_t launch_put_rows(const BankRows& b, const void* src, int64_t ld_src, int64_t n_rows, bool quantise,
+                            int64_t nb, cudaStream_t st);
+// the same partial sums from rows that are stored already (a new PSD)
+cudaError_t launch_norm_parts(const BankRows& b, int64_t n_rows, cudaStream_t st);
+// sigma^2 and 1 / sigma of n_rows rows from their partial sums
+cudaError_t launch_norms(const BankRows& b, int64_t n_rows, cudaStream_t st);
 // q = q_scale w s~ in column layout (q [n_det][ld_q], N/2 elements per row)
 cudaError_t launch_prep_cols(const float2* dtilde, int64_t ld_d, const double* w, int n1, int n2, int n_det,
                              float2* q, int64_t ld_q, unsigned long long* slots, int64_t n_slots, cudaStream_t st,
@@ -189,10 +204,17 @@ cudaError_t launch_chisq(const void* trig, const int64_t* count, int64_t cap, co
                          int64_t ld_bank, const void* q, int q_type, int64_t ld_q, int n1, int n2, const int32_t* edges,
                          int p, const float* ratio, const float* dscale, float* chi2, float* newsnr, cudaStream_t st);
 
-// TaylorF2 templates (mf_taylorf2.cu): n_tmpl natural-order complex64 rows out [n_tmpl][ld] of an n-sample
-// segment at fs, from host masses; synchronises the stream
-cudaError_t launch_taylorf2(const double* m1, const double* m2, int64_t n_tmpl, double fs, int64_t n, double f_low,
-                            float2* out, int64_t ld, cudaStream_t st);
+// TaylorF2 templates (mf_taylorf2.cu): natural-order complex64 rows out [.][ld] of an n-sample segment at fs.
+// taylorf2_tables turns valid host masses into the kernels' table (taylorf2_table_bytes(n_tmpl) bytes at dev; the
+// host masses are done with on return); launch_taylorf2 generates rows [t0, t0 + n_rows) of the table with
+// taylorf2_work_bytes(n_rows, ...) bytes of work space.
+bool taylorf2_valid(const double* m1, const double* m2, int64_t n_tmpl, double fs, int64_t n, double f_low);
+size_t taylorf2_table_bytes(int64_t n_tmpl);
+size_t taylorf2_work_bytes(int64_t n_rows, double fs, int64_t n, double f_low);
+cudaError_t taylorf2_tables(const double* m1, const double* m2, int64_t n_tmpl, double fs, int64_t n, double f_low,
+                            void* dev, cudaStream_t st);
+cudaError_t launch_taylorf2(const void* tables, int64_t t0, int64_t n_rows, double fs, int64_t n, double f_low,
+                            void* work, float2* out, int64_t ld, cudaStream_t st);
 
 // blocks x 256 threads, each 8 chains x 16 x iters FP32 FMAs (the ALU probe)
 cudaError_t launch_fma_probe(float* out, int blocks, int iters, cudaStream_t st);
@@ -219,11 +241,9 @@ cudaError_t launch_filter_batch(const FilterArgs& a, cudaStream_t st);
 // the two halves of launch_filter_batch, for per-kernel timing
 cudaError_t launch_filter_pass1(const FilterArgs& a, cudaStream_t st);
 cudaError_t launch_filter_pass2(const FilterArgs& a, cudaStream_t st);
-// sigma^2 of bank rows [row0, row0 + n_rows) in natural layout (n1 = 0: bins
-// 0..nb-1) or column layout (n1, n2 > 0: the N/2 bins of launch_to_cols)
-cudaError_t launch_sigmasq(const void* bank, int bank_type, int64_t ld_bank, const float* scales,
-                           int64_t row0, int64_t n_rows, const double* w, int64_t nb,
-                           double* sigmasq, float* inv_sigma, cudaStream_t st, int n1 = 0, int n2 = 0);
+// sigma^2 and 1 / sigma of complex64 rows in natural order (bins 0..nb-1)
+cudaError_t launch_sigmasq(const float2* rows, int64_t ld, int64_t n_rows, const double* w, int64_t nb,
+                           double* sigmasq, float* inv_sigma, cudaStream_t st);
 // compaction of window maxima into mf_trigger records (layout of the public struct)
 cudaError_t launch_compact(const unsigned long long* slots, int n_det, int64_t n_sel, int64_t n_win,
                            int64_t window, const int32_t* sel, void* trig_out, int64_t trig_cap,

@@ -336,40 +336,42 @@ __global__ void k_zero_u64(unsigned long long* p, int64_t n) {
     p[i] = 0ull;
 }
 
-// n1 = 0: row t holds bins 0..nb-1; n1 > 0: column layout (stored index
-// i = k2 n1/2 + k1 holds bin k = k1 n2 + k2, i < N/2)
-template <int BT>
-__global__ void k_sigmasq(const void* bank, int64_t ld_bank, const float* scales, int64_t row0,
-                          const double* __restrict__ w, int64_t nb, double* sigmasq, float* inv_sigma, int n1,
-                          int n2) {
-  const int64_t t = row0 + blockIdx.x;
+// a template's sigma^2 and 1 / sigma from the sum v of w |stored|^2
+__device__ __forceinline__ void write_sigma(double v, const float* scales, int64_t t, double* sigmasq,
+                                            float* inv_sigma) {
+  const double sc = scales ? (double)scales[t] : 1.0;
+  const double s2 = v * sc * sc;  // sigma^2 of the dequantised template
+  sigmasq[t] = s2;
+  inv_sigma[t] = s2 > 0.0 ? (float)(sc / sqrt(s2)) : 0.0f;  // scale folded in: z is of the stored values
+}
+
+// sum over the block (all threads return it): warp sums, then the warps' in order
+__device__ __forceinline__ double block_sum(double acc, double* red) {
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x, warps = blockDim.x * blockDim.y / 32;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((tid & 31) == 0) red[tid >> 5] = acc;
+  __syncthreads();
+  double v = 0.0;
+  for (int i = 0; i < warps; ++i) v += red[i];
+  return v;
+}
+
+// sigma^2 of FP32 rows in natural order, one CTA per row (mf_filter_noalloc)
+__global__ void k_sigmasq(const float2* bank, int64_t ld_bank, const double* __restrict__ w, int64_t nb,
+                          double* sigmasq, float* inv_sigma) {
+  __shared__ double red[32];
+  const int64_t t = blockIdx.x;
   double acc = 0.0;
-  const int64_t count = n1 > 0 ? (int64_t)n1 * n2 / 2 : nb;
-  const int R = n1 / 2;
-  for (int64_t i = threadIdx.x; i < count; i += blockDim.x) {
-    const int64_t k = n1 > 0 ? (int64_t)(i % R) * n2 + i / R : i;
+  for (int64_t k = threadIdx.x; k < nb; k += blockDim.x) {
     const double wk = w[k];
     if (wk != 0.0) {
-      const float2 h = BankElem<BT>::get(bank, t * ld_bank + i);
+      const float2 h = __ldg(bank + t * ld_bank + k);
       acc += wk * ((double)h.x * h.x + (double)h.y * h.y);
     }
   }
-  __shared__ double red[32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (threadIdx.x == 0) {
-      const double sc = scales ? (double)scales[t] : 1.0;
-      const double s2 = v * sc * sc;  // sigma^2 of the dequantised template
-      sigmasq[t] = s2;
-      inv_sigma[t] = s2 > 0.0 ? (float)(sc / sqrt(s2)) : 0.0f;  // scale folded in: z is of the stored values
-    }
-  }
+  const double v = block_sum(acc, red);
+  if (threadIdx.x == 0) write_sigma(v, nullptr, t, sigmasq, inv_sigma);
 }
 
 // --- compaction of window maxima ------------------------------------------
@@ -530,24 +532,6 @@ __global__ void k_wait_selftest(int* status, int* returned) {
   if (!mbar_wait_bounded(&bar, 0, status)) atomicAdd(returned, 1);
 }
 
-// --- column layout of spectra (the filter's bank and weighted-data layout) ----
-
-// dst[r][k2 R + k1] = src[r][k1 n2 + k2], k1 < R = n1/2, k2 < n2: 32 x 32 tiles
-// through shared memory, coalesced on both sides.  grid (n2/32, R/32, rows).
-template <typename E>
-__global__ void k_to_cols(const E* __restrict__ src, int64_t ld_src, E* __restrict__ dst, int64_t ld_dst, int n1,
-                          int n2, int64_t row0) {
-  __shared__ E tile[32][33];
-  const int R = n1 / 2;
-  const int64_t row = row0 + blockIdx.z;
-  const int k1_0 = blockIdx.y * 32, k2_0 = blockIdx.x * 32;
-  for (int y = threadIdx.y; y < 32; y += blockDim.y)
-    tile[y][threadIdx.x] = src[row * ld_src + (int64_t)(k1_0 + y) * n2 + k2_0 + threadIdx.x];
-  __syncthreads();
-  for (int y = threadIdx.y; y < 32; y += blockDim.y)
-    dst[row * ld_dst + (int64_t)(k2_0 + y) * R + k1_0 + threadIdx.x] = tile[threadIdx.x][y];
-}
-
 // q[det][k2 R + k1] = q_scale w[k] s~[det][k], k = k1 n2 + k2 (FP64 product)
 __global__ void k_prep_cols(const float2* __restrict__ d, int64_t ld_d, const double* __restrict__ w, int n1, int n2,
                             int n_det, float2* __restrict__ q, int64_t ld_q, double q_scale) {
@@ -622,23 +606,145 @@ __global__ void k_quant_q(const float2* __restrict__ q, int64_t ld_q, int64_t nb
   }
 }
 
-// one CTA per template row
-template <int BT>
-__global__ void k_quant_bank(const float2* __restrict__ src, int64_t ld_src, int64_t nb, void* dst, int64_t ld_dst,
-                             float* scales) {
+// per-row max |component| of complex64 rows into rmax (float bits, >= 0; zeroed before): grid (blocks, rows)
+__global__ void k_row_max(const float2* __restrict__ src, int64_t ld, int64_t nb, unsigned* rmax) {
   __shared__ float red[32];
-  const float2* row = src + blockIdx.x * ld_src;
+  const float2* row = src + blockIdx.y * ld;
   float m = 0.f;
-  for (int64_t k = threadIdx.x; k < nb; k += blockDim.x) {
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nb; k += (int64_t)gridDim.x * blockDim.x) {
     const float2 v = row[k];
     m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
   }
-  const float c = pow2_scale(block_max(m, red));
-  for (int64_t k = threadIdx.x; k < nb; k += blockDim.x) {
-    const float2 v = row[k];
-    store_lp<BT>(dst, blockIdx.x * ld_dst + k, v.x * c, v.y * c);
+  m = block_max(m, red);
+  if (threadIdx.x == 0) atomicMax(rmax + blockIdx.y, __float_as_uint(m));
+}
+
+// --- column layout of the bank (the filter's layout) and the templates' norms -----
+//
+// A stored row holds bin k = k1 n2 + k2 (k1 < R = n1 / 2, k2 < n2) at k2 R + k1.  A CTA owns 32 columns k2 of
+// one row and a quarter of their k1 (kNormSplit; all of it below 4 tiles), which it walks in 32 x 32 tiles through shared memory, coalesced on both sides.  sigma^2 = sum w |h|^2
+// (FP64) is taken from the tiles on their way, in natural order, where the weights' reads are coalesced too:
+// as a pass of its own over the stored row it gathered the weights n2 bins apart and took 31.7 us per template
+// at N = 2^20, four fifths of loading a bank; now the row's transpose and its norm take 4.4 us.  The few FP64
+// operations that the chip can do (2 per clock and SM) are the next bound, so bins outside the template's
+// band (exact zeros) are skipped.  Partial sums go to part[row][CTA of the row] and are added in order, so a row's
+// norm depends on its values alone: k_cols_norms takes the same partial sums from a stored row.
+
+constexpr int kNormSplit = 4;
+__host__ __device__ constexpr int norm_split(int n1) { return n1 / 64 >= kNormSplit ? kNormSplit : 1; }
+
+template <int BT>
+struct Stored {
+  using E = uint32_t;  // a pair of 16-bit values
+};
+template <>
+struct Stored<kBankF32> {
+  using E = float2;
+};
+
+template <int BT>
+__device__ __forceinline__ float2 stored_value(typename Stored<BT>::E v) {
+  if constexpr (BT == kBankF32) {
+    return v;
+  } else if constexpr (BT == kBankF16) {
+    return __half22float2(*reinterpret_cast<__half2*>(&v));
+  } else {
+    return __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&v));
   }
-  if (threadIdx.x == 0) scales[blockIdx.x] = 1.f / c;  // exact: c is a power of two
+}
+
+__device__ __forceinline__ void add_norm(double& acc, float2 h, const double* __restrict__ w, int64_t k) {
+  if (h.x != 0.f || h.y != 0.f) {
+    const double wk = w[k];
+    if (wk != 0.0) acc += wk * ((double)h.x * h.x + (double)h.y * h.y);
+  }
+}
+
+// rows src [.][ld_src] in natural order -> stored rows dst [.][ld_dst].  QUANT: src is complex64 and is scaled
+// by pow2_scale(rmax[row]) and rounded to the 16-bit type on the way (scales[row] = 1 / that); otherwise src
+// holds the stored type.  w null: no norms.  grid (n2 / 32, norm_split(n1), rows), 256 threads (32, 8).
+template <int BT, bool QUANT>
+__global__ void __launch_bounds__(256) k_put_cols(const void* __restrict__ src, int64_t ld_src, void* __restrict__ dst,
+                                                  int64_t ld_dst, int n1, int n2, const unsigned* __restrict__ rmax,
+                                                  float* __restrict__ scales, const double* __restrict__ w,
+                                                  double* __restrict__ part) {
+  using E = typename Stored<BT>::E;
+  __shared__ E tile[32][33];
+  __shared__ double red[8];
+  const int R = n1 / 2, k2_0 = blockIdx.x * 32, tx = threadIdx.x, ty = threadIdx.y;
+  const int64_t row = blockIdx.z;
+  const int span = R / norm_split(n1), first = blockIdx.y * span;
+  float c = 1.f;
+  if constexpr (QUANT) {
+    c = pow2_scale(__uint_as_float(rmax[row]));
+    if (blockIdx.x == 0 && blockIdx.y == 0 && tx == 0 && ty == 0) scales[row] = 1.f / c;  // exact: c is a power of two
+  }
+  double acc = 0.0;
+  for (int k1_0 = first; k1_0 < first + span; k1_0 += 32) {
+    E v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t i = row * ld_src + (int64_t)(k1_0 + ty + 8 * u) * n2 + k2_0 + tx;
+      if constexpr (QUANT) {
+        const float2 x = static_cast<const float2*>(src)[i];
+        store_lp<BT>(&v[u], 0, x.x * c, x.y * c);
+      } else {
+        v[u] = static_cast<const E*>(src)[i];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      tile[ty + 8 * u][tx] = v[u];
+      if (w) add_norm(acc, stored_value<BT>(v[u]), w, (int64_t)(k1_0 + ty + 8 * u) * n2 + k2_0 + tx);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      static_cast<E*>(dst)[row * ld_dst + (int64_t)(k2_0 + ty + 8 * u) * R + k1_0 + tx] = tile[tx][ty + 8 * u];
+    __syncthreads();
+  }
+  if (w) {
+    const double v = block_sum(acc, red);
+    if (tx == 0 && ty == 0) part[(row * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = v;
+  }
+}
+
+// the partial sums of k_put_cols from rows that are stored already (a new PSD)
+template <int BT>
+__global__ void __launch_bounds__(256) k_cols_norms(const void* __restrict__ bank, int64_t ld, int n1, int n2,
+                                                    const double* __restrict__ w, double* __restrict__ part) {
+  using E = typename Stored<BT>::E;
+  __shared__ E tile[32][33];
+  __shared__ double red[8];
+  const int R = n1 / 2, k2_0 = blockIdx.x * 32, tx = threadIdx.x, ty = threadIdx.y;
+  const int64_t row = blockIdx.z;
+  const int span = R / norm_split(n1), first = blockIdx.y * span;
+  double acc = 0.0;
+  for (int k1_0 = first; k1_0 < first + span; k1_0 += 32) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      tile[tx][ty + 8 * u] = static_cast<const E*>(bank)[row * ld + (int64_t)(k2_0 + ty + 8 * u) * R + k1_0 + tx];
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      add_norm(acc, stored_value<BT>(tile[ty + 8 * u][tx]), w, (int64_t)(k1_0 + ty + 8 * u) * n2 + k2_0 + tx);
+    __syncthreads();
+  }
+  const double v = block_sum(acc, red);
+  if (tx == 0 && ty == 0) part[(row * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = v;
+}
+
+// sigma^2 and 1 / sigma of rows [0, n_rows) from their partial sums: one warp per row, a fixed order
+__global__ void __launch_bounds__(128) k_norms(const double* __restrict__ part, int per_row, int64_t n_rows,
+                                               const float* __restrict__ scales, double* sigmasq, float* inv_sigma) {
+  const int64_t t = blockIdx.x * (int64_t)4 + threadIdx.x / 32;
+  const int lane = threadIdx.x & 31;
+  if (t >= n_rows) return;
+  double v = 0.0;
+  for (int i = lane; i < per_row; i += 32) v += part[t * per_row + i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) write_sigma(v, scales, t, sigmasq, inv_sigma);
 }
 
 }  // namespace
@@ -715,33 +821,79 @@ cudaError_t launch_quant_q(const float2* q, int64_t ld_q, int64_t nb, int n_det,
   return cudaGetLastError();
 }
 
-cudaError_t launch_quant_bank(const float2* src, int64_t ld_src, int64_t n_rows, int64_t nb, int bank_type, void* dst,
-                              int64_t ld_dst, float* scales, cudaStream_t st) {
+int64_t norm_parts(int n1, int n2) { return (int64_t)(n2 / 32) * norm_split(n1); }
+
+namespace {
+
+template <int BT, bool QUANT>
+void run_put_cols(const BankRows& b, const void* src, int64_t ld_src, int64_t r0, unsigned rows, cudaStream_t st) {
+  const int64_t se = QUANT || BT == kBankF32 ? 8 : 4, de = BT == kBankF32 ? 8 : 4;
+  k_put_cols<BT, QUANT><<<dim3((unsigned)(b.n2 / 32), norm_split(b.n1), rows), dim3(32, 8), 0, st>>>(
+      static_cast<const unsigned char*>(src) + r0 * ld_src * se, ld_src,
+      static_cast<unsigned char*>(b.rows) + r0 * b.ld * de, b.ld, b.n1, b.n2, QUANT ? b.rmax + r0 : nullptr,
+      QUANT ? b.scales + r0 : nullptr, b.w, b.w ? b.part + r0 * norm_parts(b.n1, b.n2) : nullptr);
+}
+
+constexpr int64_t kGridRows = 65535;  // rows of one launch
+
+}  // namespace
+
+cudaError_t launch_put_rows(const BankRows& b, const void* src, int64_t ld_src, int64_t n_rows, bool quantise,
+                            int64_t nb, cudaStream_t st) {
   if (n_rows <= 0) return cudaSuccess;
-  if (bank_type == kBankF16)
-    k_quant_bank<kBankF16><<<(unsigned)n_rows, 256, 0, st>>>(src, ld_src, nb, dst, ld_dst, scales);
-  else if (bank_type == kBankBF16)
-    k_quant_bank<kBankBF16><<<(unsigned)n_rows, 256, 0, st>>>(src, ld_src, nb, dst, ld_dst, scales);
-  else
-    return cudaErrorInvalidValue;
-  ++g_launches;
+  if (b.n1 < 64 || b.n2 < 32 || (quantise && b.type == kBankF32)) return cudaErrorInvalidValue;
+  if (quantise) {
+    cudaError_t e = cudaMemsetAsync(b.rmax, 0, (size_t)n_rows * sizeof(unsigned), st);
+    if (e != cudaSuccess) return e;
+  }
+  for (int64_t r0 = 0; r0 < n_rows; r0 += kGridRows) {
+    const unsigned rows = (unsigned)std::min<int64_t>(kGridRows, n_rows - r0);
+    if (quantise) {
+      k_row_max<<<dim3((unsigned)std::min<int64_t>(32, (nb + 2047) / 2048), rows), 256, 0, st>>>(
+          static_cast<const float2*>(src) + r0 * ld_src, ld_src, nb, b.rmax + r0);
+      ++g_launches;
+    }
+    switch (b.type) {
+      case kBankF32: run_put_cols<kBankF32, false>(b, src, ld_src, r0, rows, st); break;
+      case kBankF16:
+        if (quantise) run_put_cols<kBankF16, true>(b, src, ld_src, r0, rows, st);
+        else run_put_cols<kBankF16, false>(b, src, ld_src, r0, rows, st);
+        break;
+      case kBankBF16:
+        if (quantise) run_put_cols<kBankBF16, true>(b, src, ld_src, r0, rows, st);
+        else run_put_cols<kBankBF16, false>(b, src, ld_src, r0, rows, st);
+        break;
+      default: return cudaErrorInvalidValue;
+    }
+    ++g_launches;
+  }
   return cudaGetLastError();
 }
 
-cudaError_t launch_to_cols(const void* src, int64_t ld_src, void* dst, int64_t ld_dst, int64_t n_rows, int n1, int n2,
-                           int elem_bytes, cudaStream_t st) {
-  if (n1 < 64 || n2 < 32 || (elem_bytes != 8 && elem_bytes != 4)) return cudaErrorInvalidValue;
-  for (int64_t r0 = 0; r0 < n_rows; r0 += 65535) {
-    const dim3 g((unsigned)(n2 / 32), (unsigned)(n1 / 2 / 32), (unsigned)std::min<int64_t>(65535, n_rows - r0));
-    const dim3 b(32, 8);
-    if (elem_bytes == 8)
-      k_to_cols<float2><<<g, b, 0, st>>>(static_cast<const float2*>(src), ld_src, static_cast<float2*>(dst), ld_dst,
-                                         n1, n2, r0);
-    else
-      k_to_cols<uint32_t><<<g, b, 0, st>>>(static_cast<const uint32_t*>(src), ld_src, static_cast<uint32_t*>(dst),
-                                           ld_dst, n1, n2, r0);
+cudaError_t launch_norm_parts(const BankRows& b, int64_t n_rows, cudaStream_t st) {
+  if (n_rows <= 0) return cudaSuccess;
+  for (int64_t r0 = 0; r0 < n_rows; r0 += kGridRows) {
+    const dim3 g((unsigned)(b.n2 / 32), norm_split(b.n1), (unsigned)std::min<int64_t>(kGridRows, n_rows - r0));
+    const dim3 t(32, 8);
+    const void* rows = static_cast<const unsigned char*>(b.rows) + r0 * b.ld * (b.type == kBankF32 ? 8 : 4);
+    double* part = b.part + r0 * norm_parts(b.n1, b.n2);
+    switch (b.type) {
+      case kBankF32: k_cols_norms<kBankF32><<<g, t, 0, st>>>(rows, b.ld, b.n1, b.n2, b.w, part); break;
+      case kBankF16: k_cols_norms<kBankF16><<<g, t, 0, st>>>(rows, b.ld, b.n1, b.n2, b.w, part); break;
+      case kBankBF16: k_cols_norms<kBankBF16><<<g, t, 0, st>>>(rows, b.ld, b.n1, b.n2, b.w, part); break;
+      default: return cudaErrorInvalidValue;
+    }
     ++g_launches;
   }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_norms(const BankRows& b, int64_t n_rows, cudaStream_t st) {
+  if (n_rows <= 0) return cudaSuccess;
+  k_norms<<<(unsigned)((n_rows + 3) / 4), 128, 0, st>>>(b.part, (int)norm_parts(b.n1, b.n2), n_rows,
+                                                        b.type == kBankF32 ? nullptr : b.scales, b.sigmasq,
+                                                        b.inv_sigma);
+  ++g_launches;
   return cudaGetLastError();
 }
 
@@ -758,27 +910,11 @@ cudaError_t launch_prep_cols(const float2* dtilde, int64_t ld_d, const double* w
   return cudaGetLastError();
 }
 
-cudaError_t launch_sigmasq(const void* bank, int bank_type, int64_t ld_bank, const float* scales, int64_t row0,
-                           int64_t n_rows, const double* w, int64_t nb, double* sigmasq, float* inv_sigma,
-                           cudaStream_t st, int n1, int n2) {
+cudaError_t launch_sigmasq(const float2* rows, int64_t ld, int64_t n_rows, const double* w, int64_t nb,
+                           double* sigmasq, float* inv_sigma, cudaStream_t st) {
   if (n_rows <= 0) return cudaSuccess;
   if (n_rows > 0x7fffffff) return cudaErrorInvalidValue;
-  switch (bank_type) {
-    case kBankF32:
-      k_sigmasq<kBankF32><<<(unsigned)n_rows, 256, 0, st>>>(bank, ld_bank, scales, row0, w, nb, sigmasq, inv_sigma,
-                                                             n1, n2);
-      break;
-    case kBankF16:
-      k_sigmasq<kBankF16><<<(unsigned)n_rows, 256, 0, st>>>(bank, ld_bank, scales, row0, w, nb, sigmasq, inv_sigma,
-                                                             n1, n2);
-      break;
-    case kBankBF16:
-      k_sigmasq<kBankBF16><<<(unsigned)n_rows, 256, 0, st>>>(bank, ld_bank, scales, row0, w, nb, sigmasq, inv_sigma,
-                                                             n1, n2);
-      break;
-    default:
-      return cudaErrorInvalidValue;
-  }
+  k_sigmasq<<<(unsigned)n_rows, 256, 0, st>>>(rows, ld, w, nb, sigmasq, inv_sigma);
   ++g_launches;
   return cudaGetLastError();
 }

@@ -111,7 +111,7 @@ extern "C" mf_status mf_filter_noalloc(double fs, int64_t n, int32_t n_det, doub
   k_iota_zero<<<8, 256, 0, st>>>(sel, n_tmpl, status);
   e = cudaGetLastError();
   if (e == cudaSuccess)
-    e = mf::launch_sigmasq(htilde, mf::kBankF32, ld_h, nullptr, 0, n_tmpl, w, nb, sigmasq, inv_sigma, st);
+    e = mf::launch_sigmasq(static_cast<const float2*>(htilde), ld_h, n_tmpl, w, nb, sigmasq, inv_sigma, st);
   if (e == cudaSuccess)
     e = mf::launch_prep(static_cast<const float2*>(dtilde), ld_d, w, nb, n_det, q, ld_q, slots, n_slots, st);
   mf::FilterArgs a{};

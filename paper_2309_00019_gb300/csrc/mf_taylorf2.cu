@@ -12,6 +12,10 @@
 // near 1e-5 rad; the interpolation error is below 2e-4 rad, at the
 // lightest templates' lowest frequencies), reduced to [-pi, pi] and turned into
 // cos / sin.  The amplitude is exp2(-7/6 log2 f) (fast base-2 logarithm, ~1e-6 relative).
+// The FP64 units bound the anchors (2 operations per clock and SM, and a whole warp's slots however few of its
+// lanes are in use), so they have a kernel of their own that fills its warps and computes only the anchors that
+// bins of the band interpolate between; as part of k_taylorf2 the 20 anchors of each 2,048 bins held up its CTAs
+// (2.75 us per template at N = 2^20; now 0.65 us for the anchors and 2.1 us for the bins).
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -51,9 +55,22 @@ __device__ __forceinline__ double tf2_phase(const TF2& t, double f) {
   return -0.25 * kPi + t.pre / v5 * s;
 }
 
-__global__ void __launch_bounds__(kGenThreads) k_taylorf2(const TF2* __restrict__ tmpl, double df, float2* __restrict__ out,
-                                                          int64_t ld, int64_t nb) {
-  __shared__ double psi[kGenChunk + 4];    // anchor phases (FP64), then
+// Anchor a of a template is at bin (a - 1) K.  Those below half the lower band edge, or two intervals past the
+// upper one, only serve bins that are zeroed; they are 0.
+__global__ void __launch_bounds__(kGenThreads) k_tf2_anchors(const TF2* __restrict__ tmpl, double df, int n_anchor,
+                                                             double* __restrict__ psi) {
+  const TF2 t = tmpl[blockIdx.y];
+  const int a = blockIdx.x * kGenThreads + threadIdx.x;
+  if (a >= n_anchor) return;
+  const int K = 1 << t.K_log2;
+  const int64_t k = (int64_t)(a - 1) * K;
+  const bool used = k >= t.k_lo / 2 && k <= t.k_hi + 2 * K;
+  psi[(int64_t)blockIdx.y * n_anchor + a] = used ? tf2_phase(t, (double)k * df) : 0.0;
+}
+
+__global__ void __launch_bounds__(kGenThreads) k_taylorf2(const TF2* __restrict__ tmpl, const double* __restrict__ psi,
+                                                          int n_anchor, double df, float2* __restrict__ out, int64_t ld,
+                                                          int64_t nb) {
   __shared__ float mod2pi[kGenChunk + 4];  // anchor phase mod 2 pi
   __shared__ float dnext[kGenChunk + 4];   // Psi(anchor + 1) - Psi(anchor)
   const TF2 t = tmpl[blockIdx.y];
@@ -65,19 +82,14 @@ __global__ void __launch_bounds__(kGenThreads) k_taylorf2(const TF2* __restrict_
     return;
   }
   const int K = 1 << t.K_log2;
-  // anchors a = -1 .. n_in + 1 at bins k0 + a K (bins of the chunk lie in intervals 0 .. n_in - 1)
+  // the chunk's anchors -1 .. n_in + 1 (its bins lie in intervals 0 .. n_in - 1)
   const int n_in = (int)((k1 - k0 + K - 1) >> t.K_log2);
-  for (int a = threadIdx.x; a < n_in + 4; a += kGenThreads) {  // one FP64 phase per anchor
-    const int64_t ka = k0 + (int64_t)(a - 1) * K;
-    // anchors below half the lower band edge only serve bins that are zeroed; keep them finite
-    psi[a] = tf2_phase(t, (double)(ka > t.k_lo / 2 ? ka : t.k_lo / 2) * df);
-  }
-  __syncthreads();
+  const double* pa = psi + (int64_t)blockIdx.y * n_anchor + (k0 >> t.K_log2);
   for (int a = threadIdx.x; a < n_in + 3; a += kGenThreads) {
-    const double pa = psi[a];
+    const double p = pa[a];
     const double two_pi = 2.0 * kPi;
-    mod2pi[a] = (float)(pa - two_pi * floor(pa / two_pi));
-    dnext[a] = (float)(psi[a + 1] - pa);
+    mod2pi[a] = (float)(p - two_pi * floor(p / two_pi));
+    dnext[a] = (float)(pa[a + 1] - p);
   }
   __syncthreads();
   const float two_pi_f = 6.283185307179586f, inv_two_pi = 0.15915494309189535f;
@@ -106,6 +118,21 @@ __global__ void __launch_bounds__(kGenThreads) k_taylorf2(const TF2* __restrict_
 
 }  // namespace
 
+// first bin of the band
+static int64_t first_bin(double f_low, double df) {
+  int64_t lo = (int64_t)std::ceil(f_low / df);
+  while (lo > 0 && (double)(lo - 1) * df >= f_low) --lo;
+  while ((double)lo * df < f_low) ++lo;
+  return lo;
+}
+
+// anchors every 2^j bins (the same for every template of a call)
+static int anchor_log2(int64_t lo, double df) {
+  int lg = 0;
+  while (2.0 * (1 << lg) * df <= 0.25 && 2 * (1 << lg) <= std::max<int64_t>(lo / 4, 1) && (1 << lg) < 1024) ++lg;
+  return lg;
+}
+
 // host: per-template coefficients; the band uses the same float64 arithmetic as the host-side generators
 static TF2 make_tf2(double m1, double m2, double fs, int64_t n, double f_low) {
   TF2 t{};
@@ -129,46 +156,61 @@ static TF2 make_tf2(double m1, double m2, double fs, int64_t n, double f_low) {
   const double df = fs / (double)n;
   const double f_isco = 1.0 / (std::pow(6.0, 1.5) * pi * M);
   const double fhi = std::min(f_isco, fs / 2.0);
-  int64_t lo = (int64_t)std::ceil(f_low / df);
-  while (lo > 0 && (double)(lo - 1) * df >= f_low) --lo;
-  while ((double)lo * df < f_low) ++lo;
+  const int64_t lo = first_bin(f_low, df);
   int64_t hi = (int64_t)std::floor(fhi / df);
   while ((double)(hi + 1) * df <= fhi) ++hi;
   while (hi >= 0 && (double)hi * df > fhi) --hi;
   hi = std::min<int64_t>(hi, n / 2 - 1);
   t.k_lo = lo;
   t.k_hi = hi;
-  int K = 1;
-  while (2.0 * K * df <= 0.25 && 2 * K <= std::max<int64_t>(lo / 4, 1) && K < 1024) K *= 2;
-  int lg = 0;
-  while ((1 << lg) < K) ++lg;
-  t.K_log2 = lg;
+  t.K_log2 = anchor_log2(lo, df);
   return t;
 }
 
-cudaError_t launch_taylorf2(const double* m1, const double* m2, int64_t n_tmpl, double fs, int64_t n, double f_low,
-                            float2* out, int64_t ld, cudaStream_t st) {
-  if (n_tmpl < 1 || n < 16 || !(fs > 0) || !(f_low > 0) || ld < n / 2 + 1) return cudaErrorInvalidValue;
+// anchors of a row: -1 .. the second past the last bin
+static int anchor_count(int64_t n, double fs, double f_low) {
+  const double df = fs / (double)n;
+  const int lg = anchor_log2(first_bin(f_low, df), df);
+  return (int)(((n / 2 + 1 + (1 << lg) - 1) >> lg) + 4);
+}
+
+size_t taylorf2_table_bytes(int64_t n_tmpl) { return ((size_t)n_tmpl * sizeof(TF2) + 255) / 256 * 256; }
+
+size_t taylorf2_work_bytes(int64_t n_rows, double fs, int64_t n, double f_low) {
+  return ((size_t)n_rows * anchor_count(n, fs, f_low) * sizeof(double) + 255) / 256 * 256;
+}
+
+cudaError_t taylorf2_tables(const double* m1, const double* m2, int64_t n_tmpl, double fs, int64_t n, double f_low,
+                            void* dev, cudaStream_t st) {
   std::vector<TF2> h((size_t)n_tmpl);
-  for (int64_t i = 0; i < n_tmpl; ++i) {
-    if (!(m1[i] > 0) || !(m2[i] > 0)) return cudaErrorInvalidValue;
-    h[(size_t)i] = make_tf2(m1[i], m2[i], fs, n, f_low);
-  }
-  TF2* d = nullptr;
-  cudaError_t e = cudaMallocAsync(&d, (size_t)n_tmpl * sizeof(TF2), st);
-  if (e != cudaSuccess) return e;
-  e = cudaMemcpyAsync(d, h.data(), (size_t)n_tmpl * sizeof(TF2), cudaMemcpyHostToDevice, st);
+  for (int64_t i = 0; i < n_tmpl; ++i) h[(size_t)i] = make_tf2(m1[i], m2[i], fs, n, f_low);
+  // pageable source: the copy has taken the host table by the time the call returns
+  return cudaMemcpyAsync(dev, h.data(), (size_t)n_tmpl * sizeof(TF2), cudaMemcpyHostToDevice, st);
+}
+
+bool taylorf2_valid(const double* m1, const double* m2, int64_t n_tmpl, double fs, int64_t n, double f_low) {
+  if (n_tmpl < 1 || n < 16 || !(fs > 0) || !(f_low > 0)) return false;
+  for (int64_t i = 0; i < n_tmpl; ++i)
+    if (!(m1[i] > 0) || !(m2[i] > 0)) return false;
+  return true;
+}
+
+cudaError_t launch_taylorf2(const void* tables, int64_t t0, int64_t n_rows, double fs, int64_t n, double f_low,
+                            void* work, float2* out, int64_t ld, cudaStream_t st) {
+  const double df = fs / (double)n;
   const int64_t nb = n / 2 + 1;
-  for (int64_t t0 = 0; e == cudaSuccess && t0 < n_tmpl; t0 += 65535) {
-    const dim3 grid((unsigned)((nb + kGenChunk - 1) / kGenChunk), (unsigned)std::min<int64_t>(65535, n_tmpl - t0));
-    k_taylorf2<<<grid, kGenThreads, 0, st>>>(d + t0, fs / (double)n, out + t0 * ld, ld, nb);
-    add_launches(1);
-    e = cudaGetLastError();
+  const int na = anchor_count(n, fs, f_low);
+  const TF2* d = static_cast<const TF2*>(tables) + t0;
+  double* psi = static_cast<double*>(work);
+  for (int64_t r = 0; r < n_rows; r += 65535) {
+    const unsigned rows = (unsigned)std::min<int64_t>(65535, n_rows - r);
+    k_tf2_anchors<<<dim3((unsigned)((na + kGenThreads - 1) / kGenThreads), rows), kGenThreads, 0, st>>>(
+        d + r, df, na, psi + r * na);
+    k_taylorf2<<<dim3((unsigned)((nb + kGenChunk - 1) / kGenChunk), rows), kGenThreads, 0, st>>>(
+        d + r, psi + r * na, na, df, out + r * ld, ld, nb);
+    add_launches(2);
   }
-  // the host table must outlive the copy: wait for it before the vector goes away
-  cudaError_t e2 = cudaStreamSynchronize(st);
-  cudaFreeAsync(d, st);
-  return e != cudaSuccess ? e : e2;
+  return cudaGetLastError();
 }
 
 }  // namespace mf
@@ -179,12 +221,22 @@ extern "C" mf_status mf_taylorf2(const double* m1, const double* m2, int64_t n_t
     mf::set_global_error("mf_taylorf2: null argument");
     return MF_EINVAL;
   }
-  cudaError_t e = mf::launch_taylorf2(m1, m2, n_tmpl, fs, n, f_low, static_cast<float2*>(out), ld,
-                                      static_cast<cudaStream_t>(cuda_stream));
-  if (e == cudaErrorInvalidValue) {
+  if (ld < n / 2 + 1 || !mf::taylorf2_valid(m1, m2, n_tmpl, fs, n, f_low)) {
     mf::set_global_error("mf_taylorf2: bad sizes, masses or band");
     return MF_EINVAL;
   }
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  const int64_t block = std::min<int64_t>(n_tmpl, 256);  // rows per launch: bounds the anchors' work space
+  const size_t table = mf::taylorf2_table_bytes(n_tmpl);
+  char* dev = nullptr;
+  cudaError_t e = cudaMalloc((void**)&dev, table + mf::taylorf2_work_bytes(block, fs, n, f_low));
+  if (e == cudaSuccess) e = mf::taylorf2_tables(m1, m2, n_tmpl, fs, n, f_low, dev, st);
+  for (int64_t r = 0; r < n_tmpl && e == cudaSuccess; r += block)
+    e = mf::launch_taylorf2(dev, r, std::min(block, n_tmpl - r), fs, n, f_low, dev + table,
+                            static_cast<float2*>(out) + r * ld, ld, st);
+  const cudaError_t e2 = cudaStreamSynchronize(st);
+  if (dev) cudaFree(dev);
+  if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) {
     mf::set_global_error(std::string("mf_taylorf2: ") + cudaGetErrorString(e));
     return MF_ECUDA;
