@@ -100,109 +100,195 @@ struct TrigRecC {
   float snr, phase;
 };
 
-// One CTA per trigger: thread-owned band partials in shared memory, then a
-// fixed-order reduction, so the result is bitwise reproducible.
-template <int BT, int QT>
-__global__ void __launch_bounds__(kCT) k_chisq(const TrigRecC* __restrict__ trig, const int64_t* __restrict__ count,
-                                               int64_t cap, const void* __restrict__ bank, int64_t ld_bank,
-                                               const void* __restrict__ q, int64_t ld_q, int n1, int n2,
-                                               const int32_t* __restrict__ edges, int p, const float* __restrict__ ratio,
-                                               const float* __restrict__ dscale, float* __restrict__ chi2,
-                                               float* __restrict__ newsnr) {
-  extern __shared__ float2 zs[];  // [kCT][p]
-  const int64_t n_trig = *count < cap ? *count : cap;
-  const int R = n1 / 2;
-  const int64_t half = (int64_t)R * n2;
+// chi^2 of a run of G triggers of one template and detector at a time.
+//
+// With k = k1 N2 + k2 the phase splits, exp(2 pi i k j / N) = exp(2 pi i k1 j / N1) exp(2 pi i k2 j / N), so a
+// thread takes one row k1 (or, below 256 rows, one of `parts` equal pieces of it, so that the CTA's pieces s are
+// consecutive ranges of bins), walks its k2 with the phases of k2 from a table that the whole CTA shares, and
+// turns the sum once.  Neighbouring threads read neighbouring k1, the bank's fastest index.  A band is a range
+// of bins, so most pieces lie in one band: sums of whole pieces go to whole[s], of a piece's part behind a
+// band's first bin to head[band], of its part in front of one to tail[band]; each has one writer, and a warp per
+// band adds them in a fixed order (FP64).  The triggers of a run share the loads: reading the template and the
+// data once per trigger from L2 would bound the kernel.  Before, a thread walked its own run of consecutive
+// elements (no two lanes in one line) with a phase recurrence, and one thread added all partial sums: 4,105 us
+// for the triggers of 150 templates of two detectors at N = 2^18, threshold 4.5 (2 MB of template and data each);
+// now 469 us.
+constexpr int kChiThreads = 256;
+constexpr int kChiRun = 4;  // triggers that share their loads
+
+template <int BT, int QT, int G>
+__device__ __forceinline__ void chisq_run(const TrigRecC* __restrict__ trig, int64_t it, const void* __restrict__ bank,
+                                          int64_t ld_bank, const void* __restrict__ q, int64_t ld_q, int n1, int n2,
+                                          const int32_t* __restrict__ edges, int p, const float* __restrict__ ratio,
+                                          const float* __restrict__ dscale, float* __restrict__ chi2,
+                                          float* __restrict__ newsnr, unsigned char* sm) {
+  const int R = n1 / 2, tid = threadIdx.x;
+  const int parts = R < kChiThreads ? kChiThreads / R : 1, len = n2 / parts, pieces = R * parts;
+  float2* ph = reinterpret_cast<float2*>(sm);  // [n2][G] phases of k2
+  float2* whole = ph + n2 * G;                 // [pieces][G]
+  float2* head = whole + pieces * G;           // [p][G]
+  float2* tail = head + p * G;                 // [p][G]
+  double2* zl = reinterpret_cast<double2*>(tail + p * G);  // [p][G]
+  int32_t* e = reinterpret_cast<int32_t*>(zl + p * G);     // [p + 1]
+  const TrigRecC tr = trig[it];
   const uint32_t N = (uint32_t)n1 * (uint32_t)n2;
-  for (int64_t it = blockIdx.x; it < n_trig; it += gridDim.x) {
-    const TrigRecC tr = trig[it];
-    const int32_t* e = edges + (int64_t)tr.tmpl * (p + 1);
-    const void* hrow = static_cast<const unsigned char*>(bank) + (int64_t)tr.tmpl * ld_bank * (BT == kBankF32 ? 8 : 4);
-    const void* qrow = static_cast<const unsigned char*>(q) + (int64_t)tr.det * ld_q * (QT == kBankF32 ? 8 : 4);
-    float2* my = zs + threadIdx.x * p;
-    for (int l = 0; l < p; ++l) my[l] = make_float2(0.f, 0.f);
-    const uint32_t j = (uint32_t)tr.sample;
-    // step of the phase along a column (k += N2): exp(+2 pi i j / N1)
-    float ss, cs;
-    sincospif(2.0f * (float)(j % (uint32_t)n1) / (float)n1, &ss, &cs);
-    const float2 step = make_float2(cs, ss);
-    const int64_t L = (half + kCT - 1) / kCT;
-    const int64_t i0 = threadIdx.x * L, i1 = i0 + L < half ? i0 + L : half;
-    float2 acc = make_float2(0.f, 0.f), ph = make_float2(1.f, 0.f);
-    int band = -1;
-    int64_t next = 0;  // first bin of the next band
-    for (int64_t i = i0; i < i1; ++i) {
-      const int k1 = (int)(i % R);
-      const int64_t k = (int64_t)k1 * n2 + i / R;
-      if (i == i0 || k1 == 0 || (k1 & 31) == 0) {
-        if (i == i0 || k1 == 0) {  // new column: find the band by bisection over the edges
-          if (band >= 0) {
-            my[band].x += acc.x;
-            my[band].y += acc.y;
-            acc = make_float2(0.f, 0.f);
+  const void* hrow = static_cast<const unsigned char*>(bank) + (int64_t)tr.tmpl * ld_bank * (BT == kBankF32 ? 8 : 4);
+  const void* qrow = static_cast<const unsigned char*>(q) + (int64_t)tr.det * ld_q * (QT == kBankF32 ? 8 : 4);
+  for (int i = tid; i < n2 * G; i += kChiThreads) {
+    const uint32_t j = (uint32_t)trig[it + i % G].sample;
+    ph[i] = unit_root((uint32_t)(((uint64_t)(i / G) * j) % N), N);
+  }
+  for (int i = tid; i < (pieces + 2 * p) * G; i += kChiThreads) whole[i] = make_float2(0.f, 0.f);
+  for (int i = tid; i <= p; i += kChiThreads) e[i] = edges[(int64_t)tr.tmpl * (p + 1) + i];
+  __syncthreads();
+  for (int s0 = tid; s0 < pieces; s0 += kChiThreads) {
+    const int k1 = s0 % R, part = s0 / R, c0 = part * len, s = k1 * parts + part;
+    const int first = k1 * n2 + c0;  // the piece's bins [first, first + len)
+    int lo = -1, hi = p + 1;         // largest l with e[l] <= first (-1: below the bands)
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (e[mid] <= first) lo = mid; else hi = mid;
+    }
+    int band = lo, begin = 0;                                          // of the current stretch
+    int next = band < p ? min(e[band + 1] - first, len) : len;         // its end
+    float2 acc[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) acc[g] = make_float2(0.f, 0.f);
+    auto flush = [&](int end) {  // the stretch [begin, end) of the piece is summed
+      if (band >= 0 && band < p && end > begin) {
+        float2* to = begin == 0 ? (end == len ? whole + s * G : tail + band * G) : head + band * G;
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+          const uint32_t j = (uint32_t)trig[it + g].sample;
+          to[g] = cmul(acc[g], unit_root((uint32_t)(((uint64_t)k1 * j) % (uint32_t)n1), (uint32_t)n1));
+        }
+      }
+#pragma unroll
+      for (int g = 0; g < G; ++g) acc[g] = make_float2(0.f, 0.f);
+    };
+    auto add = [&](int c, float2 qv, float2 hv) {
+      const float2 x = cmulc(qv, hv);
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        const float2 w = ph[(c0 + c) * G + g];
+        acc[g].x = fmaf(x.x, w.x, fmaf(-x.y, w.y, acc[g].x));
+        acc[g].y = fmaf(x.x, w.y, fmaf(x.y, w.x, acc[g].y));
+      }
+    };
+    constexpr int U = 8;  // loads in flight (len is a multiple of 8)
+    for (int c = 0; c < len; c += U) {
+      float2 qv[U], hv[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int64_t i = (int64_t)(c0 + c + u) * R + k1;
+        qv[u] = elem<QT>(qrow, i);
+        hv[u] = elem<BT>(hrow, i);
+      }
+      if (c + U <= next) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) add(c + u, qv[u], hv[u]);
+      } else {
+#pragma unroll 1
+        for (int u = 0; u < U; ++u) {  // (loads again: their values stay in registers only in the unrolled path)
+          while (c + u == next && next < len) {  // the next band (or an empty one) begins here
+            flush(next);
+            begin = next;
+            ++band;
+            next = band < p ? min(e[band + 1] - first, len) : len;
           }
-          int lo = -1, hi = p;  // largest l with e[l] <= k (-1: below the band)
-          while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (e[mid] <= k) lo = mid; else hi = mid;
-          }
-          band = lo;
-          next = band + 1 <= p ? e[band + 1] : (int64_t)1 << 62;
+          const int64_t i = (int64_t)(c0 + c + u) * R + k1;
+          add(c + u, elem<QT>(qrow, i), elem<BT>(hrow, i));
         }
-        // exact phase exp(+2 pi i k j / N) every 32 bins of a column
-        const uint32_t m = (uint32_t)(((uint64_t)k * j) % N);
-        sincospif(2.0f * (float)m / (float)N, &ss, &cs);
-        ph = make_float2(cs, ss);
       }
-      while (k >= next && band < p) {  // bands advance with k inside a column
-        if (band >= 0) {
-          my[band].x += acc.x;
-          my[band].y += acc.y;
-        }
-        acc = make_float2(0.f, 0.f);
-        ++band;
-        next = band + 1 <= p ? e[band + 1] : (int64_t)1 << 62;
-      }
-      if (band >= 0 && band < p) {
-        const float2 x = cmulc(elem<QT>(qrow, i), elem<BT>(hrow, i));
-        const float2 y = cmul(x, ph);
-        acc.x += y.x;
-        acc.y += y.y;
-      }
-      ph = cmul(ph, step);
     }
-    if (band >= 0 && band < p) {
-      my[band].x += acc.x;
-      my[band].y += acc.y;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      // z_l in stored units (data / sigma_ref, template / scale): |z_true| = |z| ratio / c_d
-      float r = ratio[tr.tmpl];
-      if (dscale) r /= dscale[tr.det];
-      double zl_re[64], zl_im[64], z_re = 0.0, z_im = 0.0;
-      for (int l = 0; l < p; ++l) {
-        double a = 0.0, b = 0.0;
-        for (int th = 0; th < kCT; ++th) {
-          a += zs[th * p + l].x;
-          b += zs[th * p + l].y;
-        }
-        zl_re[l] = a;
-        zl_im[l] = b;
-        z_re += a;
-        z_im += b;
+    flush(len);
+  }
+  __syncthreads();
+  // z_l: the pieces of band l, by a warp
+  const int lane = tid & 31;
+  for (int i = tid / 32; i < p * G; i += kChiThreads / 32) {
+    const int l = i / G, g = i % G;
+    const int s_lo = e[l] / len, s_hi = (e[l + 1] < R * n2 ? e[l + 1] : R * n2) / len;  // whole pieces: (s_lo, s_hi)
+    double a = 0.0, b = 0.0;
+    if (e[l] < e[l + 1]) {
+      for (int s = s_lo + lane; s < s_hi; s += 32) {
+        if (s == s_lo && e[l] % len != 0) continue;  // its part in this band is head[l]
+        a += whole[s * G + g].x;
+        b += whole[s * G + g].y;
       }
-      double c2 = 0.0;
-      for (int l = 0; l < p; ++l) {
-        const double dr = zl_re[l] - z_re / p, di = zl_im[l] - z_im / p;
-        c2 += dr * dr + di * di;
+      if (lane == 0) {
+        a += head[i].x + (double)tail[i].x;
+        b += head[i].y + (double)tail[i].y;
       }
-      c2 *= (double)p * (double)r * (double)r;
-      chi2[it] = (float)c2;
-      const double cr = c2 / (2.0 * p - 2.0);
-      newsnr[it] = cr >= 1.0 ? (float)((double)tr.snr / pow((1.0 + cr * cr * cr) / 2.0, 1.0 / 6.0)) : tr.snr;
     }
-    __syncthreads();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    if (lane == 0) zl[i] = make_double2(a, b);
+  }
+  __syncthreads();
+  if (tid < G) {
+    // z_l in stored units (data / sigma_ref, template / scale): |z_true| = |z| ratio / c_d
+    float r = ratio[tr.tmpl];
+    if (dscale) r /= dscale[tr.det];
+    double zr = 0.0, zi = 0.0, c2 = 0.0;
+    for (int l = 0; l < p; ++l) {
+      zr += zl[l * G + tid].x;
+      zi += zl[l * G + tid].y;
+    }
+    for (int l = 0; l < p; ++l) {
+      const double dr = zl[l * G + tid].x - zr / p, di = zl[l * G + tid].y - zi / p;
+      c2 += dr * dr + di * di;
+    }
+    c2 *= (double)p * (double)r * (double)r;
+    chi2[it + tid] = (float)c2;
+    const double cr = c2 / (2.0 * p - 2.0);
+    const float snr = trig[it + tid].snr;
+    newsnr[it + tid] = cr >= 1.0 ? (float)((double)snr / pow((1.0 + cr * cr * cr) / 2.0, 1.0 / 6.0)) : snr;
+  }
+  __syncthreads();
+}
+
+constexpr int chisq_smem(int n1, int n2, int p, int g) {
+  const int pieces = n1 / 2 < kChiThreads ? kChiThreads : n1 / 2;
+  return (n2 + pieces + 2 * p) * g * 8 + p * g * 16 + (p + 1) * 4;
+}
+
+constexpr int kChisqSmemMax = chisq_smem(1024, 1024, 64, kChiRun);  // 57 KB, four CTAs per SM
+
+// A CTA takes blocks of `per` consecutive triggers (the list is ordered by detector and template), as runs of
+// the same detector and template; per grows to kChiRun with the number of triggers, so that few of them still
+// spread over the grid.
+template <int BT, int QT>
+__global__ void __launch_bounds__(kChiThreads) k_chisq(const TrigRecC* __restrict__ trig,
+                                                       const int64_t* __restrict__ count, int64_t cap,
+                                                       const void* __restrict__ bank, int64_t ld_bank,
+                                                       const void* __restrict__ q, int64_t ld_q, int n1, int n2,
+                                                       const int32_t* __restrict__ edges, int p,
+                                                       const float* __restrict__ ratio,
+                                                       const float* __restrict__ dscale, float* __restrict__ chi2,
+                                                       float* __restrict__ newsnr) {
+  extern __shared__ __align__(16) unsigned char smc[];
+  const int64_t n_trig = *count < cap ? *count : cap;
+  const int64_t per = min((int64_t)kChiRun, (n_trig + gridDim.x - 1) / gridDim.x);
+  for (int64_t b = blockIdx.x * per; b < n_trig; b += gridDim.x * per) {
+    const int64_t end = min(b + per, n_trig);
+    for (int64_t it = b; it < end;) {
+      int64_t to = it + 1;
+      while (to < end && trig[to].tmpl == trig[it].tmpl && trig[to].det == trig[it].det) ++to;
+      if (to - it == kChiRun) {
+        chisq_run<BT, QT, kChiRun>(trig, it, bank, ld_bank, q, ld_q, n1, n2, edges, p, ratio, dscale, chi2, newsnr, smc);
+        it = to;
+      } else if (to - it >= 2) {
+        chisq_run<BT, QT, 2>(trig, it, bank, ld_bank, q, ld_q, n1, n2, edges, p, ratio, dscale, chi2, newsnr, smc);
+        it += 2;
+      } else {
+        chisq_run<BT, QT, 1>(trig, it, bank, ld_bank, q, ld_q, n1, n2, edges, p, ratio, dscale, chi2, newsnr, smc);
+        it += 1;
+      }
+    }
   }
 }
 
@@ -257,11 +343,16 @@ cudaError_t launch_chisq(const void* trig, const int64_t* count, int64_t cap, co
                          int p, const float* ratio, const float* dscale, float* chi2, float* newsnr, cudaStream_t st) {
   if (p < 2 || p > 64) return cudaErrorInvalidValue;
   const int grid = sms_c() * 4;
-  const size_t smem = (size_t)kCT * p * sizeof(float2);
+  const int smem = chisq_smem(n1, n2, p, kChiRun);
   const TrigRecC* t = static_cast<const TrigRecC*>(trig);
-#define MF_CHISQ(BT, QT)                                                                                             \
-  k_chisq<BT, QT><<<grid, kCT, smem, st>>>(t, count, cap, bank, ld_bank, q, ld_q, n1, n2, edges, p, ratio, dscale, \
-                                           chi2, newsnr)
+#define MF_CHISQ(BT, QT)                                                                                        \
+  do {                                                                                                          \
+    auto k = k_chisq<BT, QT>;                                                                                   \
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kChisqSmemMax);  \
+    if (e != cudaSuccess) return e;                                                                             \
+    k<<<grid, kChiThreads, smem, st>>>(t, count, cap, bank, ld_bank, q, ld_q, n1, n2, edges, p, ratio, dscale, chi2, \
+                                       newsnr);                                                                 \
+  } while (0)
   if (q_type == kBankF32) {
     switch (bank_type) {
       case kBankF32: MF_CHISQ(kBankF32, kBankF32); break;
