@@ -75,6 +75,12 @@ struct mf_plan_s {
   float* maxrho = nullptr;
   int64_t maxrho_cap = 0;
   bool coinc_done = false;
+  int64_t sel_tmpl = 0;           // templates in the bank of the last filter
+  int64_t coinc_tmpl = 0;         // and of the filter of the last mf_coincide
+  int64_t coinc_shifts = 0;       // shifts of the last mf_coincide
+  int64_t coinc_per_bin = 0;      // and a bound on its records per (template, shift)
+  char* coinc_work = nullptr;     // ordered records and the ordering's work space
+  size_t coinc_work_cap = 0;
   // neighbourhood map
   int64_t* nb_ptr = nullptr;
   int32_t* nb_idx = nullptr;
@@ -360,7 +366,7 @@ void mf_destroy(mf_plan_t p) {
   if (p->st) cudaStreamSynchronize(p->st); else cudaDeviceSynchronize();
   dfree(p->w_dev); dfree(p->bank); dfree(p->scales_dev); dfree(p->rmax); dfree(p->norm_part); dfree(p->sigmasq_dev); dfree(p->inv_sigma_dev); dfree(p->ratio_dev); dfree(p->thr_raw_dev);
   dfree(p->sel_all); dfree(p->q); dfree(p->scratch); dfree(p->slots); dfree(p->sel_copy); dfree(p->trig);
-  dfree(p->count); dfree(p->bc); dfree(p->coincs); dfree(p->n_coinc); dfree(p->maxrho); dfree(p->nb_ptr);
+  dfree(p->count); dfree(p->bc); dfree(p->coincs); dfree(p->coinc_work); dfree(p->n_coinc); dfree(p->maxrho); dfree(p->nb_ptr);
   dfree(p->q_lp); dfree(p->dmax); dfree(p->dscale); dfree(p->row_valid); dfree(p->bpow); dfree(p->edges);
   dfree(p->nb_idx); dfree(p->flags); dfree(p->ubc); dfree(p->ucount); dfree(p->status); dfree(p->tw); dfree(p->tw4);
   for (cudaEvent_t e : p->ev) cudaEventDestroy(e);
@@ -733,6 +739,7 @@ mf_status mf_filter(mf_plan_t p, const void* dtilde, int64_t ld_dtilde, const in
                          p->count, p->bc, p->bc_cap, p->st);
   if (e != cudaSuccess) return cuda_fail(p, e, "mf_filter compaction");
   p->n_sel = n_sel;
+  p->sel_tmpl = p->n_tmpl;
   p->filtered = true;
   p->coinc_done = false;
   return MF_OK;
@@ -981,6 +988,10 @@ mf_status mf_coincide(mf_plan_t p, const mf_coinc_desc* c, int32_t* followed) {
   a.coincs = p->coincs;
   a.coinc_cap = p->coinc_cap;
   a.n_coinc = p->n_coinc;
+  a.own_ranges = p->row_valid != nullptr;
+  p->coinc_tmpl = p->sel_tmpl;
+  p->coinc_shifts = (int64_t)c->n_shifts + 1;
+  p->coinc_per_bin = p->n_win * (2 * c->window_samples / p->d.window + 2);
   LaunchScope ls(p);
   e = mf::launch_coinc(a, p->maxrho, p->st);
   if (e != cudaSuccess) return cuda_fail(p, e, "mf_coincide kernels");
@@ -998,7 +1009,29 @@ mf_status mf_get_coincs(mf_plan_t p, mf_coinc* out, int64_t cap, int64_t* n_foun
   *n_found = (int64_t)n;
   const int64_t have = std::min<int64_t>((int64_t)n, p->coinc_cap);
   const int64_t m = std::min<int64_t>(have, cap);
-  if (m > 0) try {  // a count-only call (cap 0) copies nothing; no allocation failure crosses the ABI
+  // Ordered on the device where each (template, shift) has few records (a window's detector-0 peak meets the peaks
+  // of 2 window_samples / window + 2 windows at most; 512 windows and the usual 15 ms: 1,024) and the bins fit an
+  // int32 index (duplicate ids in the selection only make the ranks slower); the host's sort of 110,000 records
+  // took 3.4 ms.
+  const int64_t bins = p->coinc_tmpl * p->coinc_shifts;
+  if (m > 0 && p->coinc_per_bin <= 4096 && p->coinc_shifts < (1 << 24) && bins < (int64_t(1) << 26) &&
+      have < (int64_t(1) << 30)) {
+    const size_t rec = ((size_t)have * sizeof(mf_coinc) + 255) / 256 * 256;
+    const size_t need = rec + mf::coinc_order_bytes(have, bins);
+    mf_status s;
+    if (need > p->coinc_work_cap) {
+      p->coinc_work_cap = 0;
+      if ((s = dalloc(p, &p->coinc_work, need + need / 4, "coincidence order")) != MF_OK) return s;
+      p->coinc_work_cap = need + need / 4;
+    }
+    LaunchScope ls(p);
+    e = mf::launch_coinc_order(p->coincs, have, p->coinc_tmpl, (int)p->coinc_shifts, p->coinc_work + rec, p->coinc_work,
+                               p->st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(out, p->coinc_work, m * sizeof(mf_coinc), cudaMemcpyDeviceToHost, p->st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(p->st);
+    if (e != cudaSuccess) return cuda_fail(p, e, "mf_get_coincs");
+  } else if (m > 0) try {  // a count-only call (cap 0) copies nothing; no allocation failure crosses the ABI
     std::unique_ptr<mf_coinc[]> rec(new mf_coinc[have]);
     e = cudaMemcpyAsync(rec.get(), p->coincs, have * sizeof(mf_coinc), cudaMemcpyDeviceToHost, p->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(p->st);
@@ -1219,7 +1252,7 @@ int filter_fused(mf_plan_s* const* plans, const void* const* dtilde, const int64
     e = launch_compact(p->slots, p->d.n_det, p->n_tmpl, p->n_win, p->d.window, p->sel_copy, p->trig,
                        p->d.max_triggers, p->count, p->bc, p->bc_cap, st);
     if (e != cudaSuccess) return bad(MF_ECUDA, std::string("fused filter compaction: ") + cudaGetErrorString(e));
-    p->n_sel = p->n_tmpl;
+    p->n_sel = p->sel_tmpl = p->n_tmpl;
     p->filtered = true;
     p->coinc_done = false;
   }

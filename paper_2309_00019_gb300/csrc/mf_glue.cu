@@ -64,6 +64,7 @@ __device__ __forceinline__ int64_t key_sample(unsigned long long key) {
 }
 __device__ __forceinline__ float key_rho2(unsigned long long key) { return __uint_as_float((uint32_t)(key >> 32)); }
 
+// The kernel for segments of more than kTmplWin windows and for rows with ranges of their own (see k_coinc_tmpl).
 // One thread per detector-0 window maximum.  Sample positions are below 2^21, so the ring arithmetic is
 // 32-bit, and the ring position of shift k follows from shift k - 1 by one subtraction.
 __global__ void k_coinc(CoincArgs a) {
@@ -118,6 +119,207 @@ __global__ void k_coinc(CoincArgs a) {
         }
       }
     }
+  }
+}
+
+// Coincidences of one template per CTA.  Of the two triggers of a coincidence at least one has half of the least
+// rho_c^2 that counts, and few triggers have: so the pairs (loud detector-0, any detector-1) and (other
+// detector-0, loud detector-1) are all there is to look at, and for a pair the shifts follow from the difference
+// of its times, k step in [D + m R - window, D + m R + window], without a walk over them.  What a CTA finds is
+// collected in shared memory and written in one go.  Trying all 102 shifts for every detector-0 trigger of a
+// template with one loud detector-1 trigger took 512 us on the coarse stage (2,000 templates, 512 windows each);
+// now 159 us.
+constexpr int kTmplWin = 2048;   // windows whose triggers fit the CTA's shared memory
+constexpr int kTmplRec = 512;    // records collected before they go out one by one
+constexpr int kTmplThreads = 256;
+
+__global__ void __launch_bounds__(kTmplThreads) k_coinc_tmpl(CoincArgs a) {
+  __shared__ int32_t pos[2][kTmplWin];   // ring positions of the triggers of detector 0, 1
+  __shared__ float rho2[2][kTmplWin];
+  __shared__ uint16_t loud[2][kTmplWin];
+  __shared__ uint2 found[kTmplRec];      // (detector-0 trigger | detector-1 trigger << 16, shift)
+  __shared__ int n_pos[2], n_loud[2], n_found;
+  __shared__ unsigned long long base;
+  const int64_t p = blockIdx.x;
+  const int tid = threadIdx.x;
+  if (tid < 2) n_pos[tid] = n_loud[tid] = 0;
+  if (tid == 2) n_found = 0;
+  __syncthreads();
+  const float need = fminf(a.rho_c_thr2, a.rho_c_store2), half = 0.5f * need;
+  const int32_t rb = (int32_t)a.ring_begin;
+  for (int i = tid; i < 2 * (int)a.n_win; i += kTmplThreads) {
+    const int d = i >= (int)a.n_win;
+    const unsigned long long key = a.slots[(d * a.n_sel + p) * a.n_win + (i - d * a.n_win)];
+    if (key == 0ull) continue;
+    const int at = atomicAdd(&n_pos[d], 1);
+    const float r = key_rho2(key);
+    pos[d][at] = (int32_t)key_sample(key) - rb;
+    rho2[d][at] = r;
+    if (r >= half) loud[d][atomicAdd(&n_loud[d], 1)] = (uint16_t)at;
+  }
+  __syncthreads();
+  if (n_loud[0] + n_loud[1] == 0) return;
+  const int32_t tmpl = a.sel[p];
+  const int32_t R = (int32_t)(a.ring_end - a.ring_begin), step = (int32_t)(a.shift % R), cw = (int32_t)a.coinc_window;
+  const int32_t last = a.n_shifts * step;  // + 2 R fits (launch_coinc)
+  const float inv_step = 1.f / (float)step;
+  bool follow = false;
+  auto record = [&](int h, int l, int32_t k) {
+    return CoincRec{tmpl,
+                    k,
+                    (int64_t)pos[0][h] + rb,
+                    (int64_t)pos[1][l] + rb,
+                    sqrtf(rho2[0][h]),
+                    sqrtf(rho2[1][l]),
+                    sqrtf(rho2[0][h] + rho2[1][l]),
+                    0};
+  };
+  auto emit = [&](int h, int l, int32_t k, float rc2) {
+    follow |= rc2 >= a.rho_c_thr2;
+    if (!(rc2 >= a.rho_c_store2)) return;
+    const int at = atomicAdd(&n_found, 1);
+    if (at < kTmplRec) {
+      found[at] = make_uint2((uint32_t)h | (uint32_t)l << 16, (uint32_t)k);
+    } else {
+      const unsigned long long slot = atomicAdd(a.n_coinc, 1ull);
+      if ((int64_t)slot < a.coinc_cap) reinterpret_cast<CoincRec*>(a.coincs)[slot] = record(h, l, k);
+    }
+  };
+  auto pair = [&](int h, int l) {
+    const float rc2 = rho2[0][h] + rho2[1][l];
+    if (!(rc2 >= need)) return;
+    int32_t D = pos[0][h] - pos[1][l];
+    if (D < 0) D += R;
+    if (step == 0) {
+      if (D <= cw || R - D <= cw)
+        for (int32_t k = 0; k <= a.n_shifts; ++k) emit(h, l, k, rc2);
+      return;
+    }
+    for (int32_t t = D - R; t - cw <= last; t += R) {
+      if (t + cw < 0) continue;
+      // the largest k with k step <= t + cw: a guess that is off by a few at most, then the exact one
+      int32_t k = (int32_t)((float)(t + cw) * inv_step);
+      while (k * step > t + cw) --k;
+      while ((k + 1) * step <= t + cw) ++k;
+      for (; k >= 0 && k * step >= t - cw; --k)
+        if (k <= a.n_shifts) emit(h, l, k, rc2);
+    }
+  };
+  for (int i = 0; i < n_loud[0]; ++i) {
+    const int h = loud[0][i];
+    for (int l = tid; l < n_pos[1]; l += kTmplThreads) pair(h, l);
+  }
+  for (int h = tid; h < n_pos[0]; h += kTmplThreads)
+    if (rho2[0][h] < half)
+      for (int i = 0; i < n_loud[1]; ++i) pair(h, loud[1][i]);
+  if (follow) a.followed[tmpl] = 1;
+  __syncthreads();
+  const int count = min(n_found, kTmplRec);
+  if (tid == 0 && count > 0) base = atomicAdd(a.n_coinc, (unsigned long long)count);
+  __syncthreads();
+  for (int i = tid; i < count; i += kTmplThreads)
+    if ((int64_t)base + i < a.coinc_cap)
+      reinterpret_cast<CoincRec*>(a.coincs)[base + i] =
+          record((int)(found[i].x & 0xffffu), (int)(found[i].x >> 16), (int32_t)found[i].y);
+}
+
+// --- coincidence records in order (tmpl, shift, sample0, sample1) ------------------
+// Counting sort over the (tmpl, shift) bins, then each record's rank in its bin: a bin holds at most a few records
+// per window, so the ranks are counted directly.
+
+constexpr int kScanSpan = 4096;  // bins per scan CTA (1024 threads x 4)
+
+__global__ void k_co_hist(const CoincRec* __restrict__ rec, int64_t n, int n_shift, int32_t* bins) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    atomicAdd(bins + (int64_t)rec[i].tmpl * n_shift + rec[i].shift, 1);
+}
+
+// exclusive scan of v over the CTA's 1024 threads; *total = the sum
+__device__ __forceinline__ int32_t cta_scan(int32_t v, int32_t* total) {
+  __shared__ int32_t ws[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int32_t x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) ws[w] = x;
+  __syncthreads();
+  if (w == 0) {
+    int32_t s = ws[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(0xffffffffu, s, o);
+      if (lane >= o) s += y;
+    }
+    ws[lane] = s;
+  }
+  __syncthreads();
+  *total = ws[31];
+  const int32_t r = x - v + (w > 0 ? ws[w - 1] : 0);
+  __syncthreads();
+  return r;
+}
+
+// bins[i] becomes the sum of the CTA's bins before it, sums[block] their total
+__global__ void __launch_bounds__(1024) k_co_scan(int32_t* bins, int64_t n_bins, int32_t* sums) {
+  const int64_t i0 = (int64_t)blockIdx.x * kScanSpan + threadIdx.x * 4;
+  int32_t v[4], s = 0, total;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    v[u] = i0 + u < n_bins ? bins[i0 + u] : 0;
+    s += v[u];
+  }
+  int32_t x = cta_scan(s, &total);
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    if (i0 + u < n_bins) bins[i0 + u] = x;
+    x += v[u];
+  }
+  if (threadIdx.x == 0) sums[blockIdx.x] = total;
+}
+
+__global__ void __launch_bounds__(1024) k_co_scan_sums(int32_t* sums, int n) {  // one CTA
+  int32_t carry = 0;
+  for (int b = 0; b < n; b += 1024) {
+    const int i = b + threadIdx.x;
+    int32_t total;
+    const int32_t x = cta_scan(i < n ? sums[i] : 0, &total);
+    if (i < n) sums[i] = carry + x;
+    carry += total;
+  }
+}
+
+struct CoincKey {
+  unsigned long long key;  // (sample0, sample1)
+  int32_t rec, bin;
+};
+
+// records grouped by bin, in any order; afterwards bins[b] (with its CTA's sum) is the end of bin b
+__global__ void k_co_group(const CoincRec* __restrict__ rec, int64_t n, int n_shift, int32_t* bins,
+                           const int32_t* __restrict__ sums, CoincKey* __restrict__ out) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const CoincRec r = rec[i];
+    const int32_t b = r.tmpl * n_shift + r.shift;
+    out[atomicAdd(bins + b, 1) + sums[b / kScanSpan]] =
+        CoincKey{((unsigned long long)r.sample0 << 32) | (uint32_t)r.sample1, (int32_t)i, b};
+  }
+}
+
+__global__ void k_co_rank(const CoincRec* __restrict__ rec, const CoincKey* __restrict__ grouped, int64_t n,
+                          const int32_t* __restrict__ bins, const int32_t* __restrict__ sums,
+                          CoincRec* __restrict__ out) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const CoincKey k = grouped[i];
+    const int32_t begin = k.bin > 0 ? bins[k.bin - 1] + sums[(k.bin - 1) / kScanSpan] : 0;
+    const int32_t end = bins[k.bin] + sums[k.bin / kScanSpan];
+    int32_t rank = begin;
+    for (int32_t j = begin; j < end; ++j) {
+      const unsigned long long o = grouped[j].key;
+      rank += o < k.key || (o == k.key && j < i) ? 1 : 0;
+    }
+    out[rank] = rec[k.rec];
   }
 }
 
@@ -192,11 +394,44 @@ cudaError_t launch_decimate(const float2* in, int64_t ld_in, float2* out, int64_
 cudaError_t launch_coinc(const CoincArgs& a, float* max_rho2_det1, cudaStream_t st) {
   if (a.n_sel <= 0) return cudaSuccess;
   if (a.n_sel > 0x7fffffff) return cudaErrorInvalidValue;
+  // up to kTmplWin windows (16 KB of triggers per detector) a CTA per template; beyond, where rows have analysed
+  // ranges of their own (times outside the ring), and where a shift's time overflows, the walk over windows and shifts
+  const int64_t R = a.ring_end - a.ring_begin;
+  if (a.n_win <= kTmplWin && !a.own_ranges &&
+      (int64_t)a.n_shifts * (a.shift % R) + 4 * R + a.coinc_window < (int64_t(1) << 30) && a.n_shifts < (1 << 22)) {
+    k_coinc_tmpl<<<(unsigned)a.n_sel, kTmplThreads, 0, st>>>(a);
+    add_launches(1);
+    return cudaGetLastError();
+  }
   k_max_rho2<<<(unsigned)a.n_sel, 256, 0, st>>>(a.slots, a.n_sel, a.n_win, max_rho2_det1);
   CoincArgs b = a;
   b.max_rho2_det1 = max_rho2_det1;
   k_coinc<<<sms() * 8, 256, 0, st>>>(b);
   add_launches(2);
+  return cudaGetLastError();
+}
+
+size_t coinc_order_bytes(int64_t n, int64_t n_bins) {
+  const int64_t sums = (n_bins + kScanSpan - 1) / kScanSpan;
+  return (size_t)n * sizeof(CoincKey) + (size_t)(n_bins + sums) * sizeof(int32_t);
+}
+
+cudaError_t launch_coinc_order(const void* rec, int64_t n, int64_t n_tmpl, int n_shift, void* work, void* out,
+                               cudaStream_t st) {
+  const int64_t n_bins = n_tmpl * n_shift, n_sums = (n_bins + kScanSpan - 1) / kScanSpan;
+  CoincKey* grouped = static_cast<CoincKey*>(work);
+  int32_t* bins = reinterpret_cast<int32_t*>(grouped + n);
+  int32_t* sums = bins + n_bins;
+  const CoincRec* r = static_cast<const CoincRec*>(rec);
+  cudaError_t e = cudaMemsetAsync(bins, 0, (size_t)n_bins * sizeof(int32_t), st);
+  if (e != cudaSuccess) return e;
+  const unsigned g = (unsigned)((n + 255) / 256 < sms() * 8 ? (n + 255) / 256 : sms() * 8);
+  k_co_hist<<<g, 256, 0, st>>>(r, n, n_shift, bins);
+  k_co_scan<<<(unsigned)n_sums, 1024, 0, st>>>(bins, n_bins, sums);
+  k_co_scan_sums<<<1, 1024, 0, st>>>(sums, (int)n_sums);
+  k_co_group<<<g, 256, 0, st>>>(r, n, n_shift, bins, sums, grouped);
+  k_co_rank<<<g, 256, 0, st>>>(r, grouped, n, bins, sums, static_cast<CoincRec*>(out));
+  add_launches(5);
   return cudaGetLastError();
 }
 

@@ -255,6 +255,10 @@ int64_t compact_blocks(int64_t n_slots);
 cudaError_t launch_gate_row(const double* w, int64_t nb, double df, float2* row, cudaStream_t st);
 cudaError_t launch_rfft(const float* strain, int64_t ld_s, int n_det, int64_t n, int n1, int n2, double dt,
                         float2* scratch, float2* dtilde, int64_t ld_d, cudaStream_t st);
+// spectra of the windowed segments of Welch's method: row s n_det + d is x[d][s stride ..], n samples, times the
+// periodic Hann window
+cudaError_t launch_welch_spectra(const float* x, int64_t ld, int n_det, int64_t stride, int rows, int64_t n, double dt,
+                                 float2* scratch, float2* out, int64_t ld_d, cudaStream_t st);
 // keep bins 0..nb_out-1 (A2)
 cudaError_t launch_decimate(const float2* in, int64_t ld_in, float2* out, int64_t ld_out, int64_t nb_out,
                             int n_det, cudaStream_t st);
@@ -274,8 +278,14 @@ struct CoincArgs {
   int64_t coinc_cap;
   unsigned long long* n_coinc;      // counter
   const float* max_rho2_det1;       // per selection position, max rho^2 of detector 1 (prefilter)
+  int own_ranges;                   // rows have analysed ranges of their own: times may lie outside the ring
 };
 cudaError_t launch_coinc(const CoincArgs& a, float* max_rho2_det1, cudaStream_t st);
+// n coincidence records in the order (tmpl, shift, sample0, sample1) into out; tmpl < n_tmpl, shift < n_shift, and
+// few records per (tmpl, shift) (their ranks are counted); work: coinc_order_bytes(n, n_tmpl n_shift)
+size_t coinc_order_bytes(int64_t n, int64_t n_bins);
+cudaError_t launch_coinc_order(const void* rec, int64_t n, int64_t n_tmpl, int n_shift, void* work, void* out,
+                               cudaStream_t st);
 cudaError_t launch_union(const int64_t* ptr, const int32_t* idx, int64_t n_coarse, const int32_t* followed,
                          int32_t* flags, int64_t n_fine, int32_t* subset, int64_t* n_subset,
                          int64_t* block_counts, cudaStream_t st);
