@@ -98,7 +98,7 @@ mf_status mf_set_psd(mf_plan_t plan, const double* psd, int64_t nbins);
  * (average = 0) or by the median divided by 1 - 1/2 + 1/3 - ... (m terms
  * after the first, m = (segments - 1) / 2; FINDCHIRP Appendix B; average = 1,
  * at most 4096 segments).  psd: device float64 [n_det][seg_len/2+1] (out).
- * Allocates segments x n_det x seg_len x 20 bytes of work space for the call.
+ * Allocates segments x n_det x seg_len x 12 bytes of work space for the call.
  * Synchronises.  Errors (mf_last_error(NULL)): MF_EINVAL, MF_ENOMEM, MF_ECUDA. */
 mf_status mf_psd_welch(double fs, int32_t n_det, int64_t n_samples, const float* strain, int64_t ld, int64_t seg_len,
                        int64_t stride, int32_t average, double* psd, void* cuda_stream);

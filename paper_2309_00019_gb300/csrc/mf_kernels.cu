@@ -100,6 +100,25 @@ struct RealLoad {
   }
 };
 
+// real strain in windowed, overlapping segments: row s n_det + d holds w[j] x[d][s stride + j], periodic Hann
+struct WelchLoad {
+  const float* x;
+  int64_t ld;
+  int n_det;
+  int64_t stride;
+  float n;
+  struct Ser {
+    const float* xs;
+  };
+  __device__ __forceinline__ Ser series(int r) const {
+    return Ser{x + (int64_t)(r % n_det) * ld + (int64_t)(r / n_det) * stride};
+  }
+  __device__ __forceinline__ float2 value(const Ser& se, int64_t j) const {
+    const float w = 0.5f - 0.5f * cospif(2.0f * (float)j / n);
+    return make_float2(__fmul_rn(w, __ldg(se.xs + j)), 0.f);  // rounded: not to be joined to the butterfly
+  }
+};
+
 // forward one-sided spectrum: dtilde[n] = dt * conj(z[n]) for n <= N/2
 struct SpectrumEpi {
   float2* out;
@@ -289,21 +308,33 @@ cudaError_t run_pass1_bt(const FilterArgs& a, cudaStream_t st) {
   }                                                  \
   return cudaErrorInvalidValue;
 
-template <int N1, int N2>
-cudaError_t run_rfft(const float* x, int64_t ld_s, int n_det, double dt, float2* scratch, float2* out,
-                     int64_t ld_d, cudaStream_t st) {
-  RealLoad ld{x, ld_s};
-  auto k1 = k_pass1<N1, N2, false, RealLoad>;
+template <int N1, int N2, class Load>
+cudaError_t run_spectra(const Load& ld, int rows, double dt, float2* scratch, float2* out, int64_t ld_d,
+                        cudaStream_t st) {
+  auto k1 = k_pass1<N1, N2, false, Load>;
   cudaError_t e = set_smem(k1, P1Geo<N1>::SMEM);
   if (e != cudaSuccess) return e;
-  k1<<<grid_for(n_det * (N2 / P1Geo<N1>::C), 2), kThreads, P1Geo<N1>::SMEM, st>>>(ld, scratch, n_det);
+  k1<<<grid_for(rows * (N2 / P1Geo<N1>::C), 2), kThreads, P1Geo<N1>::SMEM, st>>>(ld, scratch, rows);
   SpectrumEpi ep{out, ld_d, (int64_t)N1 * N2 / 2 + 1, (float)dt};
   auto k2 = k_pass2<N1, N2, SpectrumEpi>;
   e = set_smem(k2, P2Geo<N2>::SMEM);
   if (e != cudaSuccess) return e;
-  k2<<<grid_for(n_det * (N1 / P2Geo<N2>::RW), 2), kThreads, P2Geo<N2>::SMEM, st>>>(scratch, ep, n_det);
+  k2<<<grid_for(rows * (N1 / P2Geo<N2>::RW), 2), kThreads, P2Geo<N2>::SMEM, st>>>(scratch, ep, rows);
   g_launches += 2;
   return cudaGetLastError();
+}
+
+template <int N1, int N2>
+cudaError_t run_rfft(const float* x, int64_t ld_s, int n_det, double dt, float2* scratch, float2* out,
+                     int64_t ld_d, cudaStream_t st) {
+  return run_spectra<N1, N2>(RealLoad{x, ld_s}, n_det, dt, scratch, out, ld_d, st);
+}
+
+template <int N1, int N2>
+cudaError_t run_welch(const float* x, int64_t ld, int n_det, int64_t stride, int rows, double dt, float2* scratch,
+                      float2* out, int64_t ld_d, cudaStream_t st) {
+  return run_spectra<N1, N2>(WelchLoad{x, ld, n_det, stride, (float)((int64_t)N1 * N2)}, rows, dt, scratch, out, ld_d,
+                             st);
 }
 
 // ---------------------------------------------------------------------------
@@ -804,6 +835,11 @@ cudaError_t launch_rfft(const float* x, int64_t ld_s, int n_det, int64_t n, int 
   (void)n1;
   (void)n2;
   MF_DISPATCH_N(n, run_rfft, (x, ld_s, n_det, dt, scratch, out, ld_d, st))
+}
+
+cudaError_t launch_welch_spectra(const float* x, int64_t ld, int n_det, int64_t stride, int rows, int64_t n, double dt,
+                                 float2* scratch, float2* out, int64_t ld_d, cudaStream_t st) {
+  MF_DISPATCH_N(n, run_welch, (x, ld, n_det, stride, rows, dt, scratch, out, ld_d, st))
 }
 
 cudaError_t launch_quant_q(const float2* q, int64_t ld_q, int64_t nb, int n_det, int q_type, void* q_lp,

