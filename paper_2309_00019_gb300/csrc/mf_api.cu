@@ -57,7 +57,7 @@ struct mf_plan_s {
   int chisq_p = 0;
   float2* scratch = nullptr;
   int batch = 1;
-  CUtensorMap scratch_map{};  // pass-2 view of the scratch (mf::encode_scratch_map)
+  mf::ScratchMaps maps{};     // tensor maps of the scratch (mf::encode_scratch_maps)
   unsigned long long* slots = nullptr;
   int64_t slots_cap = 0;        // in slots
   int32_t* sel_copy = nullptr;  // the selection of the last filter (device copy)
@@ -344,7 +344,7 @@ mf_status mf_plan(mf_plan_t* out, const mf_plan_desc* desc) {
     mf_destroy(p);
     return s;
   }
-  if (mf::encode_scratch_map(d.n, p->scratch, scratch_series * d.n_det, &p->scratch_map) != cudaSuccess) {
+  if (mf::encode_scratch_maps(d.n, p->scratch, scratch_series * d.n_det, &p->maps) != cudaSuccess) {
     g_err = "mf_plan: tensor map of the scratch";
     mf_destroy(p);
     return MF_ECUDA;
@@ -593,7 +593,7 @@ mf_status mf_set_batch(mf_plan_t p, int32_t batch) {
   mf_status s = dalloc(p, &p->scratch, (size_t)series * per, "scratch");
   if (s != MF_OK) return s;
   p->batch = batch;
-  if (mf::encode_scratch_map(p->d.n, p->scratch, series * p->d.n_det, &p->scratch_map) != cudaSuccess)
+  if (mf::encode_scratch_maps(p->d.n, p->scratch, series * p->d.n_det, &p->maps) != cudaSuccess)
     return fail(p, MF_ECUDA, "mf_set_batch: tensor map of the scratch");
   return MF_OK;
 }
@@ -725,10 +725,10 @@ mf_status mf_filter(mf_plan_t p, const void* dtilde, int64_t ld_dtilde, const in
     const bool prof = p->prof && p->prof_count++ % p->prof_stride == 0 && (int)p->samples.size() < kProfBatches;
     const int e0 = prof ? (int)p->samples.size() * 3 : 0;
     if (prof) cudaEventRecord(p->ev[e0], p->st);
-    e = mf::launch_filter2_pass1(a, p->st);
+    e = mf::launch_filter2_pass1(a, p->maps, p->st);
     if (e != cudaSuccess) return cuda_fail(p, e, "mf_filter pass 1");
     if (prof) cudaEventRecord(p->ev[e0 + 1], p->st);
-    e = mf::launch_filter2_pass2(a, p->scratch_map, p->st);
+    e = mf::launch_filter2_pass2(a, p->maps, p->st);
     if (e != cudaSuccess) return cuda_fail(p, e, "mf_filter pass 2");
     if (prof) {
       cudaEventRecord(p->ev[e0 + 2], p->st);
@@ -1143,7 +1143,7 @@ namespace mf {
 int plan_batch(const mf_plan_s* p) { return p ? p->batch : 0; }
 
 int filter_fused(mf_plan_s* const* plans, const void* const* dtilde, const int64_t* ld, int n_plans, void* scratch,
-                 int64_t scratch_series, const CUtensorMap& scratch_map, cudaStream_t st, std::string* err) {
+                 int64_t scratch_series, const ScratchMaps& maps, cudaStream_t st, std::string* err) {
   auto bad = [&](mf_status s, const std::string& m) {
     if (err) *err = m;
     return s;
@@ -1240,7 +1240,7 @@ int filter_fused(mf_plan_s* const* plans, const void* const* dtilde, const int64
         p0->prof && p0->prof_count++ % p0->prof_stride == 0 && (int)p0->samples.size() < kProfBatches;
     const int e0 = prof ? (int)p0->samples.size() * 3 : 0;
     if (prof) cudaEventRecord(p0->ev[e0], st);
-    if ((e = launch_filter2_fused(a, ps, scratch_map, st, prof ? p0->ev[e0 + 1] : nullptr)) != cudaSuccess)
+    if ((e = launch_filter2_fused(a, ps, maps, st, prof ? p0->ev[e0 + 1] : nullptr)) != cudaSuccess)
       return bad(MF_ECUDA, std::string("fused filter launch: ") + cudaGetErrorString(e));
     if (prof) {
       cudaEventRecord(p0->ev[e0 + 2], st);

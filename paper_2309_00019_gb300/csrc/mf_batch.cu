@@ -74,10 +74,10 @@ struct mf_batch_s {
     float2* fd = nullptr;
   };
   std::vector<Cls> cls;
-  // fused runs: the scratch of one launch pair (fscratch_series series of N = fscratch_n) and its pass-2 map
+  // fused runs: the scratch of one launch pair (fscratch_series series of N = fscratch_n) and its tensor maps
   float2* fscratch = nullptr;
   int64_t fscratch_series = 0, fscratch_n = 0;
-  CUtensorMap fmap{};
+  mf::ScratchMaps fmap{};
   // captured graph of one MF_RUN_STREAMS (or MF_RUN_FUSED) pass
   cudaGraphExec_t exec = nullptr;
   int32_t g_mode = -1;
@@ -278,7 +278,7 @@ mf_status ensure_fused(mf_batch_s* b) {
     b->fscratch = nullptr;
     return bfail(b, MF_ENOMEM, std::string("mf_batch_run fused scratch: ") + cudaGetErrorString(e));
   }
-  e = mf::encode_scratch_map(n, b->fscratch, series, &b->fmap);
+  e = mf::encode_scratch_maps(n, b->fscratch, series, &b->fmap);
   if (e != cudaSuccess) return bcuda(b, e, "mf_batch_run fused scratch map");
   b->fscratch_n = n;
   b->fscratch_series = series;

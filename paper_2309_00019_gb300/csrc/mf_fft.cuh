@@ -216,6 +216,149 @@ __device__ __forceinline__ void dft(float2 (&v)[R]) {
   Dft<R, ZH>::run(v, 0, 1);
 }
 
+// ---------------------------------------------------------------------------
+// The 32-point transform on register pairs.  Packed FP32 instructions (add, multiply, fused multiply-add on two
+// adjacent registers) take the FMA pipe as long as two scalar ones but one issue slot.  The early butterfly stages,
+// which do the same to neighbouring inputs, run packed over the inputs (i, i + 1); the last stage, whose operands are
+// the two halves of a pair, runs scalar (a pair's halves are ordinary registers, so nothing is moved).  Real and
+// imaginary parts are separate arrays; multiplications by +-i are a choice of array and sign.
+// Every operation and its rounding is that of Dft<32>, where the compiler joins the factor sqrt(1/2) of an eighth root
+// to the addition that follows: the factor is kept pending and joined by hand (fma), of two such terms the first.
+// ---------------------------------------------------------------------------
+
+constexpr float kSqrtHalf = 0.707106781186547524f;
+
+__device__ __forceinline__ float2 at2(const float* x, int i) { return make_float2(x[i], x[i + 1]); }
+__device__ __forceinline__ void put2(float* x, int i, float2 v) {
+  x[i] = v.x;
+  x[i + 1] = v.y;
+}
+__device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 psub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+
+// 4-point DFT of the inputs i + s {0, 1, 2, 3} and, in the other lane, of the next ones, in place
+template <bool ZH>
+__device__ __forceinline__ void dft4_lanes(float* x, float* y, int i, int s) {
+  const float2 x0 = at2(x, i), y0 = at2(y, i), x1 = at2(x, i + s), y1 = at2(y, i + s);
+  float2 ax, ay, bx, by, cx, cy, dx, dy;  // t0, t1, t2 and x1 - x3
+  if constexpr (ZH) {
+    ax = bx = x0;
+    ay = by = y0;
+    cx = dx = x1;
+    cy = dy = y1;
+  } else {
+    const float2 x2 = at2(x, i + 2 * s), y2 = at2(y, i + 2 * s), x3 = at2(x, i + 3 * s), y3 = at2(y, i + 3 * s);
+    ax = padd(x0, x2);
+    ay = padd(y0, y2);
+    bx = psub(x0, x2);
+    by = psub(y0, y2);
+    cx = padd(x1, x3);
+    cy = padd(y1, y3);
+    dx = psub(x1, x3);
+    dy = psub(y1, y3);
+  }
+  put2(x, i, padd(ax, cx));
+  put2(y, i, padd(ay, cy));
+  put2(x, i + 2 * s, psub(ax, cx));
+  put2(y, i + 2 * s, psub(ay, cy));
+  put2(x, i + s, psub(bx, dy));
+  put2(y, i + s, padd(by, dx));
+  put2(x, i + 3 * s, padd(bx, dy));
+  put2(y, i + 3 * s, psub(by, dx));
+}
+
+// (x, y) times exp(2 pi i E / R); an eighth root leaves its factor sqrt(1/2) pending
+template <int E, int R>
+__device__ __forceinline__ void rotate(float& x, float& y) {
+  static_assert(E >= 0 && 8 * E < 8 * R && 8 * E != 5 * R && 8 * E != 7 * R, "rotations of the splits used here");
+  const float a = x, b = y;
+  if constexpr (E == 0) {
+  } else if constexpr (4 * E == R) {
+    x = -b;
+    y = a;
+  } else if constexpr (8 * E == R) {
+    x = a - b;
+    y = a + b;
+  } else if constexpr (8 * E == 3 * R) {
+    x = -(a + b);
+    y = a - b;
+  } else {
+    constexpr float c = (float)kcossin(E, R, 0), s = (float)kcossin(E, R, 1);
+    x = fmaf(a, c, -b * s);
+    y = fmaf(a, s, b * c);
+  }
+}
+
+// 4-point DFT whose first sums t0, t2 and differences t1, d are formed already: out[o + st {0, 1, 2, 3}]
+__device__ __forceinline__ void dft4_last(float2* out, int o, int st, float t0x, float t0y, float t1x, float t1y,
+                                          float t2x, float t2y, float dx, float dy) {
+  out[o] = make_float2(t0x + t2x, t0y + t2y);
+  out[o + st] = make_float2(t1x - dy, t1y + dx);
+  out[o + 2 * st] = make_float2(t0x - t2x, t0y - t2y);
+  out[o + 3 * st] = make_float2(t1x + dy, t1y - dx);
+}
+
+// 8-point DFT of x[i .. i + 7] into out[o + 4 q].  PEND: bit r set where input r has sqrt(1/2) pending (input 4, or
+// 2 and 6).
+template <int PEND>
+__device__ __forceinline__ void dft8_last(const float* x, const float* y, int i, float2* out, int o) {
+  static_assert(PEND == 0 || PEND == (1 << 4) || PEND == ((1 << 2) | (1 << 6)), "pending inputs");
+  float sx[4], sy[4], dx[4], dy[4];  // sums and differences of inputs r, r + 4
+#pragma unroll
+  for (int h = 0; h < 4; h += 2) {
+    const float2 ax = at2(x, i + h), ay = at2(y, i + h);
+    float2 bx = at2(x, i + h + 4), by = at2(y, i + h + 4);
+    const float2 f = make_float2(kSqrtHalf, 1.f), g = make_float2(-kSqrtHalf, -1.f);
+    if (PEND == (1 << 4) && h == 0) {
+      put2(sx, h, __ffma2_rn(bx, f, ax));
+      put2(sy, h, __ffma2_rn(by, f, ay));
+      put2(dx, h, __ffma2_rn(bx, g, ax));
+      put2(dy, h, __ffma2_rn(by, g, ay));
+    } else if (PEND == ((1 << 2) | (1 << 6)) && h == 2) {
+      bx.x *= kSqrtHalf;
+      by.x *= kSqrtHalf;
+      put2(sx, h, __ffma2_rn(ax, f, bx));
+      put2(sy, h, __ffma2_rn(ay, f, by));
+      put2(dx, h, __ffma2_rn(ax, f, make_float2(-bx.x, -bx.y)));
+      put2(dy, h, __ffma2_rn(ay, f, make_float2(-by.x, -by.y)));
+    } else {
+      put2(sx, h, padd(ax, bx));
+      put2(sy, h, padd(ay, by));
+      put2(dx, h, psub(ax, bx));
+      put2(dy, h, psub(ay, by));
+    }
+  }
+  {
+    const float2 tx = padd(at2(sx, 0), at2(sx, 2)), ty = padd(at2(sy, 0), at2(sy, 2));
+    const float2 ux = psub(at2(sx, 0), at2(sx, 2)), uy = psub(at2(sy, 0), at2(sy, 2));
+    dft4_last(out, o, 8, tx.x, ty.x, ux.x, uy.x, tx.y, ty.y, ux.y, uy.y);
+  }
+  {
+    const float e1x = dx[1] - dy[1], e1y = dx[1] + dy[1];
+    const float nx = -kSqrtHalf * (dx[3] + dy[3]), ny = kSqrtHalf * (dx[3] - dy[3]);
+    dft4_last(out, o + 4, 8, dx[0] - dy[2], dy[0] + dx[2], dx[0] + dy[2], dy[0] - dx[2], fmaf(kSqrtHalf, e1x, nx),
+              fmaf(kSqrtHalf, e1y, ny), fmaf(kSqrtHalf, e1x, -nx), fmaf(kSqrtHalf, e1y, -ny));
+  }
+}
+
+// out[q] = sum_r (x[r] + i y[r]) exp(2 pi i r q / 32).  x, y are overwritten.  ZH: the inputs r >= 16 are zero (not
+// read).
+template <bool ZH>
+__device__ __forceinline__ void dft_pairs(float (&x)[32], float (&y)[32], float2 (&out)[32]) {
+  // r = 8 r1 + r2, q = q1 + 4 q2
+#pragma unroll
+  for (int i = 0; i < 8; i += 2) dft4_lanes<ZH>(x, y, i, 8);
+  sfor<4>([&](auto q1c) {
+    constexpr int q1 = decltype(q1c)::value;
+    sfor<8>([&](auto r2c) {
+      constexpr int r2 = decltype(r2c)::value;
+      rotate<r2 * q1, 32>(x[8 * q1 + r2], y[8 * q1 + r2]);
+    });
+    constexpr int pend = q1 == 0 ? 0 : q1 == 2 ? (1 << 2) | (1 << 6) : 1 << 4;
+    dft8_last<pend>(x, y, 8 * q1, out, q1);
+  });
+}
+
 // exp(+2 pi i p / q) for integers 0 <= p < q <= 2^24, q a power of two.
 __device__ __forceinline__ float2 unit_root(uint32_t p, uint32_t q) {
   float s, c;

@@ -177,24 +177,16 @@ __global__ void k_fill_twiddles(float2* tw) {
 // pass 1
 // ---------------------------------------------------------------------------
 
-// IM: the intermediate (FilterArgs::inter).  IM >= 1: FP16, each series scaled by series_scale16 of its
-// template, in panels of kPanel16 rows that are the tensor-core row pass's stage-1 operand image: with
-// k2 = 32 p + q, part c (0 real, 1 imaginary) of element (j1, k2) is the half at panel j1 / 8,
-// ((q 32 + p) 2 + c) 8 + j1 % 8 (an image of 2 N2 8 halves), i.e. the MN-major layout of rows
-// m = 8 q + j1 % 8 and columns k = 2 p + c.  IM = 2: each panel holds the image of hi = the value rounded
-// to FP16, then the image of lo = the remainder rounded to FP16.
 // MP: the series of several plans' parts (FilterParts), each with its own bank, data rows and selection
-template <int N1, int N2, int BT, int QT, int IM, bool MP>
+template <int N1, int N2, int BT, int QT, bool MP>
 __global__ void __launch_bounds__(kColThreads, 3) k_cols(FilterArgs a, const __grid_constant__ FilterParts ps) {
   static_assert(!MP || QT == kBankF32, "fused launches take FP32 weighted data");
-  constexpr bool H16 = IM >= 1;
-  constexpr int IMG = IM == 2 ? 2 : 1;  // FP16 images per panel
   using G = SubFft<N1>;
   using P = ColGeo<N1, BT, QT>;
   constexpr int RA = G::RA, RB = G::RB, T = G::T, NB = G::NB, C = P::C, R = P::R, S = P::S;
   constexpr int NCB = N2 / C;
   constexpr uint32_t N = (uint32_t)N1 * (uint32_t)N2;
-  constexpr int PH = H16 ? kPanel16 : ScratchGeo<N1, N2>::P;  // scratch panel height
+  constexpr int PH = ScratchGeo<N1, N2>::P;  // scratch panel height
   extern __shared__ __align__(128) unsigned char sm[];
   const float2* tw = reinterpret_cast<const float2*>(sm + P::TW_OFF);
   uint64_t* full = reinterpret_cast<uint64_t*>(sm + P::BAR_OFF);  // [0], [1]: tiles of the slot landed
@@ -284,17 +276,11 @@ __global__ void __launch_bounds__(kColThreads, 3) k_cols(FilterArgs a, const __g
     if (!mbar_wait_bounded(full + slot, (uint32_t)((k >> 1) & 1), a.status)) break;
     const unsigned char* col = sm + slot * P::SLOT + ca * S * 8;
     int li = item, nd = a.n_det, s0 = 0;
-    const int32_t* sel = a.sel;
-    const float* isg = a.inv_sigma;
-    int64_t pos0 = a.pos0;
     if constexpr (MP) {
       const FilterPart& p = ps.p[part_of(ps, item, NCB)];
       li = item - p.series0 * NCB;
       nd = p.n_det;
       s0 = p.series0;
-      sel = p.sel;
-      isg = p.inv_sigma;
-      pos0 = p.pos0;
     }
     const int s = s0 + (li / (nd * NCB)) * nd + li % nd;
     float2 v[RA];
@@ -314,10 +300,7 @@ __global__ void __launch_bounds__(kColThreads, 3) k_cols(FilterArgs a, const __g
     for (int q = 0; q < RA; ++q) xb[ta * RA + q + ta] = v[q];
     __syncwarp();
     float2* out = a.scratch + (int64_t)s * N;
-    __half* out16 = reinterpret_cast<__half*>(a.scratch) + (int64_t)s * 2 * IMG * N;
     const int k2 = ((li / nd) % NCB) * C + ca;
-    float sc = 1.f;
-    if constexpr (H16) sc = series_scale16(__ldg(isg + sel[pos0 + li / (nd * NCB)]));
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
       const int j = ta + T * i;
@@ -331,36 +314,7 @@ __global__ void __launch_bounds__(kColThreads, 3) k_cols(FilterArgs a, const __g
       const float2* twr = a.tw4 + (int64_t)k2 * (RA + 1);
       float2 w = __ldg(twr + j);
       const float2 st = __ldg(twr + RA);
-      if constexpr (H16) {
-        static_assert(RA % PH == 0 && N2 == 1024, "FP16 panels");
-        w.x *= sc;
-        w.y *= sc;
-        // j1 = j + q RA: q RA / 8 whole panels past j's; within a panel, (k2 % 32, k2 / 32, part, j1 % 8).
-        // Lanes j, j + 1 (j even) of the column swap halves so that each writes 4 bytes: j the real parts
-        // of rows j, j + 1 and j + 1 their imaginary parts (one warp store: four whole 32-byte sectors)
-        static_assert(T == 32, "lane pairs");
-        const bool odd = (j & 1) != 0;
-        constexpr int64_t IMAGE = 2 * N2 * PH;  // halves of one FP16 image of a panel
-        __half* ob = out16 + (int64_t)(j / PH) * (IMG * IMAGE) + (((k2 & 31) * 32 + (k2 >> 5)) * 2) * PH +
-                     (odd ? PH + (j % PH) - 1 : (j % PH));
-        auto pair_store = [&](__half* dst, __half2 h) {
-          const uint32_t mine = *reinterpret_cast<const uint32_t*>(&h);
-          const uint32_t other = __shfl_xor_sync(0xffffffffu, mine, 1);
-          *reinterpret_cast<uint32_t*>(dst) = odd ? __byte_perm(other, mine, 0x7632) : __byte_perm(mine, other, 0x5410);
-        };
-#pragma unroll
-        for (int q = 0; q < RB; ++q) {
-          const float2 z = cmul(u[q], w);
-          const __half2 h = __float22half2_rn(z);
-          __half* dq = ob + (int64_t)q * (RA / PH) * (IMG * IMAGE);
-          pair_store(dq, h);
-          if constexpr (IM == 2) {  // the remainder: z - hi is exact in FP32
-            const float2 hf = __half22float2(h);
-            pair_store(dq + IMAGE, __float22half2_rn(make_float2(z.x - hf.x, z.y - hf.y)));
-          }
-          if (q + 1 < RB) w = cmul(w, st);
-        }
-      } else if constexpr (RA % PH == 0) {  // j1 = j + q RA: q RA / PH whole panels past j's
+      if constexpr (RA % PH == 0) {  // j1 = j + q RA: q RA / PH whole panels past j's
         float2* ob = out + (int64_t)(j / PH) * (N2 * PH) + k2 * PH + (j % PH);
 #pragma unroll
         for (int q = 0; q < RB; ++q) {
@@ -382,6 +336,240 @@ __global__ void __launch_bounds__(kColThreads, 3) k_cols(FilterArgs a, const __g
     if ((tid & 31) == 0) mbar_arrive(empty + slot);
   }
   pdl_launch_dependents();  // our items are done: the next kernel may launch
+}
+
+// ---------------------------------------------------------------------------
+// pass 1 into the FP16 intermediate (N = 2^20)
+// ---------------------------------------------------------------------------
+
+// Read-only loads that stay where they are written (a load in front of a wait is not moved behind it)
+__device__ __forceinline__ float2 ldg_early(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float ldg_early(const float* p) {
+  float v;
+  asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ int32_t ldg_early(const int32_t* p) {
+  int32_t v;
+  asm volatile("ld.global.nc.s32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+
+constexpr int kImgWarps = 16;  // warps of k_cols16, one column each
+constexpr int kImgThreads = kImgWarps * 32;
+
+// Shared-memory plan of k_cols16: per warp a template tile and an exchange buffer, then the sub-FFT twiddles and the
+// barriers: per warp "tile landed", then the twiddles'.
+template <int BT>
+struct ImgGeo {
+  using G = SubFft<1024>;
+  static constexpr int R = 512;                           // non-zero half of k1
+  static constexpr int HB = BT == kBankF32 ? 8 : 4;       // bytes per template element
+  static constexpr int TILE = R * HB;                     // a column's template tile, bytes
+  static constexpr int XCH = round128(G::PAD * 8);
+  static constexpr int WARP = TILE + XCH;
+  static constexpr int TW_BYTES = G::RB * G::RA * 8;
+  static constexpr int TW_OFF = kImgWarps * WARP;
+  static constexpr int BAR_OFF = TW_OFF + TW_BYTES;
+  static constexpr int SMEM = BAR_OFF + (kImgWarps + 1) * 8;
+};
+
+// The column pass of k_cols for the FP16 intermediate of the tensor-core row pass: each series is scaled by
+// series_scale16 of its template and written in panels of kPanel16 rows that are the row pass's stage-1 operand
+// image: with k2 = 32 p + q, part c (0 real, 1 imaginary) of element (j1, k2) is the half at panel j1 / 8,
+// ((q 32 + p) 2 + c) 8 + j1 % 8 (an image of 2 N2 8 halves), i.e. the MN-major layout of rows m = 8 q + j1 % 8 and
+// columns k = 2 p + c.  IM = 2: each panel holds the image of hi = the value rounded to FP16, then the image of
+// lo = the remainder rounded to FP16.  MP: the series of several plans' parts (FilterParts).
+//
+// What bounds it is issue and the shared-memory / L1 data path together, with too few warps to hide one behind the
+// other.  So:
+//  - one CTA of 16 warps per SM, each with a column at a time and no barrier between them, instead of 12 in CTAs of
+//    four with a producer each.  There is room for them because only the template tile is staged (4 KB, copied in
+//    while the column before it is transformed); the weighted data, which all templates share and which L2 holds, go
+//    straight into registers during the second transform of the column before.
+//  - a column's values are staged over its exchange buffer in image order and scattered to the panels by one
+//    tensor-map store.  From registers, a shuffle and a four-line store per value made up a quarter of the wavefronts.
+//  - the transforms run in packed FP32 (dft_pairs).
+// Per launch of 121 series (two detectors, FP32 bank) 0.229 -> 0.210 ms; issue slots used 72 -> 78%, the L1 data path
+// 81 -> 74%.  Two series per thread, everything packed, issued a third less (34 instead of 50 instructions per
+// point) and was slower (0.219 ms): a packed multiply-add of three register pairs takes three cycles, not two.  The
+// FP32 column pass gains nothing from this form (it writes twice the bytes, near the memory's rate): k_cols stays.
+template <int BT, int IM, bool MP>
+__global__ void __launch_bounds__(kImgThreads, 1) k_cols16(const __grid_constant__ CUtensorMap tm, FilterArgs a,
+                                                            const __grid_constant__ FilterParts ps) {
+  constexpr int N1 = 1024, N2 = 1024, PH = kPanel16;
+  constexpr int IMG = IM == 2 ? 2 : 1;  // FP16 images per panel
+  using G = SubFft<N1>;
+  using P = ImgGeo<BT>;
+  constexpr int RA = G::RA, RB = G::RB, R = P::R;
+  static_assert(RA == 32 && RB == 32 && RA % PH == 0, "one column per warp, whole panels");
+  extern __shared__ __align__(128) unsigned char sm[];
+  const float2* tw = reinterpret_cast<const float2*>(sm + P::TW_OFF);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  unsigned char* tile = sm + warp * P::WARP;
+  float2* xb = reinterpret_cast<float2*>(tile + P::TILE);
+  uint64_t* full = reinterpret_cast<uint64_t*>(sm + P::BAR_OFF) + warp;       // the warp's tile landed
+  uint64_t* twb = reinterpret_cast<uint64_t*>(sm + P::BAR_OFF) + kImgWarps;   // the twiddle table landed
+  const int n_items = (MP ? ps.n_series : a.count * a.n_det) * N2;
+  const int stride = gridDim.x * kImgWarps;
+  struct Item {
+    int s, k2;            // series, column
+    int tmpl;
+    const void* h;        // the column's template tile
+    const float2* q;      // this thread's first weighted value
+    const float* ratio;   // of all templates
+  };
+  auto item_of = [&](int item) {
+    int li = item, nd = a.n_det, s0 = 0;
+    const int32_t* sel = a.sel;
+    const float* isg = a.inv_sigma;
+    int64_t pos0 = a.pos0, ld_bank = a.ld_bank, ld_q = a.ld_q;
+    const void* hb = a.bank;
+    const float2* qb = a.q;
+    if constexpr (MP) {
+      const FilterPart& p = ps.p[part_of(ps, item, N2)];
+      li = item - p.series0 * N2;
+      nd = p.n_det;
+      s0 = p.series0;
+      sel = p.sel;
+      isg = p.inv_sigma;
+      pos0 = p.pos0;
+      hb = p.bank;
+      ld_bank = p.ld_bank;
+      qb = p.q;
+      ld_q = p.ld_q;
+    }
+    // detector fastest: the n_det items of one bank tile run at the same time, so the tile is read from HBM once
+    // and from L2 for the other detectors; then columns 32 apart (the same q, consecutive p), whose parts of a
+    // panel share lines
+    Item it;
+    const int d = li % nd, cb = (li / nd) % N2, b = li / (nd * N2);
+    it.k2 = ((cb / 128) * 4 + cb % 4) * 32 + cb / 4 % 32;
+    it.s = s0 + b * nd + d;
+    it.tmpl = ldg_early(sel + pos0 + b);
+    it.h = static_cast<const unsigned char*>(hb) + ((int64_t)it.tmpl * ld_bank + (int64_t)it.k2 * R) * P::HB;
+    it.q = qb + (int64_t)d * ld_q + (int64_t)it.k2 * R + lane;
+    it.ratio = isg;
+    return it;
+  };
+  auto fetch = [&](const Item& it) {  // lane 0: the item's template tile
+    mbar_expect_tx(full, (uint32_t)P::TILE);
+    bulk_g2s(tile, it.h, (uint32_t)P::TILE, full);
+  };
+  float2 qv[RA / 2];  // the item's weighted data
+  auto load_q = [&](const Item& it) {
+#pragma unroll
+    for (int r = 0; r < RA / 2; ++r) qv[r] = ldg_early(it.q + r * RB);
+  };
+  if (lane == 0) mbar_init(full, 1);
+  if (tid == 0) mbar_init(twb, 1);
+  if (lane == 0) fence_mbar_init();
+  __syncthreads();
+  if (tid == 0) {
+    mbar_expect_tx(twb, (uint32_t)P::TW_BYTES);
+    bulk_g2s(sm + P::TW_OFF, a.tw1, (uint32_t)P::TW_BYTES, twb);
+  }
+  int item = blockIdx.x * kImgWarps + warp;
+  Item it{};
+  // the weighted data come from the kernel just before only for the first batch; otherwise the first item's inputs
+  // (bank and data, both unchanged) load while the previous kernel drains
+  if (a.first_batch) pdl_wait();
+  if (item < n_items) {
+    it = item_of(item);
+    if (lane == 0) fetch(it);
+    load_q(it);
+  }
+  if (!a.first_batch) pdl_wait();  // the previous kernel (reader of the scratch we are about to write) has completed
+  bool ok = mbar_wait_bounded(twb, 0, a.status);
+  int k = 0;
+  for (; item < n_items; ++k) {
+    const int s = it.s, k2 = it.k2;
+    // the column's table entries and scale: their latency passes under the first transform
+    const float2* twr = a.tw4 + (int64_t)k2 * (RA + 1);
+    float2 w = ldg_early(twr + lane);
+    const float2 st = ldg_early(twr + RA);
+    const float ratio = ldg_early(it.ratio + it.tmpl);
+    ok = __all_sync(0xffffffffu, ok && mbar_wait_bounded(full, (uint32_t)(k & 1), a.status));
+    if (!ok) break;
+    float2 v[RA];
+    float vx[RA], vy[RA];
+#pragma unroll
+    for (int r = 0; r < RA / 2; ++r) {  // k1 = lane + 32 r < N1/2
+      const float2 x = cmulc(qv[r], smem_h<BT>(tile, lane + r * RB));
+      vx[r] = x.x;
+      vy[r] = x.y;
+    }
+    // the tile is in registers: order its reads before the next copy into it
+    fence_proxy_async();
+    __syncwarp();
+    item += stride;
+    if (item < n_items) {
+      it = item_of(item);
+      if (lane == 0) fetch(it);
+    }
+    dft_pairs<true>(vx, vy, v);
+    if (k > 0) {  // the previous column's store has long read the exchange buffer
+      if (lane == 0) bulk_wait_read();
+      __syncwarp();
+    }
+#pragma unroll
+    for (int q = 0; q < RA; ++q) xb[lane * RA + q + lane] = v[q];
+    __syncwarp();
+    const float sc = series_scale16(ratio);  // (before the loads below: late, it held up the stores)
+    float2 u[RB];
+    float ux[RB], uy[RB];
+    ux[0] = xb[lane].x;
+    uy[0] = xb[lane].y;
+#pragma unroll
+    for (int r = 1; r < RB; ++r) {
+      const float2 z = cmul(xb[lane + r * RA + r], tw[r * RA + lane]);
+      ux[r] = z.x;
+      uy[r] = z.y;
+    }
+    if (item < n_items) load_q(it);
+    dft_pairs<false>(ux, uy, u);
+    // four-step twiddle w_N^{(j + q RA) k2} = w_N^{j k2} (w_N^{RA k2})^q, j = lane; the table row of column k2
+    // holds w_N^{j k2} for j <= RA, so a warp's loads are contiguous
+    w.x *= sc;
+    w.y *= sc;
+    // every value of the exchange buffer is in registers: it becomes the stage, [image][panel][part][row]
+    constexpr int IMAGE = N1 / PH * 2 * PH;  // halves of a column in one image
+    static_assert(IMG * IMAGE * 2 <= P::XCH && P::WARP % 128 == 0 && P::TILE % 128 == 0, "image stage");
+    __syncwarp();
+    __half* stage = reinterpret_cast<__half*>(xb) + (lane / PH) * (2 * PH) + (lane % PH);
+#pragma unroll
+    for (int q = 0; q < RB; ++q) {
+      const float2 z = cmul(u[q], w);
+      const __half2 h = __float22half2_rn(z);
+      __half* dq = stage + q * (RA / PH) * (2 * PH);
+      dq[0] = __low2half(h);
+      dq[PH] = __high2half(h);
+      if constexpr (IM == 2) {  // the remainder: z - hi is exact in FP32
+        const float2 hf = __half22float2(h);
+        const __half2 l = __float22half2_rn(make_float2(z.x - hf.x, z.y - hf.y));
+        dq[IMAGE] = __low2half(l);
+        dq[IMAGE + PH] = __high2half(l);
+      }
+      if (q + 1 < RB) w = cmul(w, st);
+    }
+    fence_proxy_async();  // the stage is written: the store reads it through the async proxy
+    __syncwarp();
+    if (lane == 0) {
+      tma_store_4d(&tm, xb, 0, s * (N1 / PH), (k2 & 31) * 32 + (k2 >> 5), 0);
+      bulk_commit();
+    }
+  }
+  if (!ok && lane == 0) {
+    // a wait gave up: before the CTA exits, wait (bounded again) for the copies that may still be in flight
+    if (tid == 0) mbar_wait_bounded(twb, 0, nullptr);
+    if (item < n_items) mbar_wait_bounded(full, (uint32_t)(k & 1), nullptr);
+  }
+  if (lane == 0) bulk_wait_all();  // the stores are in global memory before this grid counts as complete
+  pdl_launch_dependents();         // our items are done: the next kernel may launch
 }
 
 // ---------------------------------------------------------------------------
@@ -533,11 +721,11 @@ int grid2(int items) {
   return items < g ? items : g;
 }
 
-template <int N1, int N2, int BT, int QT, int IM = 0, bool MP = false>
+template <int N1, int N2, int BT, int QT, bool MP = false>
 cudaError_t run_cols(const FilterArgs& a, const FilterParts& ps, cudaStream_t st) {
   using P = ColGeo<N1, BT, QT>;
   static_assert(P::SMEM * 3 <= 230400, "k_cols: three CTAs per SM must fit in shared memory");
-  auto k = k_cols<N1, N2, BT, QT, IM, MP>;
+  auto k = k_cols<N1, N2, BT, QT, MP>;
   static bool attr = false;
   if (!attr) {
     cudaError_t e = set_smem2(k, P::SMEM);
@@ -550,38 +738,51 @@ cudaError_t run_cols(const FilterArgs& a, const FilterParts& ps, cudaStream_t st
   return e;
 }
 
+template <int BT, int IM, bool MP>
+cudaError_t run_cols16(const FilterArgs& a, const FilterParts& ps, const ScratchMaps& tm, cudaStream_t st) {
+  using P = ImgGeo<BT>;
+  static_assert(P::SMEM <= 232448, "k_cols16: shared memory");
+  auto k = k_cols16<BT, IM, MP>;
+  static bool attr = false;
+  if (!attr) {
+    cudaError_t e = set_smem2(k, P::SMEM);
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  const int ctas = (MP ? ps.n_series : a.count * a.n_det) * (1024 / kImgWarps), g = sm_count();
+  cudaError_t e = launch_pdl(k, ctas < g ? ctas : g, kImgThreads, P::SMEM, st, IM == 2 ? tm.h16x2 : tm.h16, a, ps);
+  add_launches(1);
+  return e;
+}
+
+// FP16 intermediates for the tensor-core row pass: FP32 data, any bank (fused launches: an FP32 bank)
+template <int IM>
+cudaError_t run_cols16_bt(const FilterArgs& a, const FilterParts& ps, const ScratchMaps& tm, cudaStream_t st) {
+  if (a.q_type != kBankF32) return cudaErrorInvalidValue;
+  if (ps.n > 0) return a.bank_type == kBankF32 ? run_cols16<kBankF32, IM, true>(a, ps, tm, st) : cudaErrorInvalidValue;
+  switch (a.bank_type) {
+    case kBankF32: return run_cols16<kBankF32, IM, false>(a, ps, tm, st);
+    case kBankF16: return run_cols16<kBankF16, IM, false>(a, ps, tm, st);
+    case kBankBF16: return run_cols16<kBankBF16, IM, false>(a, ps, tm, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
 // (bank, data) storage pairs: FP32 data with any bank; 16-bit data with a bank of the same type.
 // Fused launches (ps.n > 0): FP32 data, an FP32 bank.
 template <int N1, int N2>
-cudaError_t run_cols_bt(const FilterArgs& a, const FilterParts& ps, cudaStream_t st) {
-  const bool mp = ps.n > 0;
-  if (mp && (a.q_type != kBankF32 || a.bank_type != kBankF32)) return cudaErrorInvalidValue;
-  if constexpr (N1 == 1024 && N2 == 1024) {
-    // FP16 intermediates for the tensor-core row pass: FP32 data, any bank
-    if (a.inter != 0 && a.q_type != kBankF32) return cudaErrorInvalidValue;
-    if (a.inter == 1) {
-      if (mp) return run_cols<N1, N2, kBankF32, kBankF32, 1, true>(a, ps, st);
-      switch (a.bank_type) {
-        case kBankF32: return run_cols<N1, N2, kBankF32, kBankF32, 1>(a, ps, st);
-        case kBankF16: return run_cols<N1, N2, kBankF16, kBankF32, 1>(a, ps, st);
-        case kBankBF16: return run_cols<N1, N2, kBankBF16, kBankF32, 1>(a, ps, st);
-      }
-      return cudaErrorInvalidValue;
+cudaError_t run_cols_bt(const FilterArgs& a, const FilterParts& ps, const ScratchMaps& tm, cudaStream_t st) {
+  if (a.inter != 0) {
+    if constexpr (N1 == 1024 && N2 == 1024) {
+      if (a.inter == 1) return run_cols16_bt<1>(a, ps, tm, st);
+      if (a.inter == 2) return run_cols16_bt<2>(a, ps, tm, st);
     }
-    if (a.inter == 2) {
-      if (mp) return run_cols<N1, N2, kBankF32, kBankF32, 2, true>(a, ps, st);
-      switch (a.bank_type) {
-        case kBankF32: return run_cols<N1, N2, kBankF32, kBankF32, 2>(a, ps, st);
-        case kBankF16: return run_cols<N1, N2, kBankF16, kBankF32, 2>(a, ps, st);
-        case kBankBF16: return run_cols<N1, N2, kBankBF16, kBankF32, 2>(a, ps, st);
-      }
-      return cudaErrorInvalidValue;
-    }
-    if (a.inter != 0) return cudaErrorInvalidValue;
-  } else {
-    if (a.inter != 0) return cudaErrorInvalidValue;
+    return cudaErrorInvalidValue;
   }
-  if (mp) return run_cols<N1, N2, kBankF32, kBankF32, 0, true>(a, ps, st);
+  if (ps.n > 0) {
+    if (a.q_type != kBankF32 || a.bank_type != kBankF32) return cudaErrorInvalidValue;
+    return run_cols<N1, N2, kBankF32, kBankF32, true>(a, ps, st);
+  }
   if (a.q_type == kBankF32) {
     switch (a.bank_type) {
       case kBankF32: return run_cols<N1, N2, kBankF32, kBankF32>(a, ps, st);
@@ -640,18 +841,39 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
+// The FP16 operand image of the scratch (FilterArgs::inter = images) by columns: position pos = 32 (k2 % 32) +
+// k2 / 32 of a panel holds the 2 x 8 halves of column k2; (half, panel, pos, image), a box is one column of a series.
+cudaError_t encode_image(const float2* scratch, int64_t series, int n1, int n2, int images, CUtensorMap* m) {
+  auto fn = encode_fn();
+  if (!fn || !scratch || series < 1) return cudaErrorInvalidValue;
+  const cuuint64_t run = 2 * kPanel16, image = run * (cuuint64_t)n2 * 2;  // halves of a column in a panel; bytes
+  cuuint64_t dims[4] = {run, (cuuint64_t)(series * (n1 / kPanel16)), (cuuint64_t)n2, (cuuint64_t)images};
+  cuuint64_t strides[3] = {image * images, run * 2, image};
+  cuuint32_t box[4] = {(cuuint32_t)run, (cuuint32_t)(n1 / kPanel16), 1u, (cuuint32_t)images};
+  cuuint32_t es[4] = {1u, 1u, 1u, 1u};
+  CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT16, 4, const_cast<float2*>(scratch), dims, strides, box, es,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 template <int N1, int N2>
-cudaError_t encode_scratch_of(const float2* scratch, int64_t series, CUtensorMap* m) {
+cudaError_t encode_scratch_of(const float2* scratch, int64_t series, ScratchMaps* m) {
   using SG = ScratchGeo<N1, N2>;
-  *m = CUtensorMap{};
-  if (SG::RW == SG::P) return cudaSuccess;  // contiguous items: no tensor map
+  *m = ScratchMaps{};
+  if constexpr (N1 == 1024 && N2 == 1024) {
+    cudaError_t e = encode_image(scratch, series, N1, N2, 1, &m->h16);
+    if (e == cudaSuccess) e = encode_image(scratch, series, N1, N2, 2, &m->h16x2);
+    if (e != cudaSuccess) return e;
+  }
+  if (SG::RW == SG::P) return cudaSuccess;  // contiguous row-pass items: no tensor map
   auto fn = encode_fn();
   if (!fn || !scratch || series < 1) return cudaErrorInvalidValue;
   cuuint64_t dims[3] = {(cuuint64_t)SG::P, (cuuint64_t)N2, (cuuint64_t)(series * (N1 / SG::P))};
   cuuint64_t strides[2] = {(cuuint64_t)SG::P * 8, (cuuint64_t)N2 * SG::P * 8};
   cuuint32_t box[3] = {(cuuint32_t)SG::RW, (cuuint32_t)SG::BOXY, 1u};
   cuuint32_t es[3] = {1u, 1u, 1u};
-  CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, const_cast<float2*>(scratch), dims, strides, box, es,
+  CUresult r = fn(&m->rows, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, const_cast<float2*>(scratch), dims, strides, box, es,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
@@ -707,33 +929,35 @@ namespace {
 
 const FilterParts kOnePlan{};  // n = 0: every per-series field from FilterArgs
 
-cudaError_t pass1_parts(const FilterArgs& a, const FilterParts& ps, cudaStream_t st) {
-  MF_DISPATCH2(a.n, run_cols_bt, (a, ps, st))
+cudaError_t pass1_parts(const FilterArgs& a, const FilterParts& ps, const ScratchMaps& tm, cudaStream_t st) {
+  MF_DISPATCH2(a.n, run_cols_bt, (a, ps, tm, st))
 }
 
-cudaError_t pass2_parts(const FilterArgs& a, const FilterParts& ps, const CUtensorMap& tm, cudaStream_t st) {
+cudaError_t pass2_parts(const FilterArgs& a, const FilterParts& ps, const ScratchMaps& tm, cudaStream_t st) {
   if (a.inter != 0) return launch_filter2_pass2_tc(a, st, ps.n > 0 ? &ps : nullptr);
-  MF_DISPATCH2(a.n, run_rows, (a, ps, tm, st))
+  MF_DISPATCH2(a.n, run_rows, (a, ps, tm.rows, st))
 }
 
 }  // namespace
 
-cudaError_t launch_filter2_pass1(const FilterArgs& a, cudaStream_t st) { return pass1_parts(a, kOnePlan, st); }
+cudaError_t launch_filter2_pass1(const FilterArgs& a, const ScratchMaps& tm, cudaStream_t st) {
+  return pass1_parts(a, kOnePlan, tm, st);
+}
 
-cudaError_t launch_filter2_pass2(const FilterArgs& a, const CUtensorMap& tm, cudaStream_t st) {
+cudaError_t launch_filter2_pass2(const FilterArgs& a, const ScratchMaps& tm, cudaStream_t st) {
   return pass2_parts(a, kOnePlan, tm, st);
 }
 
-cudaError_t launch_filter2_fused(const FilterArgs& a, const FilterParts& ps, const CUtensorMap& tm, cudaStream_t st,
+cudaError_t launch_filter2_fused(const FilterArgs& a, const FilterParts& ps, const ScratchMaps& tm, cudaStream_t st,
                                  cudaEvent_t between) {
   if (ps.n < 1 || ps.n > kMaxParts || ps.n_series < 1) return cudaErrorInvalidValue;
-  cudaError_t e = pass1_parts(a, ps, st);
+  cudaError_t e = pass1_parts(a, ps, tm, st);
   if (e == cudaSuccess && between) e = cudaEventRecord(between, st);
   if (e == cudaSuccess) e = pass2_parts(a, ps, tm, st);
   return e;
 }
 
-cudaError_t encode_scratch_map(int64_t n, const float2* scratch, int64_t series, CUtensorMap* m) {
+cudaError_t encode_scratch_maps(int64_t n, const float2* scratch, int64_t series, ScratchMaps* m) {
   MF_DISPATCH2(n, encode_scratch_of, (scratch, series, m))
 }
 

@@ -91,6 +91,12 @@ struct FilterPart {
   const int2* row_valid;
   int series0;
 };
+// Tensor maps of the pass-1 -> pass-2 scratch: rows, through which the FP32 row pass reads its items; h16 and
+// h16x2, through which the column pass writes its columns of the FP16 and the FP16-pair intermediate (N = 2^20).
+struct ScratchMaps {
+  CUtensorMap rows, h16, h16x2;
+};
+
 constexpr int kMaxParts = 8;
 struct FilterParts {
   int n;         // parts of this launch, 1..kMaxParts (0: one plan, all of FilterArgs)
@@ -125,27 +131,26 @@ int plan_batch(const ::mf_plan_s* p);
 // two passes take the series of all plans in (plan, template, row) order, one launch pair per
 // scratch_series series across plan boundaries.  The plans share N, the window and the
 // intermediate, with an FP32 bank and FP32 data; `scratch` holds scratch_series series of the
-// intermediate (N x 8 bytes each; scratch_map encoded for it) and every step runs on st.  A wait
+// intermediate (N x 8 bytes each; maps encoded for it) and every step runs on st.  A wait
 // that times out is reported by plans[0], and so are the launch counts and, when plans[0] is
 // profiling (mf_profile), the launch pairs' CUDA-event times.  On failure *err holds the message.
 int filter_fused(::mf_plan_s* const* plans, const void* const* dtilde, const int64_t* ld, int n_plans, void* scratch,
-                 int64_t scratch_series, const CUtensorMap& scratch_map, cudaStream_t st, std::string* err);
+                 int64_t scratch_series, const ScratchMaps& maps, cudaStream_t st, std::string* err);
 // The TMA-staged filter passes (mf_filter.cu).  The bank rows and the
 // weighted data are in column layout: element k = k1 N2 + k2 of the non-zero
 // half (k1 < N1/2) at k2 N1/2 + k1 (BankRows).
-cudaError_t launch_filter2_pass1(const FilterArgs& a, cudaStream_t st);
-cudaError_t launch_filter2_pass2(const FilterArgs& a, const CUtensorMap& scratch_map, cudaStream_t st);
+cudaError_t launch_filter2_pass1(const FilterArgs& a, const ScratchMaps& maps, cudaStream_t st);
+cudaError_t launch_filter2_pass2(const FilterArgs& a, const ScratchMaps& maps, cudaStream_t st);
 // the tensor-core row pass over the FP16 intermediate (mf_filter_tc.cu), N = 2^20
 cudaError_t launch_filter2_pass2_tc(const FilterArgs& a, cudaStream_t st, const FilterParts* parts = nullptr);
 // Both passes over the series of several plans' parts in one launch each (ps.n >= 1): the
 // per-part fields come from ps, the rest (geometry, types, window, scratch, tables, status)
-// from a; the scratch holds ps.n_series series (scratch_map encoded for at least as many).  `between`
+// from a; the scratch holds ps.n_series series (maps encoded for at least as many).  `between`
 // (optional) is recorded on st between the two launches.
-cudaError_t launch_filter2_fused(const FilterArgs& a, const FilterParts& ps, const CUtensorMap& scratch_map,
+cudaError_t launch_filter2_fused(const FilterArgs& a, const FilterParts& ps, const ScratchMaps& maps,
                                  cudaStream_t st, cudaEvent_t between = nullptr);
-// Tensor map of the pass-1 -> pass-2 scratch (`series` series of length n)
-// through which pass 2 reads its items; all zero where pass 2 needs none.
-cudaError_t encode_scratch_map(int64_t n, const float2* scratch, int64_t series, CUtensorMap* m);
+// Tensor maps of the pass-1 -> pass-2 scratch (`series` series of length n); all zero where a pass needs none.
+cudaError_t encode_scratch_maps(int64_t n, const float2* scratch, int64_t series, ScratchMaps* m);
 cudaError_t launch_fill_twiddles(int64_t n, float2* tw1, float2* tw2, cudaStream_t st);
 // four-step twiddles of k_cols by column: tw4[k2 (RA + 1) + j] = w_N^{j k2}, j <= RA(N1), k2 < N2;
 // tw4_count(n) entries
