@@ -702,6 +702,7 @@ mf_status mf_filter(mf_plan_t p, const void* dtilde, int64_t ld_dtilde, const in
   const double thr = p->d.snr_thr;
   a.thr2 = (float)(thr * thr);
   a.window = p->d.window;
+  a.win_recip = mf::window_recip(p->d.window);
   a.valid_begin = p->d.valid_begin;
   a.valid_end = p->d.valid_end;
   a.n_win = p->n_win;
@@ -1190,6 +1191,7 @@ int filter_fused(mf_plan_s* const* plans, const void* const* dtilde, const int64
   a.bank_type = kBankF32;
   a.scratch = static_cast<float2*>(scratch);
   a.window = p0->d.window;
+  a.win_recip = mf::window_recip(p0->d.window);
   a.n_win = p0->n_win;
   a.status = p0->status;
   a.tw1 = p0->tw;

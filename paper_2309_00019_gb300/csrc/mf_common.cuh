@@ -61,14 +61,15 @@ __device__ __forceinline__ float series_scale16(float ratio) {
 // atomic maximum into its window slot.  Out of line: it runs for a small
 // fraction of samples and keeping it out of the unrolled hot loop keeps that
 // loop's code small.
-static __device__ __noinline__ void record_peak(unsigned long long* slot_row, int64_t n, int64_t window, float a, float b,
-                                        float r2) {
+// win_recip = window_recip(window): a 64-bit division took most of its instructions.
+static __device__ __noinline__ void record_peak(unsigned long long* slot_row, int64_t n, uint64_t win_recip, float a,
+                                                float b, float r2) {
   const float ph = atan2f(b, a);
   const uint32_t code = (uint32_t)__float2int_rn(fmaf(ph, 0.15915494309189535f, 0.5f) * 2048.0f) & 2047u;
   const unsigned long long key = ((unsigned long long)__float_as_uint(r2) << 32) |
                                  ((unsigned long long)(((1u << kSampleBits) - 1u) - (uint32_t)n) << kPhaseBits) |
                                  code;
-  atomicMax(slot_row + n / window, key);
+  atomicMax(slot_row + (((uint64_t)n * win_recip) >> kRecipBits), key);
 }
 
 struct FilterEpi {
@@ -77,7 +78,8 @@ struct FilterEpi {
   int64_t pos0;
   int n_det;
   float thr2;
-  int64_t window, vb, ve, n_win, n_sel_total;
+  uint64_t win_recip;
+  int64_t vb, ve, n_win, n_sel_total;
   unsigned long long* slots;
   struct Ser {
     float is;
@@ -92,7 +94,7 @@ struct FilterEpi {
     const float a = z.x * se.is, b = z.y * se.is;
     const float r2 = fmaf(a, a, b * b);
     if (r2 >= thr2) {
-      if (n >= vb && n < ve) record_peak(se.slot, n, window, a, b, r2);
+      if (n >= vb && n < ve) record_peak(se.slot, n, win_recip, a, b, r2);
     }
   }
 };
@@ -108,7 +110,8 @@ struct RawEpi {
   const float* dscale;  // per detector: power-of-two scale of 16-bit data (z' carries it), or null
   int64_t pos0;
   int n_det;
-  int64_t window, vb, ve, n_win, n_sel_total;
+  uint64_t win_recip;
+  int64_t vb, ve, n_win, n_sel_total;
   unsigned long long* slots;
   const int2* row_valid;  // per data row [begin, end), or null: [vb, ve) for every row
   struct Ser {
@@ -139,7 +142,7 @@ struct RawEpi {
     if (m2 >= se.thr) {
       if (n >= se.vb && n < se.ve) {
         const float a = z.x * se.ratio, b = z.y * se.ratio;
-        record_peak(se.slot, n, window, a, b, fmaf(a, a, b * b));
+        record_peak(se.slot, n, win_recip, a, b, fmaf(a, a, b * b));
       }
     }
   }

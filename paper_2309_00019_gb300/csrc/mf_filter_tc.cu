@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_rows_tc(FilterArgs a, const _
     const float2* twq = tw + q * kTwStride;
     for (int k = g; k < n_mine; k += kGroups) {
       // the epilogue's fields are kernel parameters, read where used (no registers held across the loop)
-      const RawEpi ep{a.sel, a.inv_sigma, a.thr_raw, nullptr, a.pos0, a.n_det, a.window, a.valid_begin,
+      const RawEpi ep{a.sel, a.inv_sigma, a.thr_raw, nullptr, a.pos0, a.n_det, a.win_recip, a.valid_begin,
                       a.valid_end, a.n_win, a.n_sel_total, a.slots, a.row_valid};
       const int slot = k % kSlots, b = k % kBufs;
       unsigned char* sl = sm + slot * kItemBytes;
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_rows_tc(FilterArgs a, const _
       float sc;
       if constexpr (MP) {
         const FilterPart& p = ps.p[part_of(ps, s, 1)];
-        const RawEpi pe{p.sel,         p.inv_sigma, p.thr_raw, nullptr,       p.pos0,  p.n_det,    a.window,
+        const RawEpi pe{p.sel,         p.inv_sigma, p.thr_raw, nullptr,       p.pos0,  p.n_det,    a.win_recip,
                         p.valid_begin, p.valid_end, a.n_win,   p.n_sel_total, p.slots, p.row_valid};
         se = pe.series(s - p.series0);
         sc = series_scale16(__ldg(p.inv_sigma + p.sel[p.pos0 + (s - p.series0) / p.n_det]));

@@ -19,6 +19,13 @@ constexpr int kSampleBits = 21;
 constexpr int kPhaseBits = 11;
 constexpr int64_t kMaxN = int64_t(1) << 20;
 
+// n / window for 0 <= n < kMaxN, 1 <= window <= kMaxN as (n window_recip(window)) >> kRecipBits: the reciprocal is
+// high by less than 2^-kRecipBits, so the quotient by less than 2^-20 <= 1 / window, too little to reach the next.
+constexpr int kRecipBits = 40;
+constexpr uint64_t window_recip(int64_t window) {
+  return ((uint64_t(1) << kRecipBits) + (uint64_t)window - 1) / (uint64_t)window;
+}
+
 enum BankType { kBankF32 = 0, kBankF16 = 1, kBankBF16 = 2 };
 
 struct FilterArgs {
@@ -43,6 +50,7 @@ struct FilterArgs {
   // epilogue
   float thr2;
   int64_t window;
+  uint64_t win_recip;       // window_recip(window)
   int64_t valid_begin, valid_end;
   int64_t n_win;
   int64_t n_sel_total;      // slots are [n_det][n_sel_total][n_win]

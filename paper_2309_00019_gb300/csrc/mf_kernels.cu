@@ -272,7 +272,7 @@ cudaError_t run_pass1(const FilterArgs& a, cudaStream_t st) {
 template <int N1, int N2>
 cudaError_t run_pass2(const FilterArgs& a, cudaStream_t st) {
   const int n_series = a.count * a.n_det;
-  FilterEpi ep{a.sel, a.inv_sigma, a.pos0, a.n_det, a.thr2, a.window, a.valid_begin, a.valid_end,
+  FilterEpi ep{a.sel, a.inv_sigma, a.pos0, a.n_det, a.thr2, a.win_recip, a.valid_begin, a.valid_end,
                a.n_win, a.n_sel_total, a.slots};
   auto k2 = k_pass2<N1, N2, FilterEpi>;
   cudaError_t e = set_smem(k2, P2Geo<N2>::SMEM);

@@ -132,6 +132,7 @@ extern "C" mf_status mf_filter_noalloc(double fs, int64_t n, int32_t n_det, doub
   a.scratch = fft_scratch;
   a.thr2 = (float)(snr_thr * snr_thr);
   a.window = window;
+  a.win_recip = mf::window_recip(window);
   a.valid_begin = 0;
   a.valid_end = n;
   a.n_win = n_win;
