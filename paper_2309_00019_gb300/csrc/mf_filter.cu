@@ -25,6 +25,8 @@
 // when a CTA has finished all its items, so the next kernel's CTAs (which wait
 // for this one to complete before touching the scratch) take the slots of
 // retiring CTAs instead of competing with this kernel's own CTAs for them.
+#include <algorithm>
+
 #include "mf_common.cuh"
 #include "mf_tma.cuh"
 
@@ -727,9 +729,14 @@ cudaError_t launch_pdl(K kern, int grid, int block, int smem, cudaStream_t st, A
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-int grid2(int items) {
-  const int g = sm_count() * 3;
-  return items < g ? items : g;
+// CTAs of a persistent launch: as many as fit the chip at once.  Three per SM at N1, N2 >= 512 (their shared memory);
+// shorter transforms need less of it, and up to seven hide each other's waits.
+template <class K>
+int resident_ctas(K kern, int threads, int smem) {
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, (size_t)smem) != cudaSuccess || per_sm < 3)
+    per_sm = 3;
+  return sm_count() * per_sm;
 }
 
 template <int N1, int N2, int BT, int QT, bool MP = false>
@@ -737,14 +744,14 @@ cudaError_t run_cols(const FilterArgs& a, const FilterParts& ps, cudaStream_t st
   using P = ColGeo<N1, BT, QT>;
   static_assert(P::SMEM * 3 <= 230400, "k_cols: three CTAs per SM must fit in shared memory");
   auto k = k_cols<N1, N2, BT, QT, MP>;
-  static bool attr = false;
-  if (!attr) {
+  static int resident = 0;
+  if (resident == 0) {
     cudaError_t e = set_smem2(k, P::SMEM);
     if (e != cudaSuccess) return e;
-    attr = true;
+    resident = resident_ctas(k, kColThreads, P::SMEM);
   }
   const int items = (MP ? ps.n_series : a.count * a.n_det) * (N2 / P::C);
-  cudaError_t e = launch_pdl(k, grid2(items), kColThreads, P::SMEM, st, a, ps);
+  cudaError_t e = launch_pdl(k, std::min(items, resident), kColThreads, P::SMEM, st, a, ps);
   add_launches(1);
   return e;
 }
@@ -814,14 +821,14 @@ cudaError_t run_rows_mp(const FilterArgs& a, const FilterParts& ps, const CUtens
   using P = RowGeo<N2>;
   static_assert(P::SMEM * 3 <= 230400, "k_rows: three CTAs per SM must fit in shared memory");
   auto k = k_rows<N1, N2, MP>;
-  static bool attr = false;
-  if (!attr) {
+  static int resident = 0;
+  if (resident == 0) {
     cudaError_t e = set_smem2(k, P::SMEM);
     if (e != cudaSuccess) return e;
-    attr = true;
+    resident = resident_ctas(k, kT2, P::SMEM);
   }
   const int items = (MP ? ps.n_series : a.count * a.n_det) * (N1 / P::RW);
-  cudaError_t e = launch_pdl(k, grid2(items), kT2, P::SMEM, st, tm, a, ps);
+  cudaError_t e = launch_pdl(k, std::min(items, resident), kT2, P::SMEM, st, tm, a, ps);
   add_launches(1);
   return e;
 }
