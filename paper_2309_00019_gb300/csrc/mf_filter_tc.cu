@@ -48,7 +48,7 @@ constexpr int kTcK = 64;                          // 32 complex values, real and
 constexpr int kLbo = 128, kSbo = 1024;            // unpadded core-matrix layouts
 constexpr int kTileBytes = 128 * kTcK * 2;        // one M = 128 operand tile, 16 KB
 constexpr int kBBytes = 64 * kTcK * 2;            // one image of the DFT matrix B (64 x 64), 8 KB
-constexpr int kTwStride = 33;                     // padded rows of the w1024^{q u} table (float2)
+constexpr int kTwStride = 34;                     // padded rows of the w1024^{q u} table (float2, read in pairs)
 constexpr uint32_t kBufCols = 128;                // 2 tiles x 64 FP32 columns
 constexpr uint32_t kTmemCols = kBufs * kBufCols;  // all 512
 constexpr uint32_t kIdesc2 = tc_idesc_f16(128, 64);          // A K-major (stage 2)
@@ -271,7 +271,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_rows_tc(FilterArgs a, const _
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const int u = 8 * t + i;
-          const float2 z = cmul(make_float2(cur[2 * i], cur[2 * i + 1]), twq[u]);
+          const float4 f2 = *reinterpret_cast<const float4*>(twq + (u & ~1));
+          const float2 f = (u & 1) ? make_float2(f2.z, f2.w) : make_float2(f2.x, f2.y);
+          const float2 z = cmul(make_float2(cur[2 * i], cur[2 * i + 1]), f);
           const int off = cm_offset(u * 8 + r, 2 * q, kLbo, kSbo);
           const __half2 hi = __floats2half2_rn(z.x, z.y);
           *reinterpret_cast<__half2*>(sl + off) = hi;
@@ -298,10 +300,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_rows_tc(FilterArgs a, const _
         float(&cur)[16] = (t & 1) ? zb : za;
         float(&nxt)[16] = (t & 1) ? za : zb;
         if (t + 1 < 4) tmem_ld16_issue(tbuf + 16 * (t + 1), nxt);
-        float mx = 0.f;
+        float m[8];  // the largest |z|^2 of the eight samples, as a tree: a running maximum is a chain of eight waits
 #pragma unroll
-        for (int i = 0; i < 8; ++i) mx = fmaxf(mx, fmaf(cur[2 * i], cur[2 * i], cur[2 * i + 1] * cur[2 * i + 1]));
-        if (mx >= se.thr) {  // rare: some sample of this row is over the threshold
+        for (int i = 0; i < 8; ++i) m[i] = fmaf(cur[2 * i], cur[2 * i], cur[2 * i + 1] * cur[2 * i + 1]);
+        if (fmaxf(fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])), fmaxf(fmaxf(m[4], m[5]), fmaxf(m[6], m[7]))) >= se.thr) {  // rare: some sample of this row is over the threshold
 #pragma unroll
           for (int i = 0; i < 8; ++i)
             ep(se, j1 + (int64_t)N1 * (q + 32 * (8 * t + i)), make_float2(cur[2 * i], cur[2 * i + 1]));
