@@ -669,14 +669,14 @@ mf_status mf_filter(mf_plan_t p, const void* dtilde, int64_t ld_dtilde, const in
   if (s != MF_OK) return s;
   if ((s = refresh_scale(p)) != MF_OK) return s;
   cudaError_t e = cudaSuccess;
-  if (n_sel > 0)
-    e = cudaMemcpyAsync(p->sel_copy, n_subset < 0 ? p->sel_all : subset, n_sel * sizeof(int32_t), cudaMemcpyDeviceToDevice,
-                        p->st);
+  if (n_subset > 0)
+    e = cudaMemcpyAsync(p->sel_copy, subset, n_sel * sizeof(int32_t), cudaMemcpyDeviceToDevice, p->st);
   if (e != cudaSuccess) return cuda_fail(p, e, "mf_filter selection copy");
   const int64_t n_slots = (int64_t)p->d.n_det * n_sel * p->n_win;
   const int64_t launches_before = mf::launch_count();
   e = mf::launch_prep_cols((const float2*)dtilde, ld_dtilde, p->w_dev, p->n1, p->n2, p->d.n_det, p->q, p->ld_q,
-                           p->slots, n_slots, p->st, 1.0 / p->sigma_ref);
+                           p->slots, n_slots, p->sel_all, p->sel_copy, n_subset < 0 ? n_sel : 0, p->st,
+                           1.0 / p->sigma_ref);
   if (e != cudaSuccess) return cuda_fail(p, e, "mf_filter prep");
   if (p->data_dtype != MF_F32) {
     e = mf::launch_quant_q(p->q, p->ld_q, p->d.n / 2, p->d.n_det, bank_type(p->data_dtype), p->q_lp, p->dmax, p->dscale,
@@ -736,7 +736,7 @@ mf_status mf_filter(mf_plan_t p, const void* dtilde, int64_t ld_dtilde, const in
       p->samples.push_back({e0, (int64_t)a.count * p->d.n_det});
     }
   }
-  e = mf::launch_compact(p->slots, p->d.n_det, n_sel, p->n_win, p->d.window, p->sel_copy, p->trig, p->d.max_triggers,
+  e = mf::launch_compact(p->slots, p->d.n_det, n_sel, p->n_win, p->sel_copy, p->trig, p->d.max_triggers,
                          p->count, p->bc, p->bc_cap, p->st);
   if (e != cudaSuccess) return cuda_fail(p, e, "mf_filter compaction");
   p->n_sel = n_sel;
@@ -1176,10 +1176,9 @@ int filter_fused(mf_plan_s* const* plans, const void* const* dtilde, const int64
       if ((s = refresh_scale(p)) != MF_OK) return from_plan(p, s);
       if ((e = cudaStreamSynchronize(p->st)) != cudaSuccess) return bad(MF_ECUDA, "fused filter: template scales");
     }
-    e = cudaMemcpyAsync(p->sel_copy, p->sel_all, p->n_tmpl * sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
-    if (e == cudaSuccess)
-      e = launch_prep_cols(static_cast<const float2*>(dtilde[i]), ld[i], p->w_dev, p->n1, p->n2, p->d.n_det, p->q,
-                           p->ld_q, p->slots, (int64_t)p->d.n_det * p->n_tmpl * p->n_win, st, 1.0 / p->sigma_ref);
+    e = launch_prep_cols(static_cast<const float2*>(dtilde[i]), ld[i], p->w_dev, p->n1, p->n2, p->d.n_det, p->q,
+                         p->ld_q, p->slots, (int64_t)p->d.n_det * p->n_tmpl * p->n_win, p->sel_all, p->sel_copy,
+                         p->n_tmpl, st, 1.0 / p->sigma_ref);
     if (e != cudaSuccess) return bad(MF_ECUDA, std::string("fused filter prep: ") + cudaGetErrorString(e));
   }
   FilterArgs a{};
@@ -1251,7 +1250,7 @@ int filter_fused(mf_plan_s* const* plans, const void* const* dtilde, const int64
   }
   for (int j = 0; j < n_plans; ++j) {
     mf_plan_s* p = plans[j];
-    e = launch_compact(p->slots, p->d.n_det, p->n_tmpl, p->n_win, p->d.window, p->sel_copy, p->trig,
+    e = launch_compact(p->slots, p->d.n_det, p->n_tmpl, p->n_win, p->sel_copy, p->trig,
                        p->d.max_triggers, p->count, p->bc, p->bc_cap, st);
     if (e != cudaSuccess) return bad(MF_ECUDA, std::string("fused filter compaction: ") + cudaGetErrorString(e));
     p->n_sel = p->sel_tmpl = p->n_tmpl;

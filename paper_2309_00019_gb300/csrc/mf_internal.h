@@ -190,9 +190,11 @@ cudaError_t launch_put_rows(const BankRows& b, const void* src, int64_t ld_src, 
 cudaError_t launch_norm_parts(const BankRows& b, int64_t n_rows, cudaStream_t st);
 // sigma^2 and 1 / sigma of n_rows rows from their partial sums
 cudaError_t launch_norms(const BankRows& b, int64_t n_rows, cudaStream_t st);
-// q = q_scale w s~ in column layout (q [n_det][ld_q], N/2 elements per row)
+// What a filter call sets up: q = q_scale w s~ in column layout (q [n_det][ld_q], N/2 elements per row), n_slots window
+// slots cleared, n_sel template ids copied
 cudaError_t launch_prep_cols(const float2* dtilde, int64_t ld_d, const double* w, int n1, int n2, int n_det,
-                             float2* q, int64_t ld_q, unsigned long long* slots, int64_t n_slots, cudaStream_t st,
+                             float2* q, int64_t ld_q, unsigned long long* slots, int64_t n_slots,
+                             const int32_t* sel_from, int32_t* sel_to, int64_t n_sel, cudaStream_t st,
                              double q_scale);
 
 // chi^2 veto at trigger times (mf_chisq.cu): band edges of every template for
@@ -259,7 +261,7 @@ cudaError_t launch_sigmasq(const float2* rows, int64_t ld, int64_t n_rows, const
                            double* sigmasq, float* inv_sigma, cudaStream_t st);
 // compaction of window maxima into mf_trigger records (layout of the public struct)
 cudaError_t launch_compact(const unsigned long long* slots, int n_det, int64_t n_sel, int64_t n_win,
-                           int64_t window, const int32_t* sel, void* trig_out, int64_t trig_cap,
+                           const int32_t* sel, void* trig_out, int64_t trig_cap,
                            int64_t* count, int64_t* block_counts, int64_t n_blocks_cap, cudaStream_t st);
 int64_t compact_blocks(int64_t n_slots);
 // time series -> one-sided dt-normalised spectrum (A1)

@@ -145,7 +145,7 @@ extern "C" mf_status mf_filter_noalloc(double fs, int64_t n, int32_t n_det, doub
     e = mf::launch_filter_batch(a, st);
   }
   if (e == cudaSuccess)
-    e = mf::launch_compact(slots, n_det, n_tmpl, n_win, window, sel, trig, trig_cap, count, bc, n_blk, st);
+    e = mf::launch_compact(slots, n_det, n_tmpl, n_win, sel, trig, trig_cap, count, bc, n_blk, st);
   if (e != cudaSuccess) return fail(MF_ECUDA, std::string("mf_filter_noalloc: ") + cudaGetErrorString(e));
   return MF_OK;
 }
