@@ -568,7 +568,7 @@ __global__ void k_wait_selftest(int* status, int* returned) {
 // A CTA of the first grid.x - extra columns of blocks takes a 32 x 32 tile of (k1, k2) for kPrepRows data rows,
 // coalesced on both sides through shared memory, and forms q_scale w once for all of them; the FP64 operations (2 per
 // clock and SM) bound it.  A thread per element gathered the spectrum and the weights n2 bins apart and multiplied
-// three times: 190 us for the 20 rows of an uneven batch's four classes, 17 us for two detectors (N = 2^20).
+// three times: 190 us for the rows of an uneven batch, 17 us for two detectors (N = 2^20).
 constexpr int kPrepRows = 4;  // data rows per CTA
 
 struct PrepRest {
