@@ -50,38 +50,78 @@ __global__ void __launch_bounds__(kWT) k_welch_mean(const float2* __restrict__ f
   }
 }
 
-// the r-th smallest (from 0) of count keys in shared memory, by a warp: quickselect over the range [lo, hi] that
-// still holds it, the pivot a key of the range
-__device__ __forceinline__ unsigned long long select_key(const unsigned long long* v, int count, int r) {
-  const int lane = threadIdx.x & 31;
-  unsigned long long lo = 0, hi = ~0ull;
+// The r-th smallest (from 0) of count >= r + 1 keys, 32 K >= count, by a warp: lane i holds keys i, i + 32, ... (absent
+// ones all ones, which are above every key).  Quickselect over the range [lo, hi] that still holds it, the pivot a key
+// of the range from another lane each time; *less = the number of keys below the result.
+template <int K>
+__device__ __forceinline__ unsigned long long select_key(const unsigned long long (&v)[K], int r, int* less) {
+  unsigned long long lo = 0, hi = ~0ull - 1;
   for (int step = 0;; ++step) {
     unsigned long long mine = 0;
     bool have = false;
-    for (int i = lane; i < count && !have; i += 32) {
-      mine = v[i];
-      have = mine >= lo && mine <= hi;
-    }
+#pragma unroll
+    for (int i = 0; i < K; ++i)
+      if (v[i] >= lo && v[i] <= hi) {
+        mine = v[i];
+        have = true;
+      }
     const unsigned m = __ballot_sync(0xffffffffu, have);
-    const unsigned rot = __funnelshift_r(m, m, (step * 11 + 16) & 31);  // another lane's first candidate each time
-    const unsigned long long pivot = __shfl_sync(0xffffffffu, mine, ((__ffs(rot) - 1) + ((step * 11 + 16) & 31)) & 31);
-    int less = 0, equal = 0;
-    for (int i = lane; i < count; i += 32) {
-      less += v[i] < pivot ? 1 : 0;
+    if (!m) {  // (not reached by numbers: the range always holds the key)
+      *less = 0;
+      return ~0ull;
+    }
+    const int turn = (step * 11 + 16) & 31;
+    const unsigned long long pivot =
+        __shfl_sync(0xffffffffu, mine, ((__ffs(__funnelshift_r(m, m, turn)) - 1) + turn) & 31);
+    int below = 0, equal = 0;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      below += v[i] < pivot ? 1 : 0;
       equal += v[i] == pivot ? 1 : 0;
     }
-    less = __reduce_add_sync(0xffffffffu, less);
+    below = __reduce_add_sync(0xffffffffu, below);
     equal = __reduce_add_sync(0xffffffffu, equal);
-    if (r < less) hi = pivot - 1;
-    else if (r < less + equal) return pivot;
-    else lo = pivot + 1;
+    if (r < below) {
+      hi = pivot - 1;
+    } else if (r < below + equal) {
+      *less = below;
+      return pivot;
+    } else {
+      lo = pivot + 1;
+    }
   }
 }
 
+// the median of n values >= 0 given by their bits in shared memory
+template <int K>
+__device__ __forceinline__ double median_of(const unsigned long long* s, int n) {
+  const int lane = threadIdx.x & 31;
+  unsigned long long v[K];
+#pragma unroll
+  for (int i = 0; i < K; ++i) v[i] = lane + 32 * i < n ? s[lane + 32 * i] : ~0ull;
+  int less;
+  const unsigned long long upper = select_key<K>(v, n / 2, &less);
+  if (n & 1) return __longlong_as_double((long long)upper);
+  unsigned long long lower = upper;  // the one before it: the largest key below it, or another equal to it
+  if (less == n / 2) {
+    lower = 0;
+#pragma unroll
+    for (int i = 0; i < K; ++i) lower = v[i] < upper && v[i] > lower ? v[i] : lower;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long y = __shfl_xor_sync(0xffffffffu, lower, o);
+      lower = y > lower ? y : lower;
+    }
+  }
+  return 0.5 * (__longlong_as_double((long long)lower) + __longlong_as_double((long long)upper));
+}
+
 // median: a CTA takes `bins` bins (a power of two that fits shared memory) with all their values, then a warp per
-// bin selects the middle ones.  The values are >= 0, so their bits are in their order: the comparisons are integer
-// ones, not FP64 ones, of which the chip does 2 per clock and SM.  A CTA per bin that read one 8-byte value per
-// row and sorted them took 223 us for 127 segments of two detectors and 8,193 bins; now 59 us.
+// bin takes them into registers (K per lane, 32 K >= n_seg) and selects the middle ones.  The values are >= 0, so
+// their bits are in their order: the comparisons are integer ones, not FP64 ones, of which the chip does 2 per clock
+// and SM.  For 127 segments of two detectors and 8,193 bins: a CTA per bin that read one 8-byte value per row and
+// sorted them 223 us, keys read from shared memory for each comparison 59 us, now 44 us.
+template <int K>
 __global__ void __launch_bounds__(kWT) k_welch_median(const float2* __restrict__ fd, int64_t ld_fd, int n_det,
                                                       int n_seg, int64_t n, Norm nm, double median_bias, int bins,
                                                       double* __restrict__ psd) {
@@ -97,8 +137,7 @@ __global__ void __launch_bounds__(kWT) k_welch_median(const float2* __restrict__
   __syncthreads();
   for (int c = threadIdx.x >> 5; c < bins && k0 + c <= n / 2; c += kWT / 32) {
     const unsigned long long* v = keys + c * pitch;
-    const double hi = __longlong_as_double((long long)select_key(v, n_seg, n_seg / 2));
-    const double med = (n_seg & 1) ? hi : 0.5 * (__longlong_as_double((long long)select_key(v, n_seg, n_seg / 2 - 1)) + hi);
+    const double med = median_of<K>(v, n_seg);
     if ((threadIdx.x & 31) == 0) psd[(int64_t)d * (n / 2 + 1) + k0 + c] = med / median_bias;
   }
 }
@@ -144,9 +183,9 @@ extern "C" mf_status mf_psd_welch(double fs, int32_t n_det, int64_t n_samples, c
     } else {
       int bins = 32;
       while (bins > 1 && bins * (n_seg | 1) * 8 > mf::kMedianBytes) bins /= 2;
-      mf::k_welch_median<<<dim3((unsigned)((nb + bins - 1) / bins), (unsigned)n_det), mf::kWT,
-                           (size_t)(bins * (n_seg | 1) * 8), st>>>(fd, ld_fd, n_det, (int)n_seg, seg_len, nm, bias, bins,
-                                                                   psd);
+      auto k = n_seg <= 128 ? mf::k_welch_median<4> : n_seg <= 512 ? mf::k_welch_median<16> : mf::k_welch_median<128>;
+      k<<<dim3((unsigned)((nb + bins - 1) / bins), (unsigned)n_det), mf::kWT, (size_t)(bins * (n_seg | 1) * 8), st>>>(
+          fd, ld_fd, n_det, (int)n_seg, seg_len, nm, bias, bins, psd);
     }
     mf::add_launches(1);
     e = cudaGetLastError();
