@@ -45,52 +45,88 @@ __global__ void __launch_bounds__(kCT) k_block_power(const void* __restrict__ ba
     for (int c = 0; c < pb; ++c) {
       const int k2 = cb * pb + c;
       const int64_t k = (int64_t)k1 * n2 + k2;
-      const double wk = w[k];
-      if (wk != 0.0) {
-        const float2 h = BankElem<BT>::get(row, (int64_t)k2 * R + k1);
-        acc += wk * ((double)h.x * h.x + (double)h.y * h.y);
+      const float2 h = BankElem<BT>::get(row, (int64_t)k2 * R + k1);
+      if (h.x != 0.f || h.y != 0.f) {  // (FP64 bounds this kernel: exact zeros are skipped)
+        const double wk = w[k];
+        if (wk != 0.0) acc += wk * ((double)h.x * h.x + (double)h.y * h.y);
       }
     }
     bpow[t * ((int64_t)R * nbl_row) + (int64_t)k1 * nbl_row + cb] = acc;
   }
 }
 
-// edges[t][l] = first bin k of band l, i.e. the first k with w[k] != 0 and
-// floor(p C(k) / sigma^2) >= l, with C(k) the template power below k (l < p);
-// edges[t][p] = nb.  One warp per template: lane l < p finds edge l from the
-// block sums, then within its block from the column-layout bank.
+// edges[t][l] = first bin k of band l, i.e. the first k with w[k] != 0 and p C(k) / sigma^2 >= l, with C(k) the
+// template power below k (l < p); edges[t][p] = nb.  One CTA per template: a prefix sum over the blocks, then a warp
+// per edge finds its block by bisection and its bin by a prefix sum over the block.  (A warp per template whose lanes
+// walked the blocks one by one, with an FP64 division each, took 0.7 ms for 150 templates at N = 2^18.)
+constexpr int kEdgeThreads = 256;
+
 template <int BT>
-__global__ void k_chisq_edges(const void* __restrict__ bank, int64_t ld_bank, int n1, int n2, int pb,
-                              const double* __restrict__ w, int64_t nb, const double* __restrict__ bpow,
-                              int64_t n_blocks, int64_t n_tmpl, int p, int32_t* __restrict__ edges) {
-  const int64_t t = blockIdx.x * (int64_t)(blockDim.x / 32) + threadIdx.x / 32;
-  const int lane = threadIdx.x & 31;
-  if (t >= n_tmpl) return;
+__global__ void __launch_bounds__(kEdgeThreads) k_chisq_edges(const void* __restrict__ bank, int64_t ld_bank, int n1,
+                                                              int n2, int pb, const double* __restrict__ w, int64_t nb,
+                                                              const double* __restrict__ bpow, int n_blocks, int p,
+                                                              int32_t* __restrict__ edges) {
+  extern __shared__ double below[];  // [n_blocks + 1] power below each block
+  __shared__ double part[kEdgeThreads];
+  const int64_t t = blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31;
   const double* bp = bpow + t * n_blocks;
-  double total = 0.0;
-  for (int64_t b = 0; b < n_blocks; ++b) total += bp[b];
+  const int per = (n_blocks + kEdgeThreads - 1) / kEdgeThreads, b0 = min(tid * per, n_blocks), b1 = min(b0 + per, n_blocks);
+  double s = 0.0;
+  for (int b = b0; b < b1; ++b) s += bp[b];
+  part[tid] = s;
+  __syncthreads();
+  if (tid == 0) {
+    double run = 0.0;
+    for (int i = 0; i < kEdgeThreads; ++i) {
+      const double v = part[i];
+      part[i] = run;
+      run += v;
+    }
+    below[n_blocks] = run;
+  }
+  __syncthreads();
+  double run = part[tid];
+  for (int b = b0; b < b1; ++b) {
+    below[b] = run;
+    run += bp[b];
+  }
+  __syncthreads();
+  const double total = below[n_blocks];
   const int R = n1 / 2;
   const void* row = static_cast<const unsigned char*>(bank) + t * ld_bank * (BT == kBankF32 ? 8 : 4);
-  for (int l = lane; l <= p; l += 32) {
+  for (int l = tid / 32; l <= p; l += kEdgeThreads / 32) {
     int64_t e = nb;
     if (l < p && total > 0.0) {
-      double below = 0.0;
-      int64_t b = 0;
-      // the first block whose end reaches band l (band(k) >= l needs p C(k) / total >= l)
-      while (b < n_blocks - 1 && floor((double)p * (below + bp[b]) / total) < (double)l) below += bp[b++];
-      for (int64_t k = b * pb; k < nb && e == nb; ++k) {
-        const double wk = w[k];
-        if (wk != 0.0 && floor((double)p * below / total) >= (double)l) {
-          e = k;
-          break;
-        }
-        if (wk != 0.0 && k < (int64_t)R * n2) {
-          const float2 h = BankElem<BT>::get(row, (k % n2) * R + k / n2);
-          below += wk * ((double)h.x * h.x + (double)h.y * h.y);
+      const double target = (double)l * total / (double)p;
+      int lo = 0, hi = n_blocks;  // the first block with power up to its end >= target
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (below[mid + 1] >= target) hi = mid; else lo = mid + 1;
+      }
+      for (int b = lo; b < n_blocks && e == nb; ++b) {
+        double c = below[b];  // power below the bins at hand
+        for (int k0 = b * pb; k0 < (b + 1) * pb && e == nb; k0 += 32) {
+          const int64_t k = k0 + lane;
+          const double wk = w[k];
+          double v = 0.0;
+          if (wk != 0.0) {
+            const float2 h = BankElem<BT>::get(row, (k % n2) * R + k / n2);
+            v = wk * ((double)h.x * h.x + (double)h.y * h.y);
+          }
+          double x = v;  // inclusive scan
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const double y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+          }
+          const unsigned m = __ballot_sync(0xffffffffu, wk != 0.0 && c + (x - v) >= target);
+          if (m) e = k0 + __ffs(m) - 1;
+          c += __shfl_sync(0xffffffffu, x, 31);
         }
       }
     }
-    edges[t * (p + 1) + l] = (int32_t)e;
+    if (lane == 0) edges[t * (p + 1) + l] = (int32_t)e;
   }
 }
 
@@ -100,7 +136,7 @@ struct TrigRecC {
   float snr, phase;
 };
 
-// chi^2 of a run of G triggers of one template and detector at a time.
+// chi^2 of a run of up to G triggers of one template and detector at a time.
 //
 // With k = k1 N2 + k2 the phase splits, exp(2 pi i k j / N) = exp(2 pi i k1 j / N1) exp(2 pi i k2 j / N), so a
 // thread takes one row k1 (or, below 256 rows, one of `parts` equal pieces of it, so that the CTA's pieces s are
@@ -108,20 +144,23 @@ struct TrigRecC {
 // turns the sum once.  Neighbouring threads read neighbouring k1, the bank's fastest index.  A band is a range
 // of bins, so most pieces lie in one band: sums of whole pieces go to whole[s], of a piece's part behind a
 // band's first bin to head[band], of its part in front of one to tail[band]; each has one writer, and a warp per
-// band adds them in a fixed order (FP64).  The triggers of a run share the loads: reading the template and the
-// data once per trigger from L2 would bound the kernel.  Before, a thread walked its own run of consecutive
-// elements (no two lanes in one line) with a phase recurrence, and one thread added all partial sums: 4,105 us
-// for the triggers of 150 templates of two detectors at N = 2^18, threshold 4.5 (2 MB of template and data each);
-// now 469 us.
+// band adds them in a fixed order (FP64).  The triggers of a run share the loads: reading the template and the data
+// from L2 once per run is what bounds the kernel.  Before, a thread walked its own run of consecutive elements (no
+// two lanes in one line) with a phase recurrence, and one thread added all partial sums: 4,105 us for the triggers of
+// 150 templates of two detectors at N = 2^18, threshold 4.5 (2 MB of template and data each); now
+// 417 us (469 us with runs of up to four).
 constexpr int kChiThreads = 256;
-constexpr int kChiRun = 4;  // triggers that share their loads
+constexpr int kChiRun = 8;  // triggers that share their loads, at most
+
+// half of that where the tables of eight would leave one CTA per SM
+constexpr int chisq_run_max(int n2) { return n2 <= 512 ? kChiRun : kChiRun / 2; }
 
 template <int BT, int QT, int G>
 __device__ __forceinline__ void chisq_run(const TrigRecC* __restrict__ trig, int64_t it, const void* __restrict__ bank,
                                           int64_t ld_bank, const void* __restrict__ q, int64_t ld_q, int n1, int n2,
                                           const int32_t* __restrict__ edges, int p, const float* __restrict__ ratio,
                                           const float* __restrict__ dscale, float* __restrict__ chi2,
-                                          float* __restrict__ newsnr, unsigned char* sm) {
+                                          float* __restrict__ newsnr, int n_run, unsigned char* sm) {
   const int R = n1 / 2, tid = threadIdx.x;
   const int parts = R < kChiThreads ? kChiThreads / R : 1, len = n2 / parts, pieces = R * parts;
   float2* ph = reinterpret_cast<float2*>(sm);  // [n2][G] phases of k2
@@ -134,10 +173,9 @@ __device__ __forceinline__ void chisq_run(const TrigRecC* __restrict__ trig, int
   const uint32_t N = (uint32_t)n1 * (uint32_t)n2;
   const void* hrow = static_cast<const unsigned char*>(bank) + (int64_t)tr.tmpl * ld_bank * (BT == kBankF32 ? 8 : 4);
   const void* qrow = static_cast<const unsigned char*>(q) + (int64_t)tr.det * ld_q * (QT == kBankF32 ? 8 : 4);
-  for (int i = tid; i < n2 * G; i += kChiThreads) {
-    const uint32_t j = (uint32_t)trig[it + i % G].sample;
-    ph[i] = unit_root((uint32_t)(((uint64_t)(i / G) * j) % N), N);
-  }
+  // a run shorter than G repeats its last trigger (products modulo powers of two: the low bits are all that counts)
+  auto sample = [&](int g) { return (uint32_t)trig[it + min(g, n_run - 1)].sample; };
+  for (int i = tid; i < n2 * G; i += kChiThreads) ph[i] = unit_root(((uint32_t)(i / G) * sample(i % G)) & (N - 1), N);
   for (int i = tid; i < (pieces + 2 * p) * G; i += kChiThreads) whole[i] = make_float2(0.f, 0.f);
   for (int i = tid; i <= p; i += kChiThreads) e[i] = edges[(int64_t)tr.tmpl * (p + 1) + i];
   __syncthreads();
@@ -159,8 +197,7 @@ __device__ __forceinline__ void chisq_run(const TrigRecC* __restrict__ trig, int
         float2* to = begin == 0 ? (end == len ? whole + s * G : tail + band * G) : head + band * G;
 #pragma unroll
         for (int g = 0; g < G; ++g) {
-          const uint32_t j = (uint32_t)trig[it + g].sample;
-          to[g] = cmul(acc[g], unit_root((uint32_t)(((uint64_t)k1 * j) % (uint32_t)n1), (uint32_t)n1));
+          to[g] = cmul(acc[g], unit_root(((uint32_t)k1 * sample(g)) & (uint32_t)(n1 - 1), (uint32_t)n1));
         }
       }
 #pragma unroll
@@ -229,7 +266,7 @@ __device__ __forceinline__ void chisq_run(const TrigRecC* __restrict__ trig, int
     if (lane == 0) zl[i] = make_double2(a, b);
   }
   __syncthreads();
-  if (tid < G) {
+  if (tid < n_run) {
     // z_l in stored units (data / sigma_ref, template / scale): |z_true| = |z| ratio / c_d
     float r = ratio[tr.tmpl];
     if (dscale) r /= dscale[tr.det];
@@ -251,18 +288,18 @@ __device__ __forceinline__ void chisq_run(const TrigRecC* __restrict__ trig, int
   __syncthreads();
 }
 
-constexpr int chisq_smem(int n1, int n2, int p, int g) {
-  const int pieces = n1 / 2 < kChiThreads ? kChiThreads : n1 / 2;
+constexpr int chisq_smem(int n1, int n2, int p) {
+  const int pieces = n1 / 2 < kChiThreads ? kChiThreads : n1 / 2, g = chisq_run_max(n2);
   return (n2 + pieces + 2 * p) * g * 8 + p * g * 16 + (p + 1) * 4;
 }
+constexpr int kChisqSmemMax =
+    chisq_smem(1024, 512, 64) > chisq_smem(1024, 1024, 64) ? chisq_smem(1024, 512, 64) : chisq_smem(1024, 1024, 64);
 
-constexpr int kChisqSmemMax = chisq_smem(1024, 1024, 64, kChiRun);  // 57 KB, four CTAs per SM
-
-// A CTA takes blocks of `per` consecutive triggers (the list is ordered by detector and template), as runs of
-// the same detector and template; per grows to kChiRun with the number of triggers, so that few of them still
-// spread over the grid.
+// The list is ordered by detector and template.  Each stretch of triggers of one detector and template is cut into
+// runs of G from its start on; a CTA takes the runs that begin in its block of `per` triggers.  G grows with the number
+// of triggers up to chisq_run_max, so that few of them still spread over the grid.
 template <int BT, int QT>
-__global__ void __launch_bounds__(kChiThreads) k_chisq(const TrigRecC* __restrict__ trig,
+__global__ void __launch_bounds__(kChiThreads, 2) k_chisq(const TrigRecC* __restrict__ trig,
                                                        const int64_t* __restrict__ count, int64_t cap,
                                                        const void* __restrict__ bank, int64_t ld_bank,
                                                        const void* __restrict__ q, int64_t ld_q, int n1, int n2,
@@ -272,23 +309,31 @@ __global__ void __launch_bounds__(kChiThreads) k_chisq(const TrigRecC* __restric
                                                        float* __restrict__ newsnr) {
   extern __shared__ __align__(16) unsigned char smc[];
   const int64_t n_trig = *count < cap ? *count : cap;
-  const int64_t per = min((int64_t)kChiRun, (n_trig + gridDim.x - 1) / gridDim.x);
-  for (int64_t b = blockIdx.x * per; b < n_trig; b += gridDim.x * per) {
-    const int64_t end = min(b + per, n_trig);
-    for (int64_t it = b; it < end;) {
-      int64_t to = it + 1;
-      while (to < end && trig[to].tmpl == trig[it].tmpl && trig[to].det == trig[it].det) ++to;
-      if (to - it == kChiRun) {
-        chisq_run<BT, QT, kChiRun>(trig, it, bank, ld_bank, q, ld_q, n1, n2, edges, p, ratio, dscale, chi2, newsnr, smc);
-        it = to;
-      } else if (to - it >= 2) {
-        chisq_run<BT, QT, 2>(trig, it, bank, ld_bank, q, ld_q, n1, n2, edges, p, ratio, dscale, chi2, newsnr, smc);
-        it += 2;
-      } else {
-        chisq_run<BT, QT, 1>(trig, it, bank, ld_bank, q, ld_q, n1, n2, edges, p, ratio, dscale, chi2, newsnr, smc);
-        it += 1;
-      }
-    }
+  const int64_t per = (n_trig + gridDim.x - 1) / gridDim.x;
+  const int G = (int)min((int64_t)chisq_run_max(n2), per), lane = threadIdx.x & 31;
+  const int64_t b0 = blockIdx.x * per, b1 = min(b0 + per, n_trig);
+  auto same = [&](int64_t a, int64_t b) { return trig[a].tmpl == trig[b].tmpl && trig[a].det == trig[b].det; };
+  if (b0 >= b1) return;
+  int64_t start = b0;  // of b0's stretch
+  for (;;) {
+    const int64_t i = start - 1 - lane;
+    const unsigned other = __ballot_sync(0xffffffffu, i < 0 || !same(i, b0));
+    start -= other ? __ffs(other) - 1 : 32;
+    if (other) break;
+  }
+  for (int64_t it = b0; it < b1; ++it) {
+    if (it > b0 && !same(it, it - 1)) start = it;
+    if ((it - start) % G != 0) continue;
+    int len = 1;
+    while (len < G && it + len < n_trig && same(it, it + len)) ++len;
+    if (len > 4)
+      chisq_run<BT, QT, kChiRun>(trig, it, bank, ld_bank, q, ld_q, n1, n2, edges, p, ratio, dscale, chi2, newsnr, len, smc);
+    else if (len > 2)
+      chisq_run<BT, QT, 4>(trig, it, bank, ld_bank, q, ld_q, n1, n2, edges, p, ratio, dscale, chi2, newsnr, len, smc);
+    else if (len == 2)
+      chisq_run<BT, QT, 2>(trig, it, bank, ld_bank, q, ld_q, n1, n2, edges, p, ratio, dscale, chi2, newsnr, len, smc);
+    else
+      chisq_run<BT, QT, 1>(trig, it, bank, ld_bank, q, ld_q, n1, n2, edges, p, ratio, dscale, chi2, newsnr, len, smc);
   }
 }
 
@@ -314,7 +359,7 @@ cudaError_t launch_chisq_edges(const void* bank, int bank_type, int64_t ld_bank,
   if (p < 2 || p > 64 || n_tmpl <= 0) return cudaErrorInvalidValue;
   const int pb = chisq_pb(n2);
   const int64_t nbl = chisq_blocks(n1, n2);
-  const unsigned g = (unsigned)((n_tmpl + 3) / 4);
+  const size_t smem = (size_t)(nbl + 1) * sizeof(double);  // up to 2,048 blocks: 16 KB
   for (int64_t t0 = 0; t0 < n_tmpl; t0 += 65535) {
     const dim3 gp((unsigned)(n2 / pb), (unsigned)std::min<int64_t>(65535, n_tmpl - t0));
     const int64_t eb = bank_type == kBankF32 ? 8 : 4;
@@ -329,9 +374,9 @@ cudaError_t launch_chisq_edges(const void* bank, int bank_type, int64_t ld_bank,
     add_launches(1);
   }
   switch (bank_type) {
-    case kBankF32: k_chisq_edges<kBankF32><<<g, 128, 0, st>>>(bank, ld_bank, n1, n2, pb, w, nb, bpow, nbl, n_tmpl, p, edges); break;
-    case kBankF16: k_chisq_edges<kBankF16><<<g, 128, 0, st>>>(bank, ld_bank, n1, n2, pb, w, nb, bpow, nbl, n_tmpl, p, edges); break;
-    case kBankBF16: k_chisq_edges<kBankBF16><<<g, 128, 0, st>>>(bank, ld_bank, n1, n2, pb, w, nb, bpow, nbl, n_tmpl, p, edges); break;
+    case kBankF32: k_chisq_edges<kBankF32><<<(unsigned)n_tmpl, kEdgeThreads, smem, st>>>(bank, ld_bank, n1, n2, pb, w, nb, bpow, (int)nbl, p, edges); break;
+    case kBankF16: k_chisq_edges<kBankF16><<<(unsigned)n_tmpl, kEdgeThreads, smem, st>>>(bank, ld_bank, n1, n2, pb, w, nb, bpow, (int)nbl, p, edges); break;
+    case kBankBF16: k_chisq_edges<kBankBF16><<<(unsigned)n_tmpl, kEdgeThreads, smem, st>>>(bank, ld_bank, n1, n2, pb, w, nb, bpow, (int)nbl, p, edges); break;
     default: return cudaErrorInvalidValue;
   }
   add_launches(1);
@@ -343,7 +388,7 @@ cudaError_t launch_chisq(const void* trig, const int64_t* count, int64_t cap, co
                          int p, const float* ratio, const float* dscale, float* chi2, float* newsnr, cudaStream_t st) {
   if (p < 2 || p > 64) return cudaErrorInvalidValue;
   const int grid = sms_c() * 4;
-  const int smem = chisq_smem(n1, n2, p, kChiRun);
+  const int smem = chisq_smem(n1, n2, p);
   const TrigRecC* t = static_cast<const TrigRecC*>(trig);
 #define MF_CHISQ(BT, QT)                                                                                        \
   do {                                                                                                          \
