@@ -148,7 +148,7 @@ struct TrigRecC {
 // from L2 once per run is what bounds the kernel.  Before, a thread walked its own run of consecutive elements (no
 // two lanes in one line) with a phase recurrence, and one thread added all partial sums: 4,105 us for the triggers of
 // 150 templates of two detectors at N = 2^18, threshold 4.5 (2 MB of template and data each); now
-// 417 us (469 us with runs of up to four).
+// 377 us (469 us with runs of up to four).
 constexpr int kChiThreads = 256;
 constexpr int kChiRun = 8;  // triggers that share their loads, at most
 
@@ -387,7 +387,7 @@ cudaError_t launch_chisq(const void* trig, const int64_t* count, int64_t cap, co
                          int64_t ld_bank, const void* q, int q_type, int64_t ld_q, int n1, int n2, const int32_t* edges,
                          int p, const float* ratio, const float* dscale, float* chi2, float* newsnr, cudaStream_t st) {
   if (p < 2 || p > 64) return cudaErrorInvalidValue;
-  const int grid = sms_c() * 4;
+  const int grid = sms_c() * 2;  // as many as are resident; twice as many have half the triggers each, and shorter runs: 417 us
   const int smem = chisq_smem(n1, n2, p);
   const TrigRecC* t = static_cast<const TrigRecC*>(trig);
 #define MF_CHISQ(BT, QT)                                                                                        \
