@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kCT) k_block_power(const void* __restrict__ ba
       const float2 h = BankElem<BT>::get(row, (int64_t)k2 * R + k1);
       if (h.x != 0.f || h.y != 0.f) {  // (FP64 bounds this kernel: exact zeros are skipped)
         const double wk = w[k];
-        if (wk != 0.0) acc += wk * ((double)h.x * h.x + (double)h.y * h.y);
+        if (nonzero_f64(wk)) acc = fma(wk, abs2_f64(h), acc);
       }
     }
     bpow[t * ((int64_t)R * nbl_row) + (int64_t)k1 * nbl_row + cb] = acc;
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(kEdgeThreads) k_chisq_edges(const void* __rest
           double v = 0.0;
           if (wk != 0.0) {
             const float2 h = BankElem<BT>::get(row, (k % n2) * R + k / n2);
-            v = wk * ((double)h.x * h.x + (double)h.y * h.y);
+            v = wk * abs2_f64(h);
           }
           double x = v;  // inclusive scan
 #pragma unroll

@@ -22,6 +22,26 @@ constexpr int stride_for(int pad, int lanes) {
   return s;
 }
 
+// |h|^2 in FP64, of which the chip does 2 operations per clock and SM, conversions and comparisons included.  Widening
+// a float is a shift of its bits, and its square is exact in FP64, so that y^2 is an integer product m^2 2^(2 (e - 150))
+// put in place: one FP64 operation is left of five.  The result is the rounded sum of two exact squares either way.
+// Subnormals, infinities and NaN take the plain form.  (Norms of 384 rows at N = 2^20, k_put_cols: 1,706 us with it,
+// 1,275 us so.)
+__device__ __forceinline__ double abs2_f64(float2 h) {
+  const uint32_t x = __float_as_uint(h.x) & 0x7fffffffu, y = __float_as_uint(h.y) & 0x7fffffffu;
+  auto fits = [](uint32_t v) { return v == 0 || v - 0x00800000u < 0x7f000000u; };
+  if (!fits(x) || !fits(y)) return (double)h.x * h.x + (double)h.y * h.y;
+  const double wide = __hiloint2double(x ? (int)((x >> 3) + 0x38000000u) : 0, (int)(x << 29));
+  const uint32_t m = (y & 0x007fffffu) | 0x00800000u;
+  const unsigned long long mm = (unsigned long long)m * m;  // in [2^46, 2^48)
+  const uint32_t s = (mm >> 47) ? 5 : 6;                     // mm 2^s in [2^52, 2^53): its leading one adds to the exponent
+  const unsigned long long sq = ((unsigned long long)(2 * (y >> 23) + 774 - s) << 52) + (mm << s);
+  return fma(wide, wide, __longlong_as_double((long long)(y ? sq : 0)));
+}
+
+// x != 0 without an FP64 comparison
+__device__ __forceinline__ bool nonzero_f64(double x) { return (__double_as_longlong(x) << 1) != 0; }
+
 template <int BT>
 struct BankElem;
 template <>

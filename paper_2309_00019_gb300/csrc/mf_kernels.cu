@@ -720,7 +720,7 @@ __device__ __forceinline__ float2 stored_value(typename Stored<BT>::E v) {
 __device__ __forceinline__ void add_norm(double& acc, float2 h, const double* __restrict__ w, int64_t k) {
   if (h.x != 0.f || h.y != 0.f) {
     const double wk = w[k];
-    if (wk != 0.0) acc += wk * ((double)h.x * h.x + (double)h.y * h.y);
+    if (nonzero_f64(wk)) acc = fma(wk, abs2_f64(h), acc);
   }
 }
 

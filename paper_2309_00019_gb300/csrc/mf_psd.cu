@@ -6,7 +6,7 @@
 // window and no detrending, averaged by the mean or by the median divided by
 // its bias for exponential periodogram values (FINDCHIRP, Appendix B).
 // The windowed segments go straight into the library's real-input transform (k_pass1 / k_pass2 with a windowing
-// load), and k_welch_reduce reduces each bin's periodogram values, FP64, over the segments.
+// load), and k_welch_mean or k_welch_median reduces each bin's periodogram values, FP64, over the segments.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -29,7 +29,7 @@ struct Norm {
 };
 
 __device__ __forceinline__ double periodogram(float2 z, double norm) {
-  return norm * ((double)z.x * z.x + (double)z.y * z.y);
+  return norm * abs2_f64(z);
 }
 
 // mean: a CTA takes 32 bins (256-byte reads), each warp every eighth segment, the warps' sums in order
@@ -120,7 +120,8 @@ __device__ __forceinline__ double median_of(const unsigned long long* s, int n) 
 // bin takes them into registers (K per lane, 32 K >= n_seg) and selects the middle ones.  The values are >= 0, so
 // their bits are in their order: the comparisons are integer ones, not FP64 ones, of which the chip does 2 per clock
 // and SM.  For 127 segments of two detectors and 8,193 bins: a CTA per bin that read one 8-byte value per row and
-// sorted them 223 us, keys read from shared memory for each comparison 59 us, now 44 us.
+// sorted them 223 us, keys read from shared memory for each comparison 59 us, the
+// same with keys in registers 44 us, and with abs2_f64 35 us.
 template <int K>
 __global__ void __launch_bounds__(kWT) k_welch_median(const float2* __restrict__ fd, int64_t ld_fd, int n_det,
                                                       int n_seg, int64_t n, Norm nm, double median_bias, int bins,
@@ -161,7 +162,8 @@ extern "C" mf_status mf_psd_welch(double fs, int32_t n_det, int64_t n_samples, c
   const int64_t rows = n_seg * n_det;
   const int64_t nb = seg_len / 2 + 1, ld_fd = (nb + 63) / 64 * 64;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  // one allocation for the call's work space (three, with their frees, were two thirds of a call's time)
+  // one allocation for the call's work space (three, with their frees, were two thirds of a call's time; fewer bytes,
+  // as intermediates of 8 MB of segments at a time, take as long to allocate and two more launches each: 302 -> 316 us)
   const size_t scratch_bytes = (size_t)rows * seg_len * sizeof(float2);
   char* work = nullptr;
   cudaError_t e = cudaMalloc((void**)&work, scratch_bytes + (size_t)rows * ld_fd * sizeof(float2));
