@@ -1,8 +1,9 @@
 // TMA-staged matched-filter kernels (the hot path of Eq. 1-2 / Sec. V.C).
 //
-// N = N1 N2 four-step transform on sm_103a: 128-thread CTAs, three per SM,
-// each a persistent loop over work items whose inputs are brought into shared
-// memory by the bulk-copy (TMA) engine while the previous item computes.
+// N = N1 N2 four-step transform on sm_103a: CTAs of 128 computing threads, as
+// many per SM as fit (k_cols16: 16 independent warps per SM), each a persistent
+// loop over work items whose inputs are brought into shared memory by the
+// bulk-copy (TMA) engine while the previous item computes.
 //   k_cols: item = C columns k2 of one (template, detector) series, the
 //           detector fastest in the item order.  The
 //           template bank and the weighted data are stored column-major over
@@ -15,6 +16,8 @@
 //           the scratch in panels of P = max(T(N1) / 2, RW(N2)) rows:
 //           element (j1, k2) of a series at (j1 / P) N2 P + k2 P + j1 % P,
 //           so that a warp's store covers whole 128-byte lines.
+//   k_cols16: k_cols for the FP16 intermediate of N = 2^20: a warp per column,
+//           stored in image order by one tensor-map copy per column.
 //   k_rows: item = RW rows j1 of one panel, brought in by a 3-D tensor-map
 //           copy (RW of the panel's P values at each k2; one 1-D bulk copy
 //           when RW = P); N2-point row transforms; rho^2 = |z|^2 / sigma^2 of

@@ -1,6 +1,7 @@
 // Tensor-core row pass of the matched filter (Eq. 1-2, Sec. V.C: the inverse
 // transform over coalescence time), N = N1 N2 with N2 = 1024, over the FP16
-// pass-1 -> pass-2 intermediate that k_cols writes in 8-row panels.
+// pass-1 -> pass-2 intermediate that k_cols16 (k_cols for FP16 pairs) writes in
+// 8-row panels.
 //
 // A row x[k2] (k2 = 32 p + q) has the 1024-point transform
 //   z[u + 32 v] = sum_q w32^{q v} w1024^{q u} Y[u][q],   Y[u][q] = sum_p w32^{p u} x[32 p + q],
@@ -10,7 +11,7 @@
 // along K and N) with FP16 operands and FP32 accumulation in tensor memory:
 //   stage 1: D1[(q, r)][(u, c)] = sum_(p, c') A1[(q, r)][(p, c')] B[(u, c)][(p, c')]
 //   stage 2: D2[(u, r)][(v, c)] = sum_(q, c') A2[(u, r)][(q, c')] B[(v, c)][(q, c')]
-// with B the embedded DFT matrix, A1 a panel of 8 rows (r) exactly as k_cols
+// with B the embedded DFT matrix, A1 a panel of 8 rows (r) exactly as pass 1
 // stored it (the MN-major operand image, one 32 KB bulk copy) and A2 the
 // stage-1 result times w1024^{q u}, rounded to FP16 (K-major).  M = 256 rows
 // per stage, as two M = 128 tiles.

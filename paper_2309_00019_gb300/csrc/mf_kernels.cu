@@ -689,7 +689,7 @@ __global__ void k_row_max(const float2* __restrict__ src, int64_t ld, int64_t nb
 // one row and a quarter of their k1 (kNormSplit; all of it below 4 tiles), which it walks in 32 x 32 tiles through shared memory, coalesced on both sides.  sigma^2 = sum w |h|^2
 // (FP64) is taken from the tiles on their way, in natural order, where the weights' reads are coalesced too:
 // as a pass of its own over the stored row it gathered the weights n2 bins apart and took 31.7 us per template
-// at N = 2^20, four fifths of loading a bank; now the row's transpose and its norm take 4.4 us.  The few FP64
+// at N = 2^20, four fifths of loading a bank; now the row's transpose and its norm take 3.3 us.  The few FP64
 // operations that the chip can do (2 per clock and SM) are the next bound, so bins outside the template's
 // band (exact zeros) are skipped.  Partial sums go to part[row][CTA of the row] and are added in order, so a row's
 // norm depends on its values alone: k_cols_norms takes the same partial sums from a stored row.
