@@ -131,6 +131,7 @@ __global__ void k_coinc(CoincArgs a) {
 // now 159 us.
 constexpr int kTmplWin = 2048;   // windows whose triggers fit the CTA's shared memory
 constexpr int kTmplRec = 512;    // records collected before they go out one by one
+constexpr int kTmplRun = 8;      // shifts of one pair from which on they go out together
 constexpr int kTmplThreads = 256;
 
 __global__ void __launch_bounds__(kTmplThreads) k_coinc_tmpl(CoincArgs a) {
@@ -138,7 +139,8 @@ __global__ void __launch_bounds__(kTmplThreads) k_coinc_tmpl(CoincArgs a) {
   __shared__ float rho2[2][kTmplWin];
   __shared__ uint16_t loud[2][kTmplWin];
   __shared__ uint2 found[kTmplRec];      // (detector-0 trigger | detector-1 trigger << 16, shift)
-  __shared__ int n_pos[2], n_loud[2], n_found;
+  __shared__ int n_pos[2], n_loud[2];
+  __shared__ unsigned n_found;  // collected, or found before it was seen that the collection is full
   __shared__ unsigned long long base;
   const int64_t p = blockIdx.x;
   const int tid = threadIdx.x;
@@ -174,16 +176,23 @@ __global__ void __launch_bounds__(kTmplThreads) k_coinc_tmpl(CoincArgs a) {
                     sqrtf(rho2[0][h] + rho2[1][l]),
                     0};
   };
-  auto emit = [&](int h, int l, int32_t k, float rc2) {
+  // A pair's coincidences at the shifts k0 .. k1.  A template can have more records than 32 bits count (2,048 windows of
+  // each detector, millions of shifts): the collection's counter stops when it is full (each thread that saw it free
+  // may add one more), and the rest and long runs of shifts are counted in the 64 bits of n_coinc.
+  auto emit = [&](int h, int l, int32_t k0, int32_t k1, float rc2) {
+    if (k1 < k0) return;
     follow |= rc2 >= a.rho_c_thr2;
     if (!(rc2 >= a.rho_c_store2)) return;
-    const int at = atomicAdd(&n_found, 1);
-    if (at < kTmplRec) {
-      found[at] = make_uint2((uint32_t)h | (uint32_t)l << 16, (uint32_t)k);
-    } else {
-      const unsigned long long slot = atomicAdd(a.n_coinc, 1ull);
-      if ((int64_t)slot < a.coinc_cap) reinterpret_cast<CoincRec*>(a.coincs)[slot] = record(h, l, k);
-    }
+    if (k1 - k0 < kTmplRun)
+      for (; k0 <= k1 && *(volatile unsigned*)&n_found < (unsigned)kTmplRec; ++k0) {
+        const unsigned at = atomicAdd(&n_found, 1u);
+        if (at >= (unsigned)kTmplRec) break;
+        found[at] = make_uint2((uint32_t)h | (uint32_t)l << 16, (uint32_t)k0);
+      }
+    if (k1 < k0) return;
+    unsigned long long slot = atomicAdd(a.n_coinc, (unsigned long long)(k1 - k0 + 1));
+    for (; k0 <= k1 && slot < (unsigned long long)a.coinc_cap; ++k0)
+      reinterpret_cast<CoincRec*>(a.coincs)[slot++] = record(h, l, k0);
   };
   auto pair = [&](int h, int l) {
     const float rc2 = rho2[0][h] + rho2[1][l];
@@ -191,8 +200,7 @@ __global__ void __launch_bounds__(kTmplThreads) k_coinc_tmpl(CoincArgs a) {
     int32_t D = pos[0][h] - pos[1][l];
     if (D < 0) D += R;
     if (step == 0) {
-      if (D <= cw || R - D <= cw)
-        for (int32_t k = 0; k <= a.n_shifts; ++k) emit(h, l, k, rc2);
+      if (D <= cw || R - D <= cw) emit(h, l, 0, a.n_shifts, rc2);
       return;
     }
     for (int32_t t = D - R; t - cw <= last; t += R) {
@@ -201,8 +209,9 @@ __global__ void __launch_bounds__(kTmplThreads) k_coinc_tmpl(CoincArgs a) {
       int32_t k = (int32_t)((float)(t + cw) * inv_step);
       while (k * step > t + cw) --k;
       while ((k + 1) * step <= t + cw) ++k;
-      for (; k >= 0 && k * step >= t - cw; --k)
-        if (k <= a.n_shifts) emit(h, l, k, rc2);
+      int32_t k0 = k + 1;  // the smallest with k step >= t - cw
+      while (k0 > 0 && (k0 - 1) * step >= t - cw) --k0;
+      emit(h, l, k0, min(k, a.n_shifts), rc2);
     }
   };
   for (int i = 0; i < n_loud[0]; ++i) {
@@ -214,7 +223,7 @@ __global__ void __launch_bounds__(kTmplThreads) k_coinc_tmpl(CoincArgs a) {
       for (int i = 0; i < n_loud[1]; ++i) pair(h, loud[1][i]);
   if (follow) a.followed[tmpl] = 1;
   __syncthreads();
-  const int count = min(n_found, kTmplRec);
+  const int count = (int)min(n_found, (unsigned)kTmplRec);
   if (tid == 0 && count > 0) base = atomicAdd(a.n_coinc, (unsigned long long)count);
   __syncthreads();
   for (int i = tid; i < count; i += kTmplThreads)
