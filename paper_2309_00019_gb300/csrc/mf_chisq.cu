@@ -460,11 +460,13 @@ __global__ void __launch_bounds__(kCT) k_sgchisq(const TrigRecC* __restrict__ tr
       if (!(f0 < f_high)) continue;
       const double tau = tiles.q / (1.4142135623730951 * 3.141592653589793 * f0);
       const double half = 6.0 / (3.141592653589793 * tau);
-      const int64_t klo = max((int64_t)1, (int64_t)ceil((f0 - half) / df));
-      const int64_t khi = min(nb - 2, (int64_t)floor((f0 + half) / df));
+      // (a tile far below zero ends below bin 0, and with q < 8.5 begins above it: both ends are held to the bins before
+      // they become 32-bit indices)
+      const int klo = (int)min(nb, max((int64_t)1, (int64_t)ceil((f0 - half) / df)));
+      const int khi = (int)max((int64_t)0, min(nb - 2, (int64_t)floor((f0 + half) / df)));
       float ar = 0.f, ai = 0.f;
       double s2 = 0.0;
-      for (int k = (int)klo + threadIdx.x; k <= (int)khi; k += kCT) {
+      for (int k = klo + threadIdx.x; k <= khi; k += kCT) {
         const double wk = w[k];
         if (!nonzero_f64(wk)) continue;
         const float x = (float)(3.141592653589793 * tau * ((double)k * df - f0));
