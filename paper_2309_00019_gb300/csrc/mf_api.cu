@@ -76,6 +76,7 @@ struct mf_plan_s {
   int64_t maxrho_cap = 0;
   bool coinc_done = false;
   int64_t sel_tmpl = 0;           // templates in the bank of the last filter
+  bool sel_ranges = false;        // its rows had analysed ranges of their own: trigger times may lie outside the ring
   int64_t coinc_tmpl = 0;         // and of the filter of the last mf_coincide
   int64_t coinc_shifts = 0;       // shifts of the last mf_coincide
   int64_t coinc_per_bin = 0;      // and a bound on its records per (template, shift)
@@ -741,6 +742,7 @@ mf_status mf_filter(mf_plan_t p, const void* dtilde, int64_t ld_dtilde, const in
   if (e != cudaSuccess) return cuda_fail(p, e, "mf_filter compaction");
   p->n_sel = n_sel;
   p->sel_tmpl = p->n_tmpl;
+  p->sel_ranges = p->row_valid != nullptr;
   p->filtered = true;
   p->coinc_done = false;
   return MF_OK;
@@ -989,7 +991,7 @@ mf_status mf_coincide(mf_plan_t p, const mf_coinc_desc* c, int32_t* followed) {
   a.coincs = p->coincs;
   a.coinc_cap = p->coinc_cap;
   a.n_coinc = p->n_coinc;
-  a.own_ranges = p->row_valid != nullptr;
+  a.own_ranges = p->sel_ranges;
   p->coinc_tmpl = p->sel_tmpl;
   p->coinc_shifts = (int64_t)c->n_shifts + 1;
   p->coinc_per_bin = p->n_win * (2 * c->window_samples / p->d.window + 2);
@@ -1254,6 +1256,7 @@ int filter_fused(mf_plan_s* const* plans, const void* const* dtilde, const int64
                        p->d.max_triggers, p->count, p->bc, p->bc_cap, st);
     if (e != cudaSuccess) return bad(MF_ECUDA, std::string("fused filter compaction: ") + cudaGetErrorString(e));
     p->n_sel = p->sel_tmpl = p->n_tmpl;
+    p->sel_ranges = p->row_valid != nullptr;
     p->filtered = true;
     p->coinc_done = false;
   }
