@@ -79,7 +79,6 @@ struct mf_plan_s {
   bool sel_ranges = false;        // its rows had analysed ranges of their own: trigger times may lie outside the ring
   int64_t coinc_tmpl = 0;         // and of the filter of the last mf_coincide
   int64_t coinc_shifts = 0;       // shifts of the last mf_coincide
-  int64_t coinc_per_bin = 0;      // and a bound on its records per (template, shift)
   char* coinc_work = nullptr;     // ordered records and the ordering's work space
   size_t coinc_work_cap = 0;
   // neighbourhood map
@@ -994,7 +993,6 @@ mf_status mf_coincide(mf_plan_t p, const mf_coinc_desc* c, int32_t* followed) {
   a.own_ranges = p->sel_ranges;
   p->coinc_tmpl = p->sel_tmpl;
   p->coinc_shifts = (int64_t)c->n_shifts + 1;
-  p->coinc_per_bin = p->n_win * (2 * c->window_samples / p->d.window + 2);
   LaunchScope ls(p);
   e = mf::launch_coinc(a, p->maxrho, p->st);
   if (e != cudaSuccess) return cuda_fail(p, e, "mf_coincide kernels");
@@ -1012,29 +1010,39 @@ mf_status mf_get_coincs(mf_plan_t p, mf_coinc* out, int64_t cap, int64_t* n_foun
   *n_found = (int64_t)n;
   const int64_t have = std::min<int64_t>((int64_t)n, p->coinc_cap);
   const int64_t m = std::min<int64_t>(have, cap);
-  // Ordered on the device where each (template, shift) has few records (a window's detector-0 peak meets the peaks
-  // of 2 window_samples / window + 2 windows at most; 512 windows and the usual 15 ms: 1,024) and the bins fit an
-  // int32 index (duplicate ids in the selection only make the ranks slower); the host's sort of 110,000 records
-  // took 3.4 ms.
+  // Ordered on the device from kOrderMin records on, unless the (template, shift) bins are far more than the records
+  // (their counters are cleared and scanned: 16 MB of them always pass) or its memory cannot be had: then, and where
+  // k_co_rank finds a bin too crowded to count ranks in, on the host.  11 records: host 29 us, device
+  // 58 us; 1,957: 57 and 59 us; 117,000: 3,423 and 96 us.
+  constexpr int64_t kOrderMin = 2048;
   const int64_t bins = p->coinc_tmpl * p->coinc_shifts;
-  if (m > 0 && p->coinc_per_bin <= 4096 && p->coinc_shifts < (1 << 24) && bins < (int64_t(1) << 26) &&
-      have < (int64_t(1) << 30)) {
+  bool ordered = false;
+  if (m > 0 && have >= kOrderMin && have < (int64_t(1) << 30) && p->coinc_shifts < (1 << 24) &&
+      bins < (int64_t(1) << 26) && bins <= (int64_t(1) << 22) + 16 * have) {
     const size_t rec = ((size_t)have * sizeof(mf_coinc) + 255) / 256 * 256;
     const size_t need = rec + mf::coinc_order_bytes(have, bins);
-    mf_status s;
-    if (need > p->coinc_work_cap) {
+    bool room = need <= p->coinc_work_cap;
+    if (!room) {
       p->coinc_work_cap = 0;
-      if ((s = dalloc(p, &p->coinc_work, need + need / 4, "coincidence order")) != MF_OK) return s;
-      p->coinc_work_cap = need + need / 4;
+      room = dalloc(p, &p->coinc_work, need + need / 4, "coincidence order") == MF_OK;
+      if (room) p->coinc_work_cap = need + need / 4;
     }
-    LaunchScope ls(p);
-    e = mf::launch_coinc_order(p->coincs, have, p->coinc_tmpl, (int)p->coinc_shifts, p->coinc_work + rec, p->coinc_work,
-                               p->st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(out, p->coinc_work, m * sizeof(mf_coinc), cudaMemcpyDeviceToHost, p->st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(p->st);
-    if (e != cudaSuccess) return cuda_fail(p, e, "mf_get_coincs");
-  } else if (m > 0) try {  // a count-only call (cap 0) copies nothing; no allocation failure crosses the ABI
+    if (room) {
+      LaunchScope ls(p);
+      int32_t* crowded_dev = nullptr;
+      int32_t crowded = 0;
+      e = mf::launch_coinc_order(p->coincs, have, p->coinc_tmpl, (int)p->coinc_shifts, p->coinc_work + rec,
+                                 p->coinc_work, &crowded_dev, p->st);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(out, p->coinc_work, m * sizeof(mf_coinc), cudaMemcpyDeviceToHost, p->st);
+      if (e == cudaSuccess && have > mf::kCoincCrowd)  // fewer records cannot crowd a bin
+        e = cudaMemcpyAsync(&crowded, crowded_dev, sizeof(crowded), cudaMemcpyDeviceToHost, p->st);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(p->st);
+      if (e != cudaSuccess) return cuda_fail(p, e, "mf_get_coincs");
+      ordered = crowded == 0;
+    }
+  }
+  if (m > 0 && !ordered) try {  // a count-only call (cap 0) copies nothing; no allocation failure crosses the ABI
     std::unique_ptr<mf_coinc[]> rec(new mf_coinc[have]);
     e = cudaMemcpyAsync(rec.get(), p->coincs, have * sizeof(mf_coinc), cudaMemcpyDeviceToHost, p->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(p->st);

@@ -234,7 +234,9 @@ __global__ void __launch_bounds__(kTmplThreads) k_coinc_tmpl(CoincArgs a) {
 
 // --- coincidence records in order (tmpl, shift, sample0, sample1) ------------------
 // Counting sort over the (tmpl, shift) bins, then each record's rank in its bin: a bin holds at most a few records
-// per window, so the ranks are counted directly.
+// per window, so the ranks are counted directly.  That is quadratic in a bin's records, which a selection that names a
+// template many times multiplies: 394,000 records in 21 bins take 4.4 ms here and 37 ms on the host, where bins of more
+// than kCoincCrowd are left to.
 
 constexpr int kScanSpan = 4096;  // bins per scan CTA (1024 threads x 4)
 
@@ -318,11 +320,15 @@ __global__ void k_co_group(const CoincRec* __restrict__ rec, int64_t n, int n_sh
 
 __global__ void k_co_rank(const CoincRec* __restrict__ rec, const CoincKey* __restrict__ grouped, int64_t n,
                           const int32_t* __restrict__ bins, const int32_t* __restrict__ sums,
-                          CoincRec* __restrict__ out) {
+                          CoincRec* __restrict__ out, int32_t* __restrict__ crowded) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const CoincKey k = grouped[i];
     const int32_t begin = k.bin > 0 ? bins[k.bin - 1] + sums[(k.bin - 1) / kScanSpan] : 0;
     const int32_t end = bins[k.bin] + sums[k.bin / kScanSpan];
+    if (end - begin > kCoincCrowd) {
+      *crowded = 1;
+      continue;
+    }
     int32_t rank = begin;
     for (int32_t j = begin; j < end; ++j) {
       const unsigned long long o = grouped[j].key;
@@ -422,24 +428,26 @@ cudaError_t launch_coinc(const CoincArgs& a, float* max_rho2_det1, cudaStream_t 
 
 size_t coinc_order_bytes(int64_t n, int64_t n_bins) {
   const int64_t sums = (n_bins + kScanSpan - 1) / kScanSpan;
-  return (size_t)n * sizeof(CoincKey) + (size_t)(n_bins + sums) * sizeof(int32_t);
+  return (size_t)n * sizeof(CoincKey) + (size_t)(n_bins + sums + 1) * sizeof(int32_t);
 }
 
 cudaError_t launch_coinc_order(const void* rec, int64_t n, int64_t n_tmpl, int n_shift, void* work, void* out,
-                               cudaStream_t st) {
+                               int32_t** crowded, cudaStream_t st) {
   const int64_t n_bins = n_tmpl * n_shift, n_sums = (n_bins + kScanSpan - 1) / kScanSpan;
   CoincKey* grouped = static_cast<CoincKey*>(work);
   int32_t* bins = reinterpret_cast<int32_t*>(grouped + n);
-  int32_t* sums = bins + n_bins;
+  int32_t* flag = bins + n_bins;  // cleared with the bins
+  int32_t* sums = flag + 1;
+  *crowded = flag;
   const CoincRec* r = static_cast<const CoincRec*>(rec);
-  cudaError_t e = cudaMemsetAsync(bins, 0, (size_t)n_bins * sizeof(int32_t), st);
+  cudaError_t e = cudaMemsetAsync(bins, 0, (size_t)(n_bins + 1) * sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
   const unsigned g = (unsigned)((n + 255) / 256 < sms() * 8 ? (n + 255) / 256 : sms() * 8);
   k_co_hist<<<g, 256, 0, st>>>(r, n, n_shift, bins);
   k_co_scan<<<(unsigned)n_sums, 1024, 0, st>>>(bins, n_bins, sums);
   k_co_scan_sums<<<1, 1024, 0, st>>>(sums, (int)n_sums);
   k_co_group<<<g, 256, 0, st>>>(r, n, n_shift, bins, sums, grouped);
-  k_co_rank<<<g, 256, 0, st>>>(r, grouped, n, bins, sums, static_cast<CoincRec*>(out));
+  k_co_rank<<<g, 256, 0, st>>>(r, grouped, n, bins, sums, static_cast<CoincRec*>(out), flag);
   add_launches(5);
   return cudaGetLastError();
 }

@@ -296,11 +296,13 @@ struct CoincArgs {
   int own_ranges;                   // rows have analysed ranges of their own: times may lie outside the ring
 };
 cudaError_t launch_coinc(const CoincArgs& a, float* max_rho2_det1, cudaStream_t st);
-// n coincidence records in the order (tmpl, shift, sample0, sample1) into out; tmpl < n_tmpl, shift < n_shift, and
-// few records per (tmpl, shift) (their ranks are counted); work: coinc_order_bytes(n, n_tmpl n_shift)
+// n coincidence records in the order (tmpl, shift, sample0, sample1) into out; tmpl < n_tmpl, shift < n_shift; work:
+// coinc_order_bytes(n, n_tmpl n_shift).  Ranks are counted in each (tmpl, shift) bin: with more than kCoincCrowd records
+// in one (a template many times in the selection) *crowded, in the work space, becomes 1 and out is not complete.
+constexpr int kCoincCrowd = 65536;
 size_t coinc_order_bytes(int64_t n, int64_t n_bins);
 cudaError_t launch_coinc_order(const void* rec, int64_t n, int64_t n_tmpl, int n_shift, void* work, void* out,
-                               cudaStream_t st);
+                               int32_t** crowded, cudaStream_t st);
 cudaError_t launch_union(const int64_t* ptr, const int32_t* idx, int64_t n_coarse, const int32_t* followed,
                          int32_t* flags, int64_t n_fine, int32_t* subset, int64_t* n_subset,
                          int64_t* block_counts, cudaStream_t st);
