@@ -128,37 +128,53 @@ __global__ void k_coinc(CoincArgs a) {
 // of its times, k step in [D + m R - window, D + m R + window], without a walk over them.  What a CTA finds is
 // collected in shared memory and written in one go.  Trying all 102 shifts for every detector-0 trigger of a
 // template with one loud detector-1 trigger took 512 us on the coarse stage (2,000 templates, 512 windows each);
-// now 159 us.
+// now 159 us.  Where most triggers are loud the CTA walks over the shifts instead: pairs alone took 2,750 us for 50
+// templates of 2,048 windows at zero lag, the walk takes 20 us (k_coinc 22 us), and 154 us for 100 templates and 101
+// shifts (pairs 4,800 us, k_coinc 535 us).
 constexpr int kTmplWin = 2048;   // windows whose triggers fit the CTA's shared memory
 constexpr int kTmplRec = 512;    // records collected before they go out one by one
-constexpr int kTmplRun = 8;      // shifts of one pair from which on they go out together
-constexpr int kTmplThreads = 256;
+constexpr int kWalkShifts = 64;  // shifts that a thread walks at a time
 
-__global__ void __launch_bounds__(kTmplThreads) k_coinc_tmpl(CoincArgs a) {
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : 1) k_coinc_tmpl(CoincArgs a) {
   __shared__ int32_t pos[2][kTmplWin];   // ring positions of the triggers of detector 0, 1
   __shared__ float rho2[2][kTmplWin];
   __shared__ uint16_t loud[2][kTmplWin];
   __shared__ uint2 found[kTmplRec];      // (detector-0 trigger | detector-1 trigger << 16, shift)
   __shared__ int n_pos[2], n_loud[2];
   __shared__ unsigned n_found;  // collected, or found before it was seen that the collection is full
+  __shared__ unsigned max1;     // the largest rho^2 of detector 1 (float bits)
   __shared__ unsigned long long base;
   const int64_t p = blockIdx.x;
   const int tid = threadIdx.x;
   if (tid < 2) n_pos[tid] = n_loud[tid] = 0;
-  if (tid == 2) n_found = 0;
+  if (tid == 2) n_found = max1 = 0;
   __syncthreads();
   const float need = fminf(a.rho_c_thr2, a.rho_c_store2), half = 0.5f * need;
   const int32_t rb = (int32_t)a.ring_begin;
-  for (int i = tid; i < 2 * (int)a.n_win; i += kTmplThreads) {
-    const int d = i >= (int)a.n_win;
-    const unsigned long long key = a.slots[(d * a.n_sel + p) * a.n_win + (i - d * a.n_win)];
-    if (key == 0ull) continue;
-    const int at = atomicAdd(&n_pos[d], 1);
-    const float r = key_rho2(key);
-    pos[d][at] = (int32_t)key_sample(key) - rb;
-    rho2[d][at] = r;
-    if (r >= half) loud[d][atomicAdd(&n_loud[d], 1)] = (uint16_t)at;
-  }
+  const int lane = tid & 31;
+  for (int d = 0; d < 2; ++d)
+    for (int i0 = tid - lane; i0 < (int)a.n_win; i0 += THREADS) {  // a warp's triggers at a time
+      const unsigned long long key = i0 + lane < (int)a.n_win ? a.slots[(d * a.n_sel + p) * a.n_win + i0 + lane] : 0ull;
+      const float r = key_rho2(key);
+      const unsigned has = __ballot_sync(0xffffffffu, key != 0ull);
+      const unsigned big = __ballot_sync(0xffffffffu, key != 0ull && r >= half);
+      if (!has) continue;
+      int base_pos = 0, base_loud = 0;
+      if (lane == 0) {
+        base_pos = atomicAdd(&n_pos[d], __popc(has));
+        if (big) base_loud = atomicAdd(&n_loud[d], __popc(big));
+      }
+      base_pos = __shfl_sync(0xffffffffu, base_pos, 0);
+      base_loud = __shfl_sync(0xffffffffu, base_loud, 0);
+      const unsigned before = (1u << lane) - 1u;
+      const int at = base_pos + __popc(has & before);
+      if (key != 0ull) {
+        pos[d][at] = (int32_t)key_sample(key) - rb;
+        rho2[d][at] = r;
+        if (r >= half) loud[d][base_loud + __popc(big & before)] = (uint16_t)at;
+      }
+    }
   __syncthreads();
   if (n_loud[0] + n_loud[1] == 0) return;
   const int32_t tmpl = a.sel[p];
@@ -176,31 +192,33 @@ __global__ void __launch_bounds__(kTmplThreads) k_coinc_tmpl(CoincArgs a) {
                     sqrtf(rho2[0][h] + rho2[1][l]),
                     0};
   };
-  // A pair's coincidences at the shifts k0 .. k1.  A template can have more records than 32 bits count (2,048 windows of
-  // each detector, millions of shifts): the collection's counter stops when it is full (each thread that saw it free
-  // may add one more), and the rest and long runs of shifts are counted in the 64 bits of n_coinc.
-  auto emit = [&](int h, int l, int32_t k0, int32_t k1, float rc2) {
-    if (k1 < k0) return;
-    follow |= rc2 >= a.rho_c_thr2;
-    if (!(rc2 >= a.rho_c_store2)) return;
-    if (k1 - k0 < kTmplRun)
-      for (; k0 <= k1 && *(volatile unsigned*)&n_found < (unsigned)kTmplRec; ++k0) {
-        const unsigned at = atomicAdd(&n_found, 1u);
-        if (at >= (unsigned)kTmplRec) break;
-        found[at] = make_uint2((uint32_t)h | (uint32_t)l << 16, (uint32_t)k0);
-      }
-    if (k1 < k0) return;
+  // Straight to the list, counted in the 64 bits of n_coinc: a pair at the shifts k0 .. k1
+  auto emit_run = [&](int h, int l, int32_t k0, int32_t k1) {
     unsigned long long slot = atomicAdd(a.n_coinc, (unsigned long long)(k1 - k0 + 1));
     for (; k0 <= k1 && slot < (unsigned long long)a.coinc_cap; ++k0)
       reinterpret_cast<CoincRec*>(a.coincs)[slot++] = record(h, l, k0);
+  };
+  // A template can have more records than 32 bits count (2,048 windows of each detector, millions of shifts): the
+  // collection's counter stops when it is full (each thread that saw it free may add one more)
+  auto emit = [&](int h, int l, int32_t k, float rc2) {
+    follow |= rc2 >= a.rho_c_thr2;
+    if (!(rc2 >= a.rho_c_store2)) return;
+    unsigned at = kTmplRec;
+    if (*(volatile unsigned*)&n_found < (unsigned)kTmplRec) at = atomicAdd(&n_found, 1u);
+    if (at < (unsigned)kTmplRec)
+      found[at] = make_uint2((uint32_t)h | (uint32_t)l << 16, (uint32_t)k);
+    else
+      emit_run(h, l, k, k);
   };
   auto pair = [&](int h, int l) {
     const float rc2 = rho2[0][h] + rho2[1][l];
     if (!(rc2 >= need)) return;
     int32_t D = pos[0][h] - pos[1][l];
     if (D < 0) D += R;
-    if (step == 0) {
-      if (D <= cw || R - D <= cw) emit(h, l, 0, a.n_shifts, rc2);
+    if (step == 0) {  // all shifts or none
+      if (D > cw && R - D > cw) return;
+      follow |= rc2 >= a.rho_c_thr2;
+      if (rc2 >= a.rho_c_store2) emit_run(h, l, 0, a.n_shifts);
       return;
     }
     for (int32_t t = D - R; t - cw <= last; t += R) {
@@ -209,24 +227,72 @@ __global__ void __launch_bounds__(kTmplThreads) k_coinc_tmpl(CoincArgs a) {
       int32_t k = (int32_t)((float)(t + cw) * inv_step);
       while (k * step > t + cw) --k;
       while ((k + 1) * step <= t + cw) ++k;
-      int32_t k0 = k + 1;  // the smallest with k step >= t - cw
-      while (k0 > 0 && (k0 - 1) * step >= t - cw) --k0;
-      emit(h, l, k0, min(k, a.n_shifts), rc2);
+      for (; k >= 0 && k * step >= t - cw; --k)
+        if (k <= a.n_shifts) emit(h, l, k, rc2);
     }
   };
-  for (int i = 0; i < n_loud[0]; ++i) {
-    const int h = loud[0][i];
-    for (int l = tid; l < n_pos[1]; l += kTmplThreads) pair(h, l);
+  // Pairs are few where few triggers are loud.  Where most are (thresholds near sqrt(2) times the filter's, or below) it
+  // is less work to walk over the shifts of every detector-0 trigger and look into the windows of detector 1 that it
+  // falls on.  A pair whose SNRs suffice goes through the turns of the ring (of those with one quiet trigger a
+  // quarter, say); a step of the walk costs about two of a pair.
+  const int64_t loud2 = (int64_t)n_loud[0] * n_loud[1];
+  const int64_t mixed = (int64_t)n_loud[0] * n_pos[1] + (int64_t)n_pos[0] * n_loud[1] - 2 * loud2;
+  if (loud2 + mixed + a.turns * (loud2 + mixed / 4) <= n_pos[0] * a.walk_steps) {
+    for (int i = 0; i < n_loud[0]; ++i) {
+      const int h = loud[0][i];
+      for (int l = tid; l < n_pos[1]; l += THREADS) pair(h, l);
+    }
+    for (int h = tid; h < n_pos[0]; h += THREADS)
+      if (rho2[0][h] < half)
+        for (int i = 0; i < n_loud[1]; ++i) pair(h, loud[1][i]);
+  } else {
+    auto window_of = [&](int32_t x) { return (int)(((uint64_t)(x + rb) * a.win_recip) >> kRecipBits); };
+    uint16_t* at = loud[0];  // detector-1 trigger of each window (the loud ones are not looked at here)
+    for (int w = tid; w < (int)a.n_win; w += THREADS) at[w] = 0xffffu;
+    __syncthreads();
+    for (int l = tid; l < n_pos[1]; l += THREADS) {
+      at[window_of(pos[1][l])] = (uint16_t)l;
+      atomicMax(&max1, __float_as_uint(rho2[1][l]));
+    }
+    __syncthreads();
+    const int chunks = a.n_shifts / kWalkShifts + 1;
+    for (int i = tid; i < n_pos[0] * chunks; i += THREADS) {
+      const int h = i % n_pos[0], kb = i / n_pos[0] * kWalkShifts, ke = min(kb + kWalkShifts - 1, a.n_shifts);
+      if (!(rho2[0][h] + __uint_as_float(max1) >= need)) continue;
+      int32_t x = pos[0][h] - kb * step % R;  // ring position at shift kb
+      if (x < 0) x += R;
+      for (int32_t k = kb; k <= ke; ++k) {
+        for (int side = 0; side < 2; ++side) {  // [x - cw, x + cw], cut at the ring's end
+          int32_t lo = x - cw, hi = x + cw;
+          if (side == 0) {
+            lo = max(lo, 0);
+            hi = min(hi, R - 1);
+          } else if (lo < 0) {
+            lo += R;
+            hi = R - 1;
+          } else if (hi >= R) {
+            lo = 0;
+            hi -= R;
+          } else {
+            break;
+          }
+          for (int w = window_of(lo); w <= window_of(hi); ++w) {
+            const int l = at[w];
+            if (l == 0xffff || pos[1][l] < lo || pos[1][l] > hi) continue;
+            emit(h, l, k, rho2[0][h] + rho2[1][l]);
+          }
+        }
+        x -= step;
+        if (x < 0) x += R;
+      }
+    }
   }
-  for (int h = tid; h < n_pos[0]; h += kTmplThreads)
-    if (rho2[0][h] < half)
-      for (int i = 0; i < n_loud[1]; ++i) pair(h, loud[1][i]);
   if (follow) a.followed[tmpl] = 1;
   __syncthreads();
   const int count = (int)min(n_found, (unsigned)kTmplRec);
   if (tid == 0 && count > 0) base = atomicAdd(a.n_coinc, (unsigned long long)count);
   __syncthreads();
-  for (int i = tid; i < count; i += kTmplThreads)
+  for (int i = tid; i < count; i += THREADS)
     if ((int64_t)base + i < a.coinc_cap)
       reinterpret_cast<CoincRec*>(a.coincs)[base + i] =
           record((int)(found[i].x & 0xffffu), (int)(found[i].x >> 16), (int32_t)found[i].y);
@@ -414,7 +480,19 @@ cudaError_t launch_coinc(const CoincArgs& a, float* max_rho2_det1, cudaStream_t 
   const int64_t R = a.ring_end - a.ring_begin;
   if (a.n_win <= kTmplWin && !a.own_ranges &&
       (int64_t)a.n_shifts * (a.shift % R) + 4 * R + a.coinc_window < (int64_t(1) << 30) && a.n_shifts < (1 << 22)) {
-    k_coinc_tmpl<<<(unsigned)a.n_sel, kTmplThreads, 0, st>>>(a);
+    CoincArgs t = a;
+    t.win_recip = window_recip(a.window);
+    t.turns = ((int64_t)a.n_shifts * (a.shift % R) + a.coinc_window) / R + 2;
+    t.walk_steps = 2 * (int64_t)(a.n_shifts + 1) * (2 * a.coinc_window / a.window + 2);
+    // a thread per window up to 512, and up to 1,024 where every template has an SM to itself (one such CTA fits): 2,000
+    // templates of 512 windows at zero lag, most triggers loud, 35 us with 256 threads and 44 with 512; 2,048 windows,
+    // 1,000 templates at zero lag 63 / 49 / 63 us with 256 / 512 / 1,024, one template and four shifts 44 / 32 / 24 us
+    if (a.n_win <= 512)
+      k_coinc_tmpl<256><<<(unsigned)a.n_sel, 256, 0, st>>>(t);
+    else if (a.n_win <= 1024 || a.n_sel > sms())
+      k_coinc_tmpl<512><<<(unsigned)a.n_sel, 512, 0, st>>>(t);
+    else
+      k_coinc_tmpl<1024><<<(unsigned)a.n_sel, 1024, 0, st>>>(t);
     add_launches(1);
     return cudaGetLastError();
   }
