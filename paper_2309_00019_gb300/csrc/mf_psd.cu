@@ -122,6 +122,10 @@ __device__ __forceinline__ double median_of(const unsigned long long* s, int n) 
 // and SM.  For 127 segments of two detectors and 8,193 bins: a CTA per bin that read one 8-byte value per row and
 // sorted them 223 us, keys read from shared memory for each comparison 59 us, the
 // same with keys in registers 44 us, and with abs2_f64 35 us.
+// K goes in steps, for a lane compares all its K keys however few there are (segments of 2^14 samples, two detectors,
+// the whole call: 1,000 segments 2,785 us with the sort, 3,211 with K = 128, 1,046 with K = 32; 2,000 of 2^12 samples 1,696,
+// 1,753 and, K = 64, 943).  K = 128 needs more registers than there are (255, 480 bytes of spills): from 2,049 segments on
+// it is what it is, 4,096 of 2^12 samples 3,293 us with the sort and 3,102 so.
 template <int K>
 __global__ void __launch_bounds__(kWT) k_welch_median(const float2* __restrict__ fd, int64_t ld_fd, int n_det,
                                                       int n_seg, int64_t n, Norm nm, double median_bias, int bins,
@@ -185,7 +189,11 @@ extern "C" mf_status mf_psd_welch(double fs, int32_t n_det, int64_t n_samples, c
     } else {
       int bins = 32;
       while (bins > 1 && bins * (n_seg | 1) * 8 > mf::kMedianBytes) bins /= 2;
-      auto k = n_seg <= 128 ? mf::k_welch_median<4> : n_seg <= 512 ? mf::k_welch_median<16> : mf::k_welch_median<128>;
+      auto k = n_seg <= 128    ? mf::k_welch_median<4>
+               : n_seg <= 512  ? mf::k_welch_median<16>
+               : n_seg <= 1024 ? mf::k_welch_median<32>
+               : n_seg <= 2048 ? mf::k_welch_median<64>
+                               : mf::k_welch_median<128>;
       k<<<dim3((unsigned)((nb + bins - 1) / bins), (unsigned)n_det), mf::kWT, (size_t)(bins * (n_seg | 1) * 8), st>>>(
           fd, ld_fd, n_det, (int)n_seg, seg_len, nm, bias, bins, psd);
     }
