@@ -32,20 +32,23 @@ __device__ __forceinline__ double periodogram(float2 z, double norm) {
   return norm * abs2_f64(z);
 }
 
-// mean: a CTA takes 32 bins (256-byte reads), each warp every eighth segment, the warps' sums in order
-__global__ void __launch_bounds__(kWT) k_welch_mean(const float2* __restrict__ fd, int64_t ld_fd, int n_det,
-                                                    int64_t n_seg, int64_t n, Norm nm, double* __restrict__ psd) {
-  __shared__ double part[kWT / 32][32];
+// mean: a CTA takes 32 bins (256-byte reads), each of its W warps every W-th segment, the warps' sums in order.  Eight
+// warps; beyond 4,096 segments their walk is longer than everything else in the call, and 32 share it (20,000 segments of
+// 2^12 samples: 2,728 -> 2,140 us; a CTA per bin took 2,522).
+template <int W>
+__global__ void __launch_bounds__(32 * W) k_welch_mean(const float2* __restrict__ fd, int64_t ld_fd, int n_det,
+                                                       int64_t n_seg, int64_t n, Norm nm, double* __restrict__ psd) {
+  __shared__ double part[W][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, d = blockIdx.y;
   const int64_t k = (int64_t)blockIdx.x * 32 + lane;
   const double norm = k == 0 || k == n / 2 ? nm.edge : nm.inner;
   double s = 0.0;
   if (k <= n / 2)
-    for (int64_t i = w; i < n_seg; i += kWT / 32) s += periodogram(fd[(i * n_det + d) * ld_fd + k], norm);
+    for (int64_t i = w; i < n_seg; i += W) s += periodogram(fd[(i * n_det + d) * ld_fd + k], norm);
   part[w][lane] = s;
   __syncthreads();
   if (w == 0 && k <= n / 2) {
-    for (int i = 1; i < kWT / 32; ++i) s += part[i][lane];
+    for (int i = 1; i < W; ++i) s += part[i][lane];
     psd[(int64_t)d * (n / 2 + 1) + k] = s / (double)n_seg;
   }
 }
@@ -184,8 +187,11 @@ extern "C" mf_status mf_psd_welch(double fs, int32_t n_det, int64_t n_samples, c
   e = mf::launch_welch_spectra(strain, ld, n_det, stride, (int)rows, seg_len, 1.0 / fs, scratch, fd, ld_fd, st);
   if (e == cudaSuccess) {
     if (average == 0) {
-      mf::k_welch_mean<<<dim3((unsigned)((nb + 31) / 32), (unsigned)n_det), mf::kWT, 0, st>>>(fd, ld_fd, n_det, n_seg,
-                                                                                             seg_len, nm, psd);
+      const dim3 grid((unsigned)((nb + 31) / 32), (unsigned)n_det);
+      if (n_seg <= 4096)
+        mf::k_welch_mean<8><<<grid, 256, 0, st>>>(fd, ld_fd, n_det, n_seg, seg_len, nm, psd);
+      else
+        mf::k_welch_mean<32><<<grid, 1024, 0, st>>>(fd, ld_fd, n_det, n_seg, seg_len, nm, psd);
     } else {
       int bins = 32;
       while (bins > 1 && bins * (n_seg | 1) * 8 > mf::kMedianBytes) bins /= 2;
