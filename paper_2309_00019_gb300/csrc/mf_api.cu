@@ -519,9 +519,10 @@ mf_status mf_bank_generate_taylorf2(mf_plan_t p, int64_t row0, int64_t n_rows, c
   // still in L2 when they are stored; a temporary buffer takes its place where the scratch holds no row.  One
   // 256 MB block at a time in a buffer of its own cost an allocation, a free and 3 waits per 63 templates.
   const int64_t ld = (p->nb + 63) / 64 * 64;
+  const int64_t k_hi = mf::taylorf2_k_hi(m1, m2, n_rows, p->d.fs, p->d.n, f_low);
   const size_t table = mf::taylorf2_table_bytes(n_rows), row = (size_t)ld * sizeof(float2);
   auto bytes = [&](int64_t c) {
-    return table + mf::taylorf2_work_bytes(c, p->d.fs, p->d.n, f_low) + (size_t)c * row;
+    return table + mf::taylorf2_work_bytes(c, p->d.fs, p->d.n, f_low, k_hi) + (size_t)c * row;
   };
   int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(n_rows, (int64_t(128) << 20) / (int64_t)row));
   const size_t have = p->scratch ? (size_t)p->batch * p->d.n_det * p->d.n * sizeof(float2) : 0;
@@ -535,12 +536,12 @@ mf_status mf_bank_generate_taylorf2(mf_plan_t p, int64_t row0, int64_t n_rows, c
     while (bytes(chunk) > have) chunk = (chunk + 1) / 2;
   }
   char* anchors = work + table;
-  float2* rows = reinterpret_cast<float2*>(anchors + mf::taylorf2_work_bytes(chunk, p->d.fs, p->d.n, f_low));
+  float2* rows = reinterpret_cast<float2*>(anchors + mf::taylorf2_work_bytes(chunk, p->d.fs, p->d.n, f_low, k_hi));
   cudaError_t e = mf::taylorf2_tables(m1, m2, n_rows, p->d.fs, p->d.n, f_low, work, p->st);
   bank_changed(p);
   for (int64_t r = 0; r < n_rows && e == cudaSuccess; r += chunk) {
     const int64_t cnt = std::min<int64_t>(chunk, n_rows - r);
-    e = mf::launch_taylorf2(work, r, cnt, p->d.fs, p->d.n, f_low, anchors, rows, ld, p->st);
+    e = mf::launch_taylorf2(work, r, cnt, p->d.fs, p->d.n, f_low, k_hi, anchors, rows, ld, p->st);
     if (e == cudaSuccess)
       e = mf::launch_put_rows(bank_rows(p, row0 + r), rows, ld, cnt, p->bank_dtype != MF_F32, p->nb, p->st);
   }

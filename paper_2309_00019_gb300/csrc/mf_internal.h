@@ -222,14 +222,17 @@ cudaError_t launch_chisq(const void* trig, const int64_t* count, int64_t cap, co
 // TaylorF2 templates (mf_taylorf2.cu): natural-order complex64 rows out [.][ld] of an n-sample segment at fs.
 // taylorf2_tables turns valid host masses into the kernels' table (taylorf2_table_bytes(n_tmpl) bytes at dev; the
 // host masses are done with on return); launch_taylorf2 generates rows [t0, t0 + n_rows) of the table with
-// taylorf2_work_bytes(n_rows, ...) bytes of work space.
+// taylorf2_work_bytes(n_rows, ...) bytes of work space.  k_hi: the highest band edge of the table's templates
+// (taylorf2_k_hi).  taylorf2_block: rows (up to n_tmpl) whose work space stays within 64 MB (one row in any case).
 bool taylorf2_valid(const double* m1, const double* m2, int64_t n_tmpl, double fs, int64_t n, double f_low);
+int64_t taylorf2_k_hi(const double* m1, const double* m2, int64_t n_tmpl, double fs, int64_t n, double f_low);
 size_t taylorf2_table_bytes(int64_t n_tmpl);
-size_t taylorf2_work_bytes(int64_t n_rows, double fs, int64_t n, double f_low);
+size_t taylorf2_work_bytes(int64_t n_rows, double fs, int64_t n, double f_low, int64_t k_hi);
+int64_t taylorf2_block(int64_t n_tmpl, double fs, int64_t n, double f_low, int64_t k_hi);
 cudaError_t taylorf2_tables(const double* m1, const double* m2, int64_t n_tmpl, double fs, int64_t n, double f_low,
                             void* dev, cudaStream_t st);
 cudaError_t launch_taylorf2(const void* tables, int64_t t0, int64_t n_rows, double fs, int64_t n, double f_low,
-                            void* work, float2* out, int64_t ld, cudaStream_t st);
+                            int64_t k_hi, void* work, float2* out, int64_t ld, cudaStream_t st);
 
 // blocks x 256 threads, each 8 chains x 16 x iters FP32 FMAs (the ALU probe)
 cudaError_t launch_fma_probe(float* out, int blocks, int iters, cudaStream_t st);

@@ -55,21 +55,24 @@ __device__ __forceinline__ double tf2_phase(const TF2& t, double f) {
   return -0.25 * kPi + t.pre / v5 * s;
 }
 
-// Anchor a of a template is at bin (a - 1) K.  Those below half the lower band edge, or two intervals past the
-// upper one, only serve bins that are zeroed; they are 0.
+// Anchor a of a template is at bin (a - 1) K.  psi holds a row's anchors a0 .. a0 + n_anchor - 1, which are those that
+// some template's band needs; the ones below half the lower band edge, or two intervals past the template's own upper one,
+// are not needed and not written.
 __global__ void __launch_bounds__(kGenThreads) k_tf2_anchors(const TF2* __restrict__ tmpl, double df, int n_anchor,
-                                                             double* __restrict__ psi) {
-  const TF2 t = tmpl[blockIdx.y];
-  const int a = blockIdx.x * kGenThreads + threadIdx.x;
-  if (a >= n_anchor) return;
-  const int K = 1 << t.K_log2;
-  const int64_t k = (int64_t)(a - 1) * K;
-  const bool used = k >= t.k_lo / 2 && k <= t.k_hi + 2 * K;
-  psi[(int64_t)blockIdx.y * n_anchor + a] = used ? tf2_phase(t, (double)k * df) : 0.0;
+                                                             int64_t a0, double* __restrict__ psi) {
+  const int i = blockIdx.x * kGenThreads + threadIdx.x;
+  if (i >= n_anchor) return;
+  const TF2& m = tmpl[blockIdx.y];
+  const int K = 1 << m.K_log2;
+  const int64_t k = (a0 + i - 1) * K;
+  if (k < m.k_lo / 2 || k > m.k_hi + 2 * K) return;
+  const TF2 t = m;
+  psi[(int64_t)blockIdx.y * n_anchor + i] = tf2_phase(t, (double)k * df);
 }
 
 __global__ void __launch_bounds__(kGenThreads) k_taylorf2(const TF2* __restrict__ tmpl, const double* __restrict__ psi,
-                                                          int n_anchor, double df, float df32, float2* __restrict__ out,
+                                                          int n_anchor, int64_t a0, double df, float df32,
+                                                          float2* __restrict__ out,
                                                           int64_t ld, int64_t nb) {
   __shared__ float mod2pi[kGenChunk + 4];  // anchor phase mod 2 pi
   __shared__ float dnext[kGenChunk + 4];   // Psi(anchor + 1) - Psi(anchor)
@@ -82,10 +85,11 @@ __global__ void __launch_bounds__(kGenThreads) k_taylorf2(const TF2* __restrict_
     return;
   }
   const int K = 1 << t.K_log2;
-  // the chunk's anchors -1 .. n_in + 1 (its bins lie in intervals 0 .. n_in - 1)
-  const int n_in = (int)((k1 - k0 + K - 1) >> t.K_log2);
-  const double* pa = psi + (int64_t)blockIdx.y * n_anchor + (k0 >> t.K_log2);
-  for (int a = threadIdx.x; a < n_in + 3; a += kGenThreads) {
+  // the band's bins of the chunk lie in intervals i0 .. i1; interval i has the anchors i .. i + 3
+  const int i0 = (int)((k0 < t.k_lo ? t.k_lo - k0 : 0) >> t.K_log2);
+  const int i1 = (int)(((k1 - 1 < t.k_hi ? k1 - 1 : t.k_hi) - k0) >> t.K_log2);
+  const double* pa = psi + (int64_t)blockIdx.y * n_anchor + ((k0 >> t.K_log2) - a0);
+  for (int a = i0 + threadIdx.x; a < i1 + 3; a += kGenThreads) {
     const double p = pa[a];
     const double two_pi = 2.0 * kPi;
     mod2pi[a] = (float)(p - two_pi * floor(p / two_pi));
@@ -167,17 +171,35 @@ static TF2 make_tf2(double m1, double m2, double fs, int64_t n, double f_low) {
   return t;
 }
 
-// anchors of a row: -1 .. the second past the last bin
-static int anchor_count(int64_t n, double fs, double f_low) {
+// the anchors that a call's rows need: from a0 on, to the second past the highest band edge k_hi
+struct Anchors {
+  int64_t a0;
+  int count;
+};
+static Anchors anchors_of(int64_t n, double fs, double f_low, int64_t k_hi) {
   const double df = fs / (double)n;
-  const int lg = anchor_log2(first_bin(f_low, df), df);
-  return (int)(((n / 2 + 1 + (1 << lg) - 1) >> lg) + 4);
+  const int64_t lo = first_bin(f_low, df);
+  const int lg = anchor_log2(lo, df);
+  const int64_t a0 = ((lo / 2) >> lg) + 1, a1 = ((k_hi + 2 * (int64_t(1) << lg)) >> lg) + 2;
+  return Anchors{a0, (int)std::max<int64_t>(a1 - a0, 0)};  // (k_hi < n / 2)
+}
+
+int64_t taylorf2_k_hi(const double* m1, const double* m2, int64_t n_tmpl, double fs, int64_t n, double f_low) {
+  int64_t light = 0;
+  for (int64_t i = 1; i < n_tmpl; ++i)
+    if (m1[i] + m2[i] < m1[light] + m2[light]) light = i;
+  return make_tf2(m1[light], m2[light], fs, n, f_low).k_hi;
 }
 
 size_t taylorf2_table_bytes(int64_t n_tmpl) { return ((size_t)n_tmpl * sizeof(TF2) + 255) / 256 * 256; }
 
-size_t taylorf2_work_bytes(int64_t n_rows, double fs, int64_t n, double f_low) {
-  return ((size_t)n_rows * anchor_count(n, fs, f_low) * sizeof(double) + 255) / 256 * 256;
+size_t taylorf2_work_bytes(int64_t n_rows, double fs, int64_t n, double f_low, int64_t k_hi) {
+  return ((size_t)n_rows * anchors_of(n, fs, f_low, k_hi).count * sizeof(double) + 255) / 256 * 256;
+}
+
+int64_t taylorf2_block(int64_t n_tmpl, double fs, int64_t n, double f_low, int64_t k_hi) {
+  const int64_t row = std::max(anchors_of(n, fs, f_low, k_hi).count, 1) * (int64_t)sizeof(double);
+  return std::max<int64_t>(1, std::min<int64_t>(n_tmpl, (int64_t(64) << 20) / row));
 }
 
 cudaError_t taylorf2_tables(const double* m1, const double* m2, int64_t n_tmpl, double fs, int64_t n, double f_low,
@@ -196,10 +218,14 @@ bool taylorf2_valid(const double* m1, const double* m2, int64_t n_tmpl, double f
 }
 
 cudaError_t launch_taylorf2(const void* tables, int64_t t0, int64_t n_rows, double fs, int64_t n, double f_low,
-                            void* work, float2* out, int64_t ld, cudaStream_t st) {
+                            int64_t k_hi, void* work, float2* out, int64_t ld, cudaStream_t st) {
   const double df = fs / (double)n;
   const int64_t nb = n / 2 + 1;
-  const int na = anchor_count(n, fs, f_low);
+  // Only the anchors that a band needs.  Where an anchor per bin is called for (bins of 0.25 Hz) and the band is a small
+  // part of the row, space and blocks for all of them took longer than the phases: 300 rows of 2^18 samples at
+  // 65,536 Hz 649 us, 331 us so (425 us with the phases in the kernel of the bins).
+  const Anchors an = anchors_of(n, fs, f_low, k_hi);
+  const int na = an.count;
   // The frequency k df to FP32.  With a df that FP32 holds exactly (any whole sampling rate up to 2^24 Hz) the FP64
   // product is exact, so one FP32 multiplication rounds it alike; otherwise two conversions and a product in FP64, 2 of
   // which the chip does per clock and SM: 340 us of k_taylorf2 instead of 804 us for 384 rows at N = 2^20.
@@ -208,11 +234,14 @@ cudaError_t launch_taylorf2(const void* tables, int64_t t0, int64_t n_rows, doub
   double* psi = static_cast<double*>(work);
   for (int64_t r = 0; r < n_rows; r += 65535) {
     const unsigned rows = (unsigned)std::min<int64_t>(65535, n_rows - r);
-    k_tf2_anchors<<<dim3((unsigned)((na + kGenThreads - 1) / kGenThreads), rows), kGenThreads, 0, st>>>(
-        d + r, df, na, psi + r * na);
+    if (na > 0) {
+      k_tf2_anchors<<<dim3((unsigned)((na + kGenThreads - 1) / kGenThreads), rows), kGenThreads, 0, st>>>(
+          d + r, df, na, an.a0, psi + r * na);
+      add_launches(1);
+    }
     k_taylorf2<<<dim3((unsigned)((nb + kGenChunk - 1) / kGenChunk), rows), kGenThreads, 0, st>>>(
-        d + r, psi + r * na, na, df, df32, out + r * ld, ld, nb);
-    add_launches(2);
+        d + r, psi + r * na, na, an.a0, df, df32, out + r * ld, ld, nb);
+    add_launches(1);
   }
   return cudaGetLastError();
 }
@@ -230,13 +259,15 @@ extern "C" mf_status mf_taylorf2(const double* m1, const double* m2, int64_t n_t
     return MF_EINVAL;
   }
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const int64_t block = std::min<int64_t>(n_tmpl, 256);  // rows per launch: bounds the anchors' work space
+  const int64_t k_hi = mf::taylorf2_k_hi(m1, m2, n_tmpl, fs, n, f_low);
+  const int64_t block = mf::taylorf2_block(n_tmpl, fs, n, f_low, k_hi);
   const size_t table = mf::taylorf2_table_bytes(n_tmpl);
   char* dev = nullptr;
-  cudaError_t e = cudaMalloc((void**)&dev, table + mf::taylorf2_work_bytes(block, fs, n, f_low));
+  cudaError_t e = cudaMalloc((void**)&dev, table + mf::taylorf2_work_bytes(block, fs, n, f_low, k_hi));
+  if (e != cudaSuccess) cudaGetLastError();
   if (e == cudaSuccess) e = mf::taylorf2_tables(m1, m2, n_tmpl, fs, n, f_low, dev, st);
   for (int64_t r = 0; r < n_tmpl && e == cudaSuccess; r += block)
-    e = mf::launch_taylorf2(dev, r, std::min(block, n_tmpl - r), fs, n, f_low, dev + table,
+    e = mf::launch_taylorf2(dev, r, std::min(block, n_tmpl - r), fs, n, f_low, k_hi, dev + table,
                             static_cast<float2*>(out) + r * ld, ld, st);
   const cudaError_t e2 = cudaStreamSynchronize(st);
   if (dev) cudaFree(dev);
