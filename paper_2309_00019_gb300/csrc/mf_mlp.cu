@@ -34,7 +34,7 @@ namespace {
 // backward pass that wait for the same operand share a launch, and the bias, GELU and GELU' are the epilogue's.
 // K runs in steps of 16 in order whatever the tiles, so the sums are those of the plain loop.  64 x 64 tiles with
 // 2-byte loads and no overlap took 65 us per product, 904 us of a training step's 1,259 us at batch 1,024, width 256
-// and 2,000 slots; the ten launches now take 87 us of 159.
+// and 2,000 slots; as ten launches 87 us of 159 (153 with z read ahead).
 // ---------------------------------------------------------------------------
 
 constexpr int kTM = 64, kTN = 32, kTK = 64, kStages = 3;
@@ -71,7 +71,7 @@ __device__ __forceinline__ uint32_t swz128(int r, int c) { return (uint32_t)(r *
 __device__ __forceinline__ uint32_t swz64(int r, int c) { return (uint32_t)(r * 64 + ((c ^ ((r >> 1) & 3)) << 4)); }
 
 // what becomes of acc: kStore: C = acc (+ bias); kGelu: C = z = acc + bias, out = GELU(z);
-// kGeluGrad: C = out = acc GELU'(z)
+// kGeluGrad: C = out = acc GELU'(z), with z what C holds (a thread reads and writes its own elements)
 enum Epi { kStore = 0, kGelu = 1, kGeluGrad = 2 };
 
 struct Gemm {
@@ -82,7 +82,6 @@ struct Gemm {
   int ldc;
   const float* bias;
   int epi;
-  const float* z;     // kGeluGrad, as C
   bf16* out;          // kGelu, kGeluGrad
   int ldo;
   int tiles_n, tiles;
@@ -121,6 +120,20 @@ __device__ __forceinline__ void gemm_tile(const Gemm& g, int tile, unsigned char
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   float acc[2][2][4] = {};
+  const int gr = lane >> 2, tq = lane & 3;
+  auto row_of = [&](int mi, int e) { return m0 + wm + mi * 16 + gr + 8 * (e >> 1); };
+  auto col_of = [&](int ni, int e) { return n0 + wn + ni * 8 + tq * 2 + (e & 1); };
+  // read ahead: between the stores to C the reads would wait for one another (the training step 166 us, 153 us so)
+  float z[2][2][4] = {};
+  if (g.epi == kGeluGrad) {
+#pragma unroll
+    for (int mi = 0; mi < 2; ++mi)
+#pragma unroll
+      for (int ni = 0; ni < 2; ++ni)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (row_of(mi, e) < g.M && col_of(ni, e) < g.N) z[mi][ni][e] = g.C[(int64_t)row_of(mi, e) * g.ldc + col_of(ni, e)];
+  }
 #pragma unroll
   for (int s = 0; s < kStages - 1; ++s) load(s);
   for (int step = 0; step < steps; ++step) {
@@ -151,18 +164,17 @@ __device__ __forceinline__ void gemm_tile(const Gemm& g, int tile, unsigned char
       }
     }
   }
-  const int gr = lane >> 2, tq = lane & 3;
 #pragma unroll
   for (int mi = 0; mi < 2; ++mi)
 #pragma unroll
     for (int ni = 0; ni < 2; ++ni)
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const int r = m0 + wm + mi * 16 + gr + 8 * (e >> 1), c = n0 + wn + ni * 8 + tq * 2 + (e & 1);
+        const int r = row_of(mi, e), c = col_of(ni, e);
         if (r >= g.M || c >= g.N) continue;
         float v = acc[mi][ni][e] + (g.bias ? g.bias[c] : 0.f);
         const int64_t at = (int64_t)r * g.ldc + c;
-        if (g.epi == kGeluGrad) v = v * gelu_grad(g.z[at]);
+        if (g.epi == kGeluGrad) v = v * gelu_grad(z[mi][ni][e]);
         g.C[at] = v;
         if (g.epi == kGelu) g.out[(int64_t)r * g.ldo + c] = __float2bfloat16(gelu(v));
         if (g.epi == kGeluGrad) g.out[(int64_t)r * g.ldo + c] = __float2bfloat16(v);
@@ -437,9 +449,8 @@ struct mf_mlp_s {
   int ldx = 0, ldh = 0, ldo = 0;       // padded rows of the BF16 operands: input, activations, logit gradients
   bf16* wb = nullptr;                  // BF16 copy of the weights, padded rows (the products' operand)
   bf16* xb = nullptr;                  // input [B][ldx]
-  std::vector<float*> z;               // pre-activations [B][width], l = 1..depth
+  std::vector<float*> z;               // pre-activations [B][width], l = 1..depth; after the backward pass, gradients
   std::vector<bf16*> h;                // activations [B][ldh]
-  std::vector<float*> dz;              // their gradients [B][width]
   float* logits = nullptr;             // [B][n_out]
   float* dlog = nullptr;               // [B][n_out]
   bf16* dlogb = nullptr;               // [B][ldo]
@@ -556,12 +567,11 @@ mf_status mf_mlp_create(mf_mlp_t* out, int32_t n_in, int32_t width, int32_t dept
             dal(&p->dlogb, B * p->ldo) && dal(&p->dzb[0], B * p->ldh) && dal(&p->dzb[1], B * p->ldh) &&
             dal(&p->loss, 1);
   for (int l = 0; ok && l < depth; ++l) {
-    float *zz = nullptr, *dd = nullptr;
+    float* zz = nullptr;
     bf16* hh = nullptr;
-    ok = dal(&zz, B * width) && dal(&hh, B * p->ldh) && dal(&dd, B * width);
+    ok = dal(&zz, B * width) && dal(&hh, B * p->ldh);
     p->z.push_back(zz);
     p->h.push_back(hh);
-    p->dz.push_back(dd);
     if (ok) cudaMemsetAsync(hh, 0, B * p->ldh * sizeof(bf16), p->st);
   }
   if (!ok) {
@@ -588,7 +598,6 @@ void mf_mlp_destroy(mf_mlp_t p) {
                   (void*)p->loss})
     if (q) cudaFree(q);
   for (auto* q : p->z) if (q) cudaFree(q);
-  for (auto* q : p->dz) if (q) cudaFree(q);
   for (auto* q : p->h) if (q) cudaFree(q);
   delete p;
 }
@@ -647,9 +656,8 @@ mf_status mf_mlp_loss_grad(mf_mlp_t p, const float* x, const int32_t* n_valid, c
                       p->grad + p->w_off[l], dout);
     Gemm dh{};
     if (l > 0) {
-      dh = product(Bi, W, dout, dz, ldz, p->wb + p->layers.p[l], p->layers.ld[l], p->dz[l - 1], W);
+      dh = product(Bi, W, dout, dz, ldz, p->wb + p->layers.p[l], p->layers.ld[l], p->z[l - 1], W);
       dh.epi = kGeluGrad;
-      dh.z = p->z[l - 1];
       dh.out = p->dzb[l & 1];
       dh.ldo = p->ldh;
     }
@@ -660,7 +668,7 @@ mf_status mf_mlp_loss_grad(mf_mlp_t p, const float* x, const int32_t* n_valid, c
   ColSums cs{};
   int wide = 0;
   for (int l = 0; l <= D; ++l) {
-    cs.G[l] = l < D ? p->dz[l] : p->dlog;
+    cs.G[l] = l < D ? p->z[l] : p->dlog;
     cs.db[l] = p->grad + p->b_off[l];
     cs.cols[l] = p->layers.dout[l];
     wide = std::max(wide, cs.cols[l]);
