@@ -41,8 +41,8 @@ WORKLOAD = ("two-stage hierarchical search: 2 det x 512 s @ 2048 Hz, coarse 2000
             "fine 20000 @ 2048 Hz (N=2^20) on the union of exact-match (>= 0.9) neighbourhoods")
 FP32_LANES_PER_SM = 128
 # names of the two filter kernels per plan implementation (mf_plan_stats.impl)
-# k_cols_h16 / k_cols_h16x2: k_cols with FP16 / FP16-pair output; k_rows_tc2: the split-product row pass
-KERNEL_NAMES = {2: ("k_cols", "k_rows"), 3: ("k_cols_h16", "k_rows_tc"), 4: ("k_cols_h16x2", "k_rows_tc2")}
+# k_cols16 / k_cols16x2: the column pass with FP16 / FP16-pair output; k_rows_tc2: the split-product row pass
+KERNEL_NAMES = {2: ("k_cols", "k_rows"), 3: ("k_cols16", "k_rows_tc"), 4: ("k_cols16x2", "k_rows_tc2")}
 # the timed steps time every PROFILE_STRIDE-th launch pair of the filter kernels: the events between the two
 # passes of a timed pair keep the second kernel from launching early, so the others run undisturbed
 PROFILE_STRIDE = 8
