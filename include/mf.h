@@ -98,7 +98,8 @@ mf_status mf_set_psd(mf_plan_t plan, const double* psd, int64_t nbins);
  * (average = 0) or by the median divided by 1 - 1/2 + 1/3 - ... (m terms
  * after the first, m = (segments - 1) / 2; FINDCHIRP Appendix B; average = 1,
  * at most 4096 segments).  psd: device float64 [n_det][seg_len/2+1] (out).
- * Allocates segments x n_det x seg_len x 12 bytes of work space for the call.
+ * Allocates work space for the call: 8 bytes x segments x n_det x (seg_len +
+ * the seg_len/2+1 bins rounded up to 64).
  * Synchronises.  Errors (mf_last_error(NULL)): MF_EINVAL, MF_ENOMEM, MF_ECUDA. */
 mf_status mf_psd_welch(double fs, int32_t n_det, int64_t n_samples, const float* strain, int64_t ld, int64_t seg_len,
                        int64_t stride, int32_t average, double* psd, void* cuda_stream);
@@ -286,8 +287,8 @@ typedef struct {
   double pass1_ms;
   int64_t pass2_launches, pass2_series;
   double pass2_ms;
-  int32_t impl;       /* filter kernels in use: 2 = k_cols / k_rows (FP32 intermediate), 3 = k_cols /
-                         k_rows_tc (FP16 intermediate, tensor-core row pass), 4 = k_cols / k_rows_tc
+  int32_t impl;       /* filter kernels in use: 2 = k_cols / k_rows (FP32 intermediate), 3 = k_cols16 /
+                         k_rows_tc (FP16 intermediate, tensor-core row pass), 4 = k_cols16 / k_rows_tc
                          with FP16 pairs (MF_F16X2) */
   int32_t batch;      /* templates per pass-1 / pass-2 launch pair */
 } mf_plan_stats;

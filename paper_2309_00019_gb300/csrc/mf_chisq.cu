@@ -9,8 +9,9 @@
 // floor(p C(k) / sigma^2) = l (clamped to p - 1): k_block_power and
 // k_chisq_edges find the first bin of every band with FP64 block sums, once
 // per bank and p; k_chisq then
-// sums each trigger's terms in the bank's column layout (contiguous reads of
-// the template and the weighted data), one CTA per trigger.
+// sums the triggers' terms in the bank's column layout (contiguous reads of
+// the template and the weighted data), a CTA per run of up to eight triggers
+// of one template and detector.
 #include <algorithm>
 
 #include "mf_common.cuh"

@@ -16,7 +16,7 @@
 //           the scratch in panels of P = max(T(N1) / 2, RW(N2)) rows:
 //           element (j1, k2) of a series at (j1 / P) N2 P + k2 P + j1 % P,
 //           so that a warp's store covers whole 128-byte lines.
-//   k_cols16: k_cols for the FP16 intermediate of N = 2^20: a warp per column,
+//   k_cols16: k_cols for the FP16 and FP16-pair intermediates of N = 2^20: a warp per column,
 //           stored in image order by one tensor-map copy per column.
 //   k_rows: item = RW rows j1 of one panel, brought in by a 3-D tensor-map
 //           copy (RW of the panel's P values at each k2; one 1-D bulk copy

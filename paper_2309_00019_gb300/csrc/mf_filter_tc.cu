@@ -1,6 +1,6 @@
 // Tensor-core row pass of the matched filter (Eq. 1-2, Sec. V.C: the inverse
 // transform over coalescence time), N = N1 N2 with N2 = 1024, over the FP16
-// pass-1 -> pass-2 intermediate that k_cols16 (k_cols for FP16 pairs) writes in
+// pass-1 -> pass-2 intermediate, FP16 or FP16 pairs, that k_cols16 writes in
 // 8-row panels.
 //
 // A row x[k2] (k2 = 32 p + q) has the 1024-point transform

@@ -126,7 +126,7 @@ class Hierarchy:
         with self.torch.cuda.stream(self.stream):
             self.strain.copy_(strain_host, non_blocking=True)
         self.run()
-        # stage 1's stream is idle by now: its coincidences are read (and ordered on the host) while stage 2 runs
+        # stage 1's stream is idle by now: its coincidences are ordered and read while stage 2 runs
         co, nco, _ = self.p1.coincs(pinned=True)
         trig2, n2, _ = self.p2.triggers(pinned=True)  # page-locked readback, valid until the next step
         return trig2, co
