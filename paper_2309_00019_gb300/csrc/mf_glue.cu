@@ -2,6 +2,8 @@
 // the stage-1 rate, two-detector coincidence with time shifts on the stage-1
 // window maxima, and the union of the neighbourhoods of followed-up coarse
 // templates that becomes the stage-2 template selection.
+#include <algorithm>
+
 #include "mf_internal.h"
 
 namespace mf {
@@ -122,74 +124,100 @@ __global__ void k_coinc(CoincArgs a) {
   }
 }
 
-// Coincidences of one template per CTA.  Of the two triggers of a coincidence at least one has half of the least
+// Coincidences of one template per CTA, or of a share of its detector-0 triggers where there are fewer templates than
+// SMs.  Of the two triggers of a coincidence at least one has half of the least
 // rho_c^2 that counts, and few triggers have: so the pairs (loud detector-0, any detector-1) and (other
 // detector-0, loud detector-1) are all there is to look at, and for a pair the shifts follow from the difference
 // of its times, k step in [D + m R - window, D + m R + window], without a walk over them.  What a CTA finds is
-// collected in shared memory and written in one go.  Trying all 102 shifts for every detector-0 trigger of a
-// template with one loud detector-1 trigger took 512 us on the coarse stage (2,000 templates, 512 windows each);
-// now 159 us.  Where most triggers are loud the CTA walks over the shifts instead: pairs alone took 2,750 us for 50
-// templates of 2,048 windows at zero lag, the walk takes 20 us (k_coinc 22 us), and 154 us for 100 templates and 101
-// shifts (pairs 4,800 us, k_coinc 535 us).
+// collected in shared memory and written in one go.
+// Where most triggers are loud the CTA walks over the shifts of every detector-0 trigger instead and looks into the
+// windows of detector 1 that it falls on.
+// What bounds both is the latency of short dependent steps.  In both a warp's lanes go from pair to pair, turn to turn or
+// shift to shift together (a vote or a __syncwarp): a lane that finds something goes its own way, and left to themselves
+// the lanes did not come together again but finished their loops one by one.
+// Whole calls, us: one thread per detector-0 window over the shifts (k_coinc) / this kernel without that / now
+//   2,000 templates, 2,048 windows, zero lag, rho_c 1.5 times the filter's threshold   77 / 90 / 60 (pairs alone 860)
+//   300 templates, 64 windows, 501 shifts, 1.42 times                                 405 / 5,570 / 134
+//   300 templates, 512 windows, 102 shifts, 1.8 times                                  70 / 18.4 / 18.6
 constexpr int kTmplWin = 2048;   // windows whose triggers fit the CTA's shared memory
 constexpr int kTmplRec = 512;    // records collected before they go out one by one
-constexpr int kWalkShifts = 64;  // shifts that a thread walks at a time
+constexpr int kTmplSplit = 16;   // CTAs of one template, at most
+constexpr int kWalkShifts = 64;  // shifts that a thread walks at a time, at most
+constexpr size_t tmpl_smem(int64_t n_win) { return kTmplRec * sizeof(uint2) + (size_t)n_win * 18; }
+constexpr uint16_t kNoTrigger = 0xffff;
 
 template <int THREADS>
-__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : 1) k_coinc_tmpl(CoincArgs a) {
-  __shared__ int32_t pos[2][kTmplWin];   // ring positions of the triggers of detector 0, 1
-  __shared__ float rho2[2][kTmplWin];
-  __shared__ uint16_t loud[2][kTmplWin];
-  __shared__ uint2 found[kTmplRec];      // (detector-0 trigger | detector-1 trigger << 16, shift)
-  __shared__ int n_pos[2], n_loud[2];
+__global__ void __launch_bounds__(THREADS, THREADS <= 256 ? 1280 / THREADS : 1) k_coinc_tmpl(CoincArgs a) {
+  extern __shared__ __align__(16) unsigned char sm[];  // tmpl_smem(n_win)
+  uint2* found = reinterpret_cast<uint2*>(sm);  // [kTmplRec] (detector-0 trigger | detector-1 trigger << 16, shift)
+  // ring positions and rho^2 of the triggers of detector 0, 1: the loud ones from the front, the others from the end
+  int32_t* pos0 = reinterpret_cast<int32_t*>(found + kTmplRec);
+  int32_t* pos1 = pos0 + a.n_win;
+  float* rho0 = reinterpret_cast<float*>(pos1 + a.n_win);
+  float* rho1 = rho0 + a.n_win;
+  __shared__ int n_loud[2], n_quiet[2];
   __shared__ unsigned n_found;  // collected, or found before it was seen that the collection is full
   __shared__ unsigned max1;     // the largest rho^2 of detector 1 (float bits)
   __shared__ unsigned long long base;
   const int64_t p = blockIdx.x;
-  const int tid = threadIdx.x;
-  if (tid < 2) n_pos[tid] = n_loud[tid] = 0;
+  const int tid = threadIdx.x, lane = tid & 31, n_win = (int)a.n_win;
+  if (tid < 2) n_loud[tid] = n_quiet[tid] = 0;
   if (tid == 2) n_found = max1 = 0;
   __syncthreads();
   const float need = fminf(a.rho_c_thr2, a.rho_c_store2), half = 0.5f * need;
   const int32_t rb = (int32_t)a.ring_begin;
-  const int lane = tid & 31;
-  for (int d = 0; d < 2; ++d)
-    for (int i0 = tid - lane; i0 < (int)a.n_win; i0 += THREADS) {  // a warp's triggers at a time
-      const unsigned long long key = i0 + lane < (int)a.n_win ? a.slots[(d * a.n_sel + p) * a.n_win + i0 + lane] : 0ull;
-      const float r = key_rho2(key);
-      const unsigned has = __ballot_sync(0xffffffffu, key != 0ull);
-      const unsigned big = __ballot_sync(0xffffffffu, key != 0ull && r >= half);
-      if (!has) continue;
-      int base_pos = 0, base_loud = 0;
-      if (lane == 0) {
-        base_pos = atomicAdd(&n_pos[d], __popc(has));
-        if (big) base_loud = atomicAdd(&n_loud[d], __popc(big));
-      }
-      base_pos = __shfl_sync(0xffffffffu, base_pos, 0);
-      base_loud = __shfl_sync(0xffffffffu, base_loud, 0);
-      const unsigned before = (1u << lane) - 1u;
-      const int at = base_pos + __popc(has & before);
-      if (key != 0ull) {
-        pos[d][at] = (int32_t)key_sample(key) - rb;
-        rho2[d][at] = r;
-        if (r >= half) loud[d][base_loud + __popc(big & before)] = (uint16_t)at;
-      }
+  auto put = [&](int d, int w, unsigned long long key) {  // a warp's windows of detector d
+    const float r = key_rho2(key);
+    const bool listed = key != 0ull && (d == 1 || w % gridDim.y == blockIdx.y);  // detector 0: this CTA's share
+    const unsigned big = __ballot_sync(0xffffffffu, listed && r >= half);
+    const unsigned rest = __ballot_sync(0xffffffffu, listed) & ~big;
+    if (!(big | rest)) return;
+    int l0 = 0, q0 = 0;
+    if (lane == 0) {
+      if (big) l0 = atomicAdd(&n_loud[d], __popc(big));
+      if (rest) q0 = atomicAdd(&n_quiet[d], __popc(rest));
     }
+    l0 = __shfl_sync(0xffffffffu, l0, 0);
+    q0 = __shfl_sync(0xffffffffu, q0, 0);
+    const unsigned before = (1u << lane) - 1u;
+    if (listed) {
+      const int at = r >= half ? l0 + __popc(big & before) : n_win - 1 - q0 - __popc(rest & before);
+      (d ? pos1 : pos0)[at] = (int32_t)key_sample(key) - rb;
+      (d ? rho1 : rho0)[at] = r;
+    }
+  };
+  const unsigned long long *s0 = a.slots + p * a.n_win, *s1 = a.slots + (a.n_sel + p) * a.n_win;
+  constexpr int U = 2;  // windows per thread and detector in flight
+  for (int i0 = tid - lane; i0 < n_win; i0 += U * THREADS) {
+    unsigned long long k0[U], k1[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int w = i0 + u * THREADS + lane;
+      k0[u] = w < n_win ? __ldg(s0 + w) : 0ull;
+      k1[u] = w < n_win ? __ldg(s1 + w) : 0ull;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      put(0, i0 + u * THREADS + lane, k0[u]);
+      put(1, i0 + u * THREADS + lane, k1[u]);
+    }
+  }
   __syncthreads();
-  if (n_loud[0] + n_loud[1] == 0) return;
+  const int loud0 = n_loud[0], loud1 = n_loud[1], all0 = loud0 + n_quiet[0], all1 = loud1 + n_quiet[1];
+  if (loud0 + loud1 == 0 || all0 == 0 || all1 == 0) return;
+  auto trig0 = [&](int i) { return i < loud0 ? i : n_win - 1 - (i - loud0); };
+  auto trig1 = [&](int i) { return i < loud1 ? i : n_win - 1 - (i - loud1); };
   const int32_t tmpl = a.sel[p];
   const int32_t R = (int32_t)(a.ring_end - a.ring_begin), step = (int32_t)(a.shift % R), cw = (int32_t)a.coinc_window;
-  const int32_t last = a.n_shifts * step;  // + 2 R fits (launch_coinc)
-  const float inv_step = 1.f / (float)step;
   bool follow = false;
   auto record = [&](int h, int l, int32_t k) {
     return CoincRec{tmpl,
                     k,
-                    (int64_t)pos[0][h] + rb,
-                    (int64_t)pos[1][l] + rb,
-                    sqrtf(rho2[0][h]),
-                    sqrtf(rho2[1][l]),
-                    sqrtf(rho2[0][h] + rho2[1][l]),
+                    (int64_t)pos0[h] + rb,
+                    (int64_t)pos1[l] + rb,
+                    sqrtf(rho0[h]),
+                    sqrtf(rho1[l]),
+                    sqrtf(rho0[h] + rho1[l]),
                     0};
   };
   // Straight to the list, counted in the 64 bits of n_coinc: a pair at the shifts k0 .. k1
@@ -210,78 +238,92 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : 1) k_coinc_tmpl(
     else
       emit_run(h, l, k, k);
   };
-  auto pair = [&](int h, int l) {
-    const float rc2 = rho2[0][h] + rho2[1][l];
-    if (!(rc2 >= need)) return;
-    int32_t D = pos[0][h] - pos[1][l];
-    if (D < 0) D += R;
-    if (step == 0) {  // all shifts or none
-      if (D > cw && R - D > cw) return;
-      follow |= rc2 >= a.rho_c_thr2;
-      if (rc2 >= a.rho_c_store2) emit_run(h, l, 0, a.n_shifts);
-      return;
-    }
-    for (int32_t t = D - R; t - cw <= last; t += R) {
-      if (t + cw < 0) continue;
-      // the largest k with k step <= t + cw: a guess that is off by a few at most, then the exact one
-      int32_t k = (int32_t)((float)(t + cw) * inv_step);
-      while (k * step > t + cw) --k;
-      while ((k + 1) * step <= t + cw) ++k;
-      for (; k >= 0 && k * step >= t - cw; --k)
-        if (k <= a.n_shifts) emit(h, l, k, rc2);
+  const uint32_t inv = step > 0 ? 0xffffffffu / (uint32_t)step : 0u;
+  // the triggers h = first(i / n), l = trig1(i % n) of the pairs i < m n
+  auto pairs = [&](int m, int n, auto first) {
+    if (m == 0 || n == 0) return;
+    const int32_t last = a.n_shifts * step;
+    const int ja = THREADS / n, jb = THREADS - ja * n;
+    int ia = tid / n, ib = tid - ia * n;
+    for (int i0 = tid - lane; i0 < m * n; i0 += THREADS) {
+      const bool in = i0 + lane < m * n;
+      const int h = first(min(ia, m - 1)), l = trig1(ib);
+      ib += jb;
+      ia += ja + (ib >= n ? 1 : 0);
+      ib -= ib >= n ? n : 0;
+      const float rc2 = rho0[h] + rho1[l];
+      const bool live = in && rc2 >= need;
+      if (!__any_sync(0xffffffffu, live)) continue;
+      int32_t D = pos0[h] - pos1[l];
+      if (D < 0) D += R;
+      if (step == 0) {  // all shifts or none
+        if (live && (D <= cw || R - D <= cw)) {
+          follow |= rc2 >= a.rho_c_thr2;
+          if (rc2 >= a.rho_c_store2) emit_run(h, l, 0, a.n_shifts);
+        }
+        __syncwarp();
+        continue;
+      }
+      int32_t x = D + cw;  // the shifts k with x - 2 cw <= k step <= x, turn by turn (last + 4 R fits)
+      x -= x >= R ? R : 0;
+      bool more = live && x - 2 * cw <= last;
+      while (__any_sync(0xffffffffu, more))
+        if (more) {
+          uint32_t k = __umulhi((uint32_t)x, inv);  // x / step, or one less
+          k += (k + 1) * (uint32_t)step <= (uint32_t)x ? 1 : 0;
+          for (int32_t j = (int32_t)k; j >= 0 && j * step >= x - 2 * cw; --j)
+            if (j <= a.n_shifts) emit(h, l, j, rc2);
+          x += R;
+          more = x - 2 * cw <= last;
+        }
     }
   };
-  // Pairs are few where few triggers are loud.  Where most are (thresholds near sqrt(2) times the filter's, or below) it
-  // is less work to walk over the shifts of every detector-0 trigger and look into the windows of detector 1 that it
-  // falls on.  A pair whose SNRs suffice goes through the turns of the ring (of those with one quiet trigger a
-  // quarter, say); a step of the walk costs about two of a pair.
-  const int64_t loud2 = (int64_t)n_loud[0] * n_loud[1];
-  const int64_t mixed = (int64_t)n_loud[0] * n_pos[1] + (int64_t)n_pos[0] * n_loud[1] - 2 * loud2;
-  if (loud2 + mixed + a.turns * (loud2 + mixed / 4) <= n_pos[0] * a.walk_steps) {
-    for (int i = 0; i < n_loud[0]; ++i) {
-      const int h = loud[0][i];
-      for (int l = tid; l < n_pos[1]; l += THREADS) pair(h, l);
-    }
-    for (int h = tid; h < n_pos[0]; h += THREADS)
-      if (rho2[0][h] < half)
-        for (int i = 0; i < n_loud[1]; ++i) pair(h, loud[1][i]);
+  int len = kWalkShifts;  // shifts that a thread walks at a time: fewer where there are threads for them
+  while (len > 8 && all0 * (a.n_shifts / len + 1) < THREADS) len >>= 1;
+  const int items = all0 * (a.n_shifts / len + 1), steps = min(len, a.n_shifts + 1);
+  // What the two ways cost a thread, fitted to 3,907 calls by both (12 lengths with their windows and thresholds, 1 to 2,000
+  // templates, up to 1,501 shifts): 1 for a pair, 1 for each of its turns of the ring if its SNRs suffice (half of those
+  // with one quiet trigger, say), 2 for a shift of the walk and 2 for each window that it looks into beyond the first.
+  // The way so chosen takes 0.8% longer than the better one in the mean, 2.4 times as long at worst.
+  auto rounds = [](int64_t n) { return (n + THREADS - 1) / THREADS; };
+  const int64_t loud2 = (int64_t)loud0 * loud1;
+  const int64_t mixed = (int64_t)loud0 * all1 + (int64_t)all0 * loud1 - 2 * loud2;
+  if (rounds(loud2 + mixed) + a.turns * rounds(loud2 + mixed / 2) <= rounds(items) * steps * a.walk_step) {
+    pairs(loud0, all1, trig0);
+    pairs(all0 - loud0, loud1, [&](int i) { return trig0(loud0 + i); });
   } else {
-    auto window_of = [&](int32_t x) { return (int)(((uint64_t)(x + rb) * a.win_recip) >> kRecipBits); };
-    uint16_t* at = loud[0];  // detector-1 trigger of each window (the loud ones are not looked at here)
-    for (int w = tid; w < (int)a.n_win; w += THREADS) at[w] = 0xffffu;
+    uint16_t* at = reinterpret_cast<uint16_t*>(rho1 + n_win);  // detector-1 trigger of each window
+    for (int w = tid; w < n_win; w += THREADS) at[w] = kNoTrigger;
     __syncthreads();
-    for (int l = tid; l < n_pos[1]; l += THREADS) {
-      at[window_of(pos[1][l])] = (uint16_t)l;
-      atomicMax(&max1, __float_as_uint(rho2[1][l]));
+    auto window_of = [&](int32_t x) { return (int)(((uint64_t)(x + rb) * a.win_recip) >> kRecipBits); };
+    for (int i = tid; i < all1; i += THREADS) {
+      const int l = trig1(i);
+      at[window_of(pos1[l])] = (uint16_t)l;
+      atomicMax(&max1, __float_as_uint(rho1[l]));
     }
     __syncthreads();
-    const int chunks = a.n_shifts / kWalkShifts + 1;
-    for (int i = tid; i < n_pos[0] * chunks; i += THREADS) {
-      const int h = i % n_pos[0], kb = i / n_pos[0] * kWalkShifts, ke = min(kb + kWalkShifts - 1, a.n_shifts);
-      if (!(rho2[0][h] + __uint_as_float(max1) >= need)) continue;
-      int32_t x = pos[0][h] - kb * step % R;  // ring position at shift kb
+    for (int i0 = tid - lane; i0 < items; i0 += THREADS) {
+      const int i = min(i0 + lane, items - 1), kb = i / all0 * len, h = trig0(i % all0);
+      const float r0 = rho0[h];
+      const bool live = i0 + lane < items && r0 + __uint_as_float(max1) >= need;
+      if (!__any_sync(0xffffffffu, live)) continue;
+      int32_t x = pos0[h] - kb * step % R;  // ring position at shift kb
       if (x < 0) x += R;
-      for (int32_t k = kb; k <= ke; ++k) {
-        for (int side = 0; side < 2; ++side) {  // [x - cw, x + cw], cut at the ring's end
-          int32_t lo = x - cw, hi = x + cw;
-          if (side == 0) {
-            lo = max(lo, 0);
-            hi = min(hi, R - 1);
-          } else if (lo < 0) {
-            lo += R;
-            hi = R - 1;
-          } else if (hi >= R) {
-            lo = 0;
-            hi -= R;
-          } else {
-            break;
-          }
-          for (int w = window_of(lo); w <= window_of(hi); ++w) {
+      for (int32_t k = kb; k < kb + steps; ++k) {
+        // windows that meet [lo, hi] in the ring
+        auto look = [&](int32_t lo, int32_t hi) {
+          const int end = window_of(hi);
+          for (int w = window_of(lo); w <= end; ++w) {
             const int l = at[w];
-            if (l == 0xffff || pos[1][l] < lo || pos[1][l] > hi) continue;
-            emit(h, l, k, rho2[0][h] + rho2[1][l]);
+            if (l != kNoTrigger && pos1[l] >= lo && pos1[l] <= hi) emit(h, l, k, r0 + rho1[l]);
           }
+        };
+        if (live && k <= a.n_shifts) {
+          look(max(x - cw, 0), min(x + cw, R - 1));
+          if (x < cw) look(x - cw + R, R - 1);
+          else if (x + cw >= R) look(0, x + cw - R);
         }
+        __syncwarp();
         x -= step;
         if (x < 0) x += R;
       }
@@ -475,7 +517,7 @@ cudaError_t launch_decimate(const float2* in, int64_t ld_in, float2* out, int64_
 cudaError_t launch_coinc(const CoincArgs& a, float* max_rho2_det1, cudaStream_t st) {
   if (a.n_sel <= 0) return cudaSuccess;
   if (a.n_sel > 0x7fffffff) return cudaErrorInvalidValue;
-  // up to kTmplWin windows (16 KB of triggers per detector) a CTA per template; beyond, where rows have analysed
+  // up to kTmplWin windows (16 KB of triggers per detector) k_coinc_tmpl; beyond, where rows have analysed
   // ranges of their own (times outside the ring), and where a shift's time overflows, the walk over windows and shifts
   const int64_t R = a.ring_end - a.ring_begin;
   if (a.n_win <= kTmplWin && !a.own_ranges &&
@@ -483,16 +525,22 @@ cudaError_t launch_coinc(const CoincArgs& a, float* max_rho2_det1, cudaStream_t 
     CoincArgs t = a;
     t.win_recip = window_recip(a.window);
     t.turns = ((int64_t)a.n_shifts * (a.shift % R) + a.coinc_window) / R + 2;
-    t.walk_steps = 2 * (int64_t)(a.n_shifts + 1) * (2 * a.coinc_window / a.window + 2);
-    // a thread per window up to 512, and up to 1,024 where every template has an SM to itself (one such CTA fits): 2,000
-    // templates of 512 windows at zero lag, most triggers loud, 35 us with 256 threads and 44 with 512; 2,048 windows,
-    // 1,000 templates at zero lag 63 / 49 / 63 us with 256 / 512 / 1,024, one template and four shifts 44 / 32 / 24 us
-    if (a.n_win <= 512)
-      k_coinc_tmpl<256><<<(unsigned)a.n_sel, 256, 0, st>>>(t);
+    t.walk_step = 2 + 4 * a.coinc_window / a.window;
+    // Threads: a thread per window for short rows (2,000 templates of 64 windows with 128 threads 7% faster than with 256);
+    // for long ones 256 where the CTAs wait for SMs (1,024 windows 5% faster than with 512, 2,048 as fast), else up to 1,024.
+    // Where there are fewer templates than SMs, several CTAs share a template's detector-0 triggers: one template of 1,024
+    // windows over 501 shifts 315 us with one CTA, 41 us with 16 (k_coinc 213 us).
+    const size_t smem = tmpl_smem(a.n_win);
+    const bool many = a.n_sel > 2 * sms();
+    const dim3 g((unsigned)a.n_sel, (unsigned)(a.n_sel < sms() ? std::min<int64_t>(kTmplSplit, sms() / a.n_sel) : 1));
+    if (a.n_win <= 128)
+      k_coinc_tmpl<128><<<g, 128, smem, st>>>(t);
+    else if (a.n_win <= 512 || many)
+      k_coinc_tmpl<256><<<g, 256, smem, st>>>(t);
     else if (a.n_win <= 1024 || a.n_sel > sms())
-      k_coinc_tmpl<512><<<(unsigned)a.n_sel, 512, 0, st>>>(t);
+      k_coinc_tmpl<512><<<g, 512, smem, st>>>(t);
     else
-      k_coinc_tmpl<1024><<<(unsigned)a.n_sel, 1024, 0, st>>>(t);
+      k_coinc_tmpl<1024><<<g, 1024, smem, st>>>(t);
     add_launches(1);
     return cudaGetLastError();
   }

@@ -299,7 +299,7 @@ struct CoincArgs {
   int own_ranges;                   // rows have analysed ranges of their own: times may lie outside the ring
   // set by launch_coinc for k_coinc_tmpl
   uint64_t win_recip;               // window_recip(window)
-  int64_t turns, walk_steps;        // turns of the ring per pair; steps of the walk per detector-0 trigger
+  int64_t turns, walk_step;         // turns of the ring per pair; what a shift of the walk costs
 };
 cudaError_t launch_coinc(const CoincArgs& a, float* max_rho2_det1, cudaStream_t st);
 // n coincidence records in the order (tmpl, shift, sample0, sample1) into out; tmpl < n_tmpl, shift < n_shift; work:
